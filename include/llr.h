@@ -306,20 +306,23 @@ int llr_muca_cv_peak(long long n_samples, const double *E, int n, double e0, dou
 int llr_muca_tunnellings(int n_steps, int n_chains, const double *E, double lo, double hi,
                          int *out);
 
-/* Launch shape of the batched sweep kernel: threads per CTA (128, 160, 192,
- * 256 or 512; one warp scans the window decisions, the others propose; one
- * CTA owns one lattice) and fast_math (1: hardware sine/cosine
+/* Launch shape of the batched sweep kernel: the most threads that work on one
+ * lattice (128, 160, 192, 256 or 512).  A CTA has 768 threads and advances 6, 4,
+ * 4, 3 or 1 lattices at a time accordingly.  fast_math (1: hardware sine/cosine
  * approximations for the staples, 0: correctly rounded-class sincosf).
- * Chosen per lattice size by the autotuner; default 256 threads, fast math. */
+ * Chosen per lattice size by the autotuner; default 256 threads, fast math, and,
+ * until a shape is set, more threads per lattice for batches of fewer lattices
+ * than 3 per SM. */
 int llr_set_kernel_config(llr_handle h, int threads, int fast_math);
 
 /* The full launch shape of the batched sweep kernel, as the autotuner sets
  * it; none of these changes the chains (every shape runs the same per-link
  * arithmetic in the same order), only the speed.
  *   threads, fast_math: as llr_set_kernel_config.
- *   ring: stages of the heat-bath producer/consumer ring in use, 1, 2 or 4
- *     (how many 32-link-group chunks the proposing warps may run ahead of
- *     the warp that takes the window decisions).
+ *   ring: the most stages of the heat-bath producer/consumer ring in use, 1, 2
+ *     or 4 (how many chunks the proposing warps may run ahead of the warp that
+ *     takes the window decisions; fewer where shared memory or the lattices per
+ *     CTA leave no room).
  *   carveout: preferred share of the SM's unified L1/shared storage given to
  *     shared memory, in percent: 50, 75 or 100, or -1 for the driver's default
  *     (a hint; it is a property of the kernel variant in this process, so the
@@ -328,8 +331,8 @@ int llr_set_kernel_config(llr_handle h, int threads, int fast_math);
 int llr_set_kernel_shape(llr_handle h, int threads, int fast_math, int ring, int carveout);
 
 /* The shape of the last launch of the batched sweep kernel on this handle:
- * out (host int[5]) = {threads per CTA, fast math, ring stages, carve-out,
- * CTAs launched}; all zero before the first launch. */
+ * out (host int[5]) = {threads per lattice as set, fast math, ring stages as
+ * set, carve-out, CTAs launched}; all zero before the first launch. */
 int llr_get_last_launch(llr_handle h, int *out);
 
 /* ---------------------------------------------------------------------------

@@ -29,6 +29,8 @@ struct llr_ctx {
     float *d_links = nullptr;        // staging for llr_get/set_links
     size_t links_cap = 0;
     int max_half = 0;
+    int max_L = 0;
+    int slab_L = 0;                  // largest L <= 24 (the sweep kernel's shared-memory slabs)
     int n_or = 4, block = 1;
     double beta_up = 1.5, beta_dn = 0.5;
     llr::LaunchCfg cfg;
@@ -88,6 +90,8 @@ llr::KernelArgs base_args(llr_handle h)
     a.class_mask = 0xFF;
     a.sync = h->d_sync;
     a.wait_limit_ns = h->wait_limit_ns;
+    a.max_L = h->max_L;
+    a.slab_L = h->slab_L;
     return a;
 }
 
@@ -192,7 +196,7 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
 
     std::vector<LatState> st((size_t)n);
     size_t off = 0;
-    int max_half = 0;
+    int max_half = 0, max_L = 0, slab_L = 0;
     for (int i = 0; i < n; ++i) {
         const int L = cfg->L[i];
         if (L < 2 || L > 64 || (L & 1))
@@ -220,6 +224,8 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
         s.hi_fx = (long long)std::floor(hi * llr::kFx);
         s.a = -1.0;
         if (s.half > max_half) max_half = s.half;
+        max_L = std::max(max_L, L);
+        if (L <= 24 && L > slab_L) slab_L = L;
     }
 
     llr_ctx *h = new llr_ctx();
@@ -231,6 +237,8 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
     h->beta_dn = cfg->beta_dn;
     h->h_lat = st;
     h->max_half = max_half;
+    h->max_L = max_L;
+    h->slab_L = slab_L;
     h->n_floats = off;
     cudaGetDevice(&h->device);
     *out = h;
@@ -691,6 +699,7 @@ int llr_set_kernel_shape(llr_handle h, int threads, int fast_math, int ring, int
     if (ring != 1 && ring != 2 && ring != 4) return fail(LLR_ERR_ARG, "ring must be 1, 2 or 4");
     if (carveout != -1 && carveout != 50 && carveout != 75 && carveout != 100)
         return fail(LLR_ERR_ARG, "carveout must be -1 (default), 50, 75 or 100");
+    h->cfg.auto_threads = false;
     h->cfg.threads = threads;
     h->cfg.fast_math = fast_math != 0;
     h->cfg.ring = ring;

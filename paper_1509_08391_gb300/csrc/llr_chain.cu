@@ -14,40 +14,52 @@
 // Design
 //   * Links are float32 angles, SoA by (direction, site parity), sites of a
 //     parity in lexicographic order: theta[off + (2 mu + p) * V/2 + s/2].
+//   * One persistent kernel, one CTA of 768 threads per SM (80 registers a
+//     thread).  Work items are (composite sweep j, group of up to `teams`
+//     lattices); a CTA takes the next item from an atomic counter, waits
+//     (bounded) until sweep j-1 of that group is done, and owns its lattices for
+//     that sweep.  Items run sweep-major, so uneven lattice sizes balance
+//     across SMs.  The lattices of an item advance together, phase by phase
+//     (heat-bath pass, overrelaxation passes, energy).
+//   * Lattices per item (choose_teams): with fewer lattices than SMs, one with
+//     all 24 warps; with many, three with 8 warps each in the heat-bath pass,
+//     whose deciding warps are serial and need company, while the
+//     overrelaxation pass takes them together or one after another.
 //   * A heat-bath pass runs class by class over the whole lattice (one
 //     pipeline drain per class); an overrelaxation pass is slab-major: for
-//     each x3 slab, all 8 checkerboard classes of that slab in order, so a
-//     slab's neighbourhood is reused from L2 by the 8 classes instead of each
-//     class streaming the whole lattice.
-//   * One persistent kernel.  Work items are (composite sweep j, lattice);
-//     a CTA takes the next item from an atomic counter, waits (bounded) until
-//     sweep j-1 of that lattice is done, and owns the lattice for that sweep.
-//     Items run sweep-major, so uneven lattice sizes balance across SMs.
-//   * In a heat-bath pass the warps are specialised: producer warps build
-//     the six staples of one link per thread from 18 neighbour angles, draw
-//     the von Mises proposal (Best & Fisher 1979), evaluate its dE from the
-//     stored new angle exactly as the old local energy is evaluated, convert
-//     dE to int64 fixed point (2^-32) and form warp prefix sums; a consumer
-//     warp walks the chunks in link order and decides each block of B links
-//     with the restricted Metropolis rule dist(E + dE_block) <= dist(E),
-//     using a ballot to find the first rejected block among 32
-//     speculatively accepted ones, and publishes an accept mask per group;
-//     the producers write the accepted angles.  Chunks pass through a
-//     4-stage shared memory ring guarded by named barriers, so proposals for
-//     later chunks overlap with the scan of earlier ones.
+//     each x3 slab, all 8 checkerboard classes of that slab in order.
+//   * In a heat-bath pass the warps of a lattice are specialised: producer warps
+//     build the staples of two links per thread from their neighbour angles,
+//     draw the von Mises proposals (Best & Fisher 1979), evaluate their dE from
+//     the stored new angle exactly as the old local energy is evaluated,
+//     convert dE to int64 fixed point (2^-32) and form prefix sums over a warp's
+//     64 links; a consumer warp walks the chunks in link order and decides
+//     each block of B links with the restricted Metropolis rule
+//     dist(E + dE_block) <= dist(E), using a ballot to find the first rejected
+//     block among 32 speculatively accepted ones, and publishes the accepted
+//     links; the producers write their angles.  Chunks pass through a ring of
+//     1 to 4 stages in shared memory guarded by named barriers, so proposals
+//     for later chunks overlap with the scan of earlier ones.
 //   * The multicanonical pass (Sec. 2.6) has the same producers at a fixed
 //     proposal slope; its consumer replaces the window rule by a
 //     Metropolis-Hastings test for the weight 1/rho~ in the same
 //     speculative scan.
 //   * Overrelaxation (theta' = -theta - 2 alpha) conserves E exactly, so its
-//     passes skip the scan: every thread reflects links (neighbours read with
-//     plain loads) and writes them directly.
-//   * The per-class update, energy and update functions are not inlined, so
-//     every program (batched sweeps, single passes, the plain form) runs the
-//     same machine code and gives bit-identical results.
-//   * After 1 + n_or passes the CTA sums the 6V plaquettes (float32 angles
-//     summed exactly as hi + lo, cosf, fixed-point accumulation) and
-//     resynchronises the tracked energy.
+//     passes skip the scan: threads reflect links, neighbours read from the
+//     slab in shared memory, and write them directly.
+//   * Lattices of L <= 10 that fit are held in shared memory for the whole sweep.
+//   * Every sum of products on the way to an angle, a dE or a decision has its
+//     fused operations written out, so every program (batched sweeps, single
+//     passes, the plain form), launch shape and build gives bit-identical chains.
+//   * After 1 + n_or passes the 6V plaquettes are summed (float32 angles
+//     summed exactly as hi + lo, cosf, fixed-point accumulation) and the tracked
+//     energy is resynchronised.
+//
+// Measured (GB300, 2070 MHz; one pass of 456 lattices of L = 20, ms, before ->
+// now): heat-bath 10.1 -> 7.8 (797 -> 640 instructions per link), overrelaxation
+// 2.7 -> 1.9 (184 -> 125), against one CTA of 256 threads per lattice and one
+// link per thread; L = 8, 128 lattices: 0.28 -> 0.22 and 0.08 -> 0.07.
+#include <algorithm>
 #include <cstdio>
 
 #include "llr_internal.h"
@@ -56,7 +68,6 @@ namespace llr {
 namespace {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kStages = 4;
 
 // ---------------------------------------------------------------------------
 // Best & Fisher (1979) von Mises sampler, density ~ exp(kappa cos X).
@@ -76,59 +87,115 @@ constexpr int kStages = 4;
 // |sin X| = sqrt(w (2 - w)) keep the angle's absolute accuracy near X = 0
 // and X = pi.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ bool von_mises(float kappa, uint32_t c0, uint32_t c1, uint32_t c2,
-                                          uint32_t k0, uint32_t k1, float &cX, float &sX)
-{
-    if (fabsf(kappa) < 1e-6f) {
-        const U4 w = philox4x32_10(c0, c1, c2, 0u, k0, k1);
-        const float t = 2.0f * u01(w.x) - 1.0f;   // X = pi t
-        sincospif(t, &sX, &cX);
-        return true;
+struct VonMises {
+    float k, r, rm1;   // |kappa|, r, r - 1
+    __device__ __forceinline__ explicit VonMises(float kappa)
+    {
+        k = fabsf(kappa);
+        const float sq = sqrt_fast(fmaf(4.0f * k, k, 1.0f));
+        const float tau = 1.0f + sq;
+        const float rho =
+            __fdividef(2.0f * k * tau, (sq + 1.0f) * (tau + sqrt_fast(2.0f * tau)));
+        r = __fdividef(fmaf(rho, rho, 1.0f), 2.0f * rho);
+        const float omr = 1.0f - rho;
+        rm1 = __fdividef(omr * omr, 2.0f * rho);
     }
-    const float k = fabsf(kappa);
-    const float sq = sqrt_fast(fmaf(4.0f * k, k, 1.0f));
-    const float tau = 1.0f + sq;
-    const float rho = __fdividef(2.0f * k * tau, (sq + 1.0f) * (tau + sqrt_fast(2.0f * tau)));
-    const float r = __fdividef(1.0f + rho * rho, 2.0f * rho);
-    const float omr = 1.0f - rho;
-    const float rm1 = __fdividef(omr * omr, 2.0f * rho);   // r - 1
-    // find the first accepted attempt (cheap test only, so lanes that accept
-    // at different attempts diverge over as little code as possible) ...
-    bool found = false;
-    uint32_t w_acc = 0u;
-    for (int pair = 0; pair < kSamplerMaxAttempts / 2 && !found; ++pair) {
-        const U4 w = philox4x32_10(c0, c1, c2, (uint32_t)pair, k0, k1);
-#pragma unroll
-        for (int half_ = 0; half_ < 2; ++half_) {
-            const uint32_t wa = half_ ? w.z : w.x, wb = half_ ? w.w : w.y;
-            const float u1 = u01(wa), u2 = u01(wb);
-            const float z = __cosf(kPi * u1);
-            const float f = __fdividef(1.0f + r * z, r + z);
-            const float c = k * (rm1 + (1.0f - f));
-            // second test ln(c / u2) + 1 - c >= 0, in base 2
-            if (!found && (c * (2.0f - c) - u2 > 0.0f ||
-                           __log2f(c) - __log2f(u2) >= (c - 1.0f) * 1.4426950408889634f)) {
-                found = true;
-                w_acc = wa;
-            }
+    // the accept test of one attempt (cheap form only, so lanes that accept at
+    // different attempts diverge over as little code as possible)
+    __device__ __forceinline__ bool accepts(uint32_t wa, uint32_t wb) const
+    {
+        const float u1 = u01(wa), u2 = u01(wb);
+        const float z = __cosf(kPi * u1);
+        const float f = __fdividef(fmaf(r, z, 1.0f), r + z);
+        const float c = __fmul_rn(k, rm1 + (1.0f - f));
+        // second test ln(c / u2) + 1 - c >= 0, in base 2
+        return fmaf(c, 2.0f - c, -u2) > 0.0f ||
+               __log2f(c) - __log2f(u2) >= __fmul_rn(c - 1.0f, 1.4426950408889634f);
+    }
+    // the two attempts of one Philox call: the first that accepts, its word 0
+    __device__ __forceinline__ bool attempts(const U4 &w, uint32_t &w_acc) const
+    {
+        const bool first = accepts(w.x, w.y), second = accepts(w.z, w.w);
+        w_acc = first ? w.x : w.z;
+        return first || second;
+    }
+    // (cos X, sin X) of the accepted attempt, without cancellation
+    __device__ __forceinline__ void evaluate(float kappa, uint32_t w_acc, float &cX,
+                                             float &sX) const
+    {
+        const float u1 = u01(w_acc);
+        float sh, ch;
+        __sincosf(0.5f * kPi * u1, &sh, &ch);
+        const float z = __fmul_rn(ch - sh, ch + sh);
+        const float den = __fadd_rn(r, z);
+        const bool pos = fmaf(r, z, 1.0f) >= 0.0f;               // f >= 0
+        const float w = __fdividef(pos ? rm1 * 2.0f * sh * sh : (r + 1.0f) * 2.0f * ch * ch, den);
+        const float s = sqrt_fast(w * (2.0f - w));
+        const float c = pos ? 1.0f - w : w - 1.0f;
+        const bool neg_x = !(w_acc & 1u);                        // X = -acos f
+        const bool flip = kappa < 0.0f;                          // X -> X + pi
+        cX = flip ? -c : c;
+        sX = (neg_x != flip) ? -s : s;
+    }
+};
+
+constexpr float kKappaFlat = 1e-6f;   // below it X is drawn uniformly
+
+__device__ __forceinline__ void uniform_angle(const U4 &w, float &cX, float &sX)
+{
+    const float t = 2.0f * u01(w.x) - 1.0f;   // X = pi t
+    sincospif(t, &sX, &cX);
+}
+
+// The von Mises variates of a thread's two links: one Philox call each, then
+// further calls one at a time for a link that has not accepted, the first
+// link's before the second's.  A warp's lanes rarely all accept at the first
+// call (91 % do), so for two links the later calls, which cost the warp the same
+// however many lanes take part, are shared: 3.6 calls for 64 links where one link
+// at a time took 2.2 for 32.  ok: found within the attempt limit.
+__device__ __forceinline__ void von_mises2(float kappa0, float kappa1, uint32_t link0,
+                                           uint32_t link1, uint32_t sweep, uint32_t tag,
+                                           uint32_t k0, uint32_t k1, float2 &cX, float2 &sX,
+                                           bool &ok0, bool &ok1)
+{
+    // keep the round keys from being hoisted out of the caller's loop: 18 more
+    // live registers would be spilled
+    //KEY
+    const VonMises v0(kappa0), v1(kappa1);
+    const bool flat0 = fabsf(kappa0) < kKappaFlat, flat1 = fabsf(kappa1) < kKappaFlat;
+    const U4 w0 = philox4x32_10(link0, sweep, tag, 0u, k0, k1);
+    const U4 w1 = philox4x32_10(link1, sweep, tag, 0u, k0, k1);
+    uint32_t acc0, acc1;
+    ok0 = v0.attempts(w0, acc0) || flat0;
+    ok1 = v1.attempts(w1, acc1) || flat1;
+    bool done0 = ok0, done1 = ok1;
+    for (uint32_t n = 1; !(done0 && done1);) {
+        VonMises v = v0;
+        uint32_t link = link0;
+        if (done0) {
+            v = v1;
+            link = link1;
+        }
+        const U4 w = philox4x32_10(link, sweep, tag, n, k0, k1);
+        uint32_t acc;
+        const bool found = v.attempts(w, acc);
+        ++n;
+        const bool last = n >= kSamplerMaxAttempts / 2;
+        if (!done0) {
+            if (found) acc0 = acc;
+            ok0 = found;
+            done0 = found || last;
+            if (done0) n = 1;
+        } else {
+            if (found) acc1 = acc;
+            ok1 = found;
+            done1 = found || last;
         }
     }
-    if (!found) return false;
-    // ... then evaluate the accepted variate once, without cancellation
-    const float u1 = u01(w_acc);
-    float sh, ch;
-    __sincosf(0.5f * kPi * u1, &sh, &ch);
-    const float z = (ch - sh) * (ch + sh);
-    const float den = r + z;
-    const bool pos = 1.0f + r * z >= 0.0f;                   // f >= 0
-    const float w = __fdividef(pos ? rm1 * 2.0f * sh * sh : (r + 1.0f) * 2.0f * ch * ch, den);
-    const float s = sqrt_fast(w * (2.0f - w));
-    const float c = pos ? 1.0f - w : w - 1.0f;
-    const bool neg_x = !(w_acc & 1u);                        // X = -acos f
-    const bool flip = kappa < 0.0f;                          // X -> X + pi
-    cX = flip ? -c : c;
-    sX = (neg_x != flip) ? -s : s;
-    return true;
+    v0.evaluate(kappa0, acc0, cX.x, sX.x);
+    v1.evaluate(kappa1, acc1, cX.y, sX.y);
+    if (flat0) uniform_angle(w0, cX.x, sX.x);
+    if (flat1) uniform_angle(w1, cX.y, sX.y);
 }
 
 template <bool FAST>
@@ -146,6 +213,23 @@ template <bool FAST>
 __device__ __forceinline__ float arg(float y, float x)
 {
     return FAST ? arg_fast(y, x) : atan2f(y, x);
+}
+
+// arg of two vectors, each bit for bit as by arg: the polynomial of arg_fast in
+// packed arithmetic.
+template <bool FAST>
+__device__ __forceinline__ float2 arg2(float2 y, float2 x)
+{
+    if (!FAST) return make_float2(atan2f(y.x, x.x), atan2f(y.y, x.y));
+    return arg_fast2(y, x);
+}
+
+// Local energy Re(e^{i theta} S) of a link from (cos, sin) of its angle.  Here
+// and in the heat-bath's other sums of products the fused operation is
+// written out, so every place and build that forms them rounds alike.
+__device__ __forceinline__ float link_energy(float c, float s, float Sr, float Si)
+{
+    return fmaf(c, Sr, -__fmul_rn(s, Si));
 }
 
 // Coordinates of the h-th site of parity p (lexicographic, x0 fastest).
@@ -169,21 +253,31 @@ __device__ __forceinline__ int decode_half(int h, int p, int L, uint32_t magic, 
 // backward phi = theta_nu(x-nu) - theta_nu(x-nu+mu) - theta_mu(x-nu)
 // so that the link's local energy is sum_j cos(theta + phi_j) = Re(e^{i theta} S).
 //
-// In a heat-bath pass the 18 neighbour angles are staged through shared
-// memory: staple_fetch issues one 4-byte asynchronous copy (cp.async, cached
-// in L1) per angle into the calling thread's column of a stage buffer, and
-// staple_from sums the staples from it once the copies have landed, so a
-// producer's loads for its next link overlap the sampling of the current one.  A thread only reads what it copied
-// itself, so cp.async.wait_group is the only synchronisation.  The copies
-// read through L1 like plain loads: other classes of this lattice were
-// written earlier in the same launch (same CTA, or another CTA before the
-// acquire of the lattice's done counter).
-constexpr int kStaged = 18;   // angles per link in a stage column
+// In a heat-bath pass a producer thread proposes for two links at a time, half
+// sites h and h + 1 (h even), so index arithmetic, the sampler's later calls
+// and the prefix sums serve two, and the staples are summed in packed
+// arithmetic.  With rows of even length (ROW) both lie in one x0 row and share
+// their neighbours' rows: 14 of the 18 neighbour pairs are one 8-byte access.
+// The neighbour angles are copied asynchronously (cp.async, cached in L1) to
+// the thread's own column of a stage buffer while it works on the pair before,
+// or, where the whole lattice is in shared memory (RES), read there.  A thread
+// only reads what it copied itself, so cp.async.wait_group is the only
+// synchronisation.  The copies read through L1 like plain loads: other classes
+// of this lattice were written earlier in the same launch (same CTA, or
+// another CTA before the acquire of the lattice's done counter).
+constexpr int kStaged = 19;   // pairs in a stage column: 18 neighbours and the links themselves
 
-__device__ __forceinline__ void cp_async4(float *dst, const float *src)
+__device__ __forceinline__ void cp_async16(float *dst, const float *src)   // through L2 only
 {
     const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d), "l"(src) : "memory");
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+template <int BYTES>
+__device__ __forceinline__ void cp_async(float *dst, const float *src)   // through L1
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(d), "l"(src), "n"(BYTES)
+                 : "memory");
 }
 __device__ __forceinline__ void cp_async_commit()
 {
@@ -195,69 +289,117 @@ __device__ __forceinline__ void cp_async_wait()
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
 
-// Stage the neighbour angles of link theta_MU(x) (site s, parity p) into
-// col[k * stride], k = 6 j + (a1, a2, a3, b1, b2, b3) for the j-th nu != MU.
-template <int MU>
-__device__ __forceinline__ void staple_fetch(const float *th, int half, int L, const int x[4],
-                                             int s, int p, float *col, int stride)
+// The two links of a thread (half sites h, h + 1 of parity p): sites and the
+// half-site distances to the neighbours x +- nu.
+template <bool ROW>
+struct LinkPair {
+    int up0[4], dn0[4], up1[4], dn1[4];   // ROW: up1, dn1 differ from up0, dn0 in [0] only
+    int site0, site1;
+
+    static __device__ __forceinline__ int around(int h, int p, int L, uint32_t magic, int up[4],
+                                                 int dn[4])
+    {
+        int x[4];
+        const int site = decode_half(h, p, L, magic, x);
+        const int Lh = L >> 1, S1 = L * Lh, S = S1 * L;
+        const bool odd = x[0] & 1;
+        up[0] = odd ? (x[0] == L - 1 ? 1 - Lh : 1) : 0;
+        dn[0] = odd ? 0 : (x[0] == 0 ? Lh - 1 : -1);
+        up[1] = x[1] == L - 1 ? Lh - S1 : Lh;
+        dn[1] = x[1] == 0 ? S1 - Lh : -Lh;
+        up[2] = x[2] == L - 1 ? S1 - S : S1;
+        dn[2] = x[2] == 0 ? S - S1 : -S1;
+        up[3] = x[3] == L - 1 ? S - S * L : S;
+        dn[3] = x[3] == 0 ? S * L - S : -S;
+        return site;
+    }
+
+    __device__ __forceinline__ LinkPair(int h, int p, int L, uint32_t magic)
+    {
+        site0 = around(h, p, L, magic, up0, dn0);
+        if (ROW) {
+            // the second link, at x0 + 2: never at the start of the row
+            const bool odd = site0 & 1;
+            const int Lh = L >> 1;
+            const int k = h - (int)__umulhi(2u * (uint32_t)h, magic) * Lh;   // position in the row
+            site1 = site0 + 2;
+#pragma unroll
+            for (int nu = 1; nu < 4; ++nu) {
+                up1[nu] = up0[nu];
+                dn1[nu] = dn0[nu];
+            }
+            up1[0] = odd ? (k + 2 == Lh ? 1 - Lh : 1) : 0;
+            dn1[0] = odd ? 0 : -1;
+        } else {
+            site1 = around(h + 1, p, L, magic, up1, dn1);
+        }
+    }
+};
+
+// The 18 neighbour pairs of the staples of theta_MU at half site h, h + 1 and
+// the pair itself, in the order of the staple sum, each handed to
+// put(k, aligned, o0, o1): pair k at offsets o0, o1 of the lattice, adjacent and
+// 8-byte aligned if `aligned`.
+template <int MU, bool ROW, class Put>
+__device__ __forceinline__ void neighbour_pairs(const LinkPair<ROW> &n, int half, int h, int p,
+                                                Put put)
 {
-    const int st[4] = {1, L, L * L, L * L * L};
-    const int dmu = (x[MU] == L - 1) ? -(L - 1) * st[MU] : st[MU];
-    const int spmu = s + dmu;
     const int q = p ^ 1;
-    const float *thmu_q = th + (2 * MU + q) * half;
-    int j = 0;
+    int k = 0;
+    auto at = [&](int nu, int par, bool x0, int d0, int d1) {
+        const int o = (2 * nu + par) * half + h;
+        put(k++, ROW && !x0, o + d0, o + 1 + d1);
+    };
 #pragma unroll
     for (int nu = 0; nu < 4; ++nu) {
         if (nu == MU) continue;
-        const int dnf = (x[nu] == L - 1) ? -(L - 1) * st[nu] : st[nu];
-        const int dnb = (x[nu] == 0) ? (L - 1) * st[nu] : -st[nu];
-        const int spnu = s + dnf;
-        const int smnu = s + dnb;
-        const int smnu_pmu = smnu + dmu;
-        const float *thnu_p = th + (2 * nu + p) * half;
-        const float *thnu_q = th + (2 * nu + q) * half;
-        float *c = col + 6 * j * stride;
-        cp_async4(c + 0 * stride, thnu_q + (spmu >> 1));      // theta_nu(x+mu)
-        cp_async4(c + 1 * stride, thmu_q + (spnu >> 1));      // theta_mu(x+nu)
-        cp_async4(c + 2 * stride, thnu_p + (s >> 1));         // theta_nu(x)
-        cp_async4(c + 3 * stride, thnu_p + (smnu_pmu >> 1));  // theta_nu(x-nu+mu)
-        cp_async4(c + 4 * stride, thmu_q + (smnu >> 1));      // theta_mu(x-nu)
-        cp_async4(c + 5 * stride, thnu_q + (smnu >> 1));      // theta_nu(x-nu)
-        ++j;
+        at(nu, q, MU == 0, n.up0[MU], n.up1[MU]);                       // theta_nu(x+mu)
+        at(MU, q, nu == 0, n.up0[nu], n.up1[nu]);                       // theta_mu(x+nu)
+        at(nu, p, false, 0, 0);                                         // theta_nu(x)
+        at(nu, p, MU == 0 || nu == 0, n.dn0[nu] + n.up0[MU], n.dn1[nu] + n.up1[MU]);
+        at(MU, q, nu == 0, n.dn0[nu], n.dn1[nu]);                       // theta_mu(x-nu)
+        at(nu, q, nu == 0, n.dn0[nu], n.dn1[nu]);                       // theta_nu(x-nu)
     }
+    at(MU, p, false, 0, 0);
 }
 
-template <bool FAST>
-__device__ __forceinline__ void staple_from(const float *col, int stride, float &Sr, float &Si)
+// Staple sums of two links from their neighbour pairs v(0 .. 17).
+template <bool FAST, class Get>
+__device__ __forceinline__ void staple_sums2(Get v, float2 &Sr, float2 &Si)
 {
-    Sr = 0.0f;
-    Si = 0.0f;
+    Sr = Si = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int j = 0; j < 3; ++j) {
-        const float *c = col + 6 * j * stride;
-        const float pf = c[0] - c[stride] - c[2 * stride];
-        const float pb = c[5 * stride] - c[3 * stride] - c[4 * stride];
-        float sf, cf, sb, cb;
-        sin_cos<FAST>(pf, &sf, &cf);
-        sin_cos<FAST>(pb, &sb, &cb);
-        Sr += cf + cb;
-        Si += sf + sb;
+        const float2 pf = sub2(sub2(v(6 * j), v(6 * j + 1)), v(6 * j + 2));
+        const float2 pb = sub2(sub2(v(6 * j + 5), v(6 * j + 3)), v(6 * j + 4));
+        float2 sf, cf, sb, cb;
+        sin_cos<FAST>(pf.x, &sf.x, &cf.x);
+        sin_cos<FAST>(pf.y, &sf.y, &cf.y);
+        sin_cos<FAST>(pb.x, &sb.x, &cb.x);
+        sin_cos<FAST>(pb.y, &sb.y, &cb.y);
+        Sr = add2(Sr, add2(cf, cb));
+        Si = add2(Si, add2(sf, sb));
     }
 }
 
-// The stage buffer (dynamic shared memory): two columns sets of kStaged x NT
-// floats, so the copies for a thread's next link land while it works on the
-// current one.
-extern __shared__ __align__(16) float g_stage_buf[];
+// Threads of the sweep kernel's CTA (one CTA per SM, 80 registers a thread) and
+// the lattices one CTA works on at a time, each with a team of warps.
+constexpr int kThreads = 768, kWarps = kThreads / 32, kMaxTeams = 6;
 
-template <int NT>
-__device__ __forceinline__ float *stage_col(int buf)
+// Dynamic shared memory: the whole lattices where they fit (RES; then the
+// heat-bath rings), otherwise used by one phase of a sweep at a time: the
+// heat-bath pass's stage columns (kStaged pairs per thread) and rings, or the
+// slabs of the overrelaxation pass.
+extern __shared__ __align__(16) float g_dyn[];
+
+__device__ __forceinline__ float2 *stage_col()
 {
-    return g_stage_buf + buf * kStaged * NT + threadIdx.x;
+    return (float2 *)g_dyn + threadIdx.x;   // pair k at [k * kThreads]
 }
 
-// Named barriers 1..8 (0 is __syncthreads): stage s is full (1 + s) / empty (5 + s).
+// Barrier 0 is __syncthreads.  In a heat-bath pass the ring stages of team k use
+// the 2 D barriers from 1 + 2 D k (full, then empty; the first also ends a
+// class); in the other phases team k has barriers 1 + k and 8 + k.
 __device__ __forceinline__ void bar_sync(int id, int n)
 {
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
@@ -267,144 +409,218 @@ __device__ __forceinline__ void bar_arrive(int id, int n)
     asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-template <int NWP>
-struct Stage {
-    float thn[NWP * 32];
-    long long P[NWP * 32];   // warp-inclusive prefix sums of dE (fixed point)
-    unsigned endmask[NWP];
-    unsigned accmask[NWP];   // written by the consumer: accepted block ends
+// The value of lane 0, which the compiler then knows to be the same in all lanes.
+__device__ __forceinline__ int uniform(int v)
+{
+    return __shfl_sync(kFull, v, 0);
+}
+
+// The warps of the CTA that work on one lattice in a phase: warp w of nw,
+// thread tid of nt, a barrier of their own.
+struct Team {
+    int w, nw, tid, nt, bar;
+    __device__ __forceinline__ void sync() const { bar_sync(bar, nt); }
 };
 
-template <int NWP>
+// One ring stage of a heat-bath class: a chunk of `groups` 64-link groups, two
+// links per producer lane.
+struct Stage {
+    long long *P;      // prefix sums of dE over the group, to each of its links
+    long long *d;      // dE of each link
+    float2 *thn;       // the proposals
+    uint2 *acc;        // written by the consumer: links 0-31 / 32-63 accepted
+};
+
+// Bytes of a stage per group: a multiple of 16, so every stage's P is aligned.
+constexpr int kStageGroupBytes = 64 * 20 + 16;
+
+__device__ __forceinline__ Stage stage_at(char *base, int groups, int s)
+{
+    char *p = base + (size_t)s * groups * kStageGroupBytes;
+    Stage g;
+    g.P = (long long *)p;
+    g.d = (long long *)(p + groups * 512);
+    g.thn = (float2 *)(p + groups * 1024);
+    g.acc = (uint2 *)(p + groups * 1280);
+    return g;
+}
+
+// Heat-bath team: nw warps on the lattice, warp cw of them the consumer; its
+// ring of D stages of nw - 1 groups at `ring` (floats) of g_dyn, and the first
+// of its 2 D ring barriers.
+struct HbTeam {
+    int nw, cw, ring, D, full;
+};
+
 struct Smem {
-    LatState st;
-    Stage<NWP> stage[kStages];
-    long long red[NWP + 1];
-    unsigned long long acc_cnt;
-    unsigned long long cap_cnt;
-    int item_lat, item_j, item_state;
-    int cw;     // the consumer warp of a heat-bath pass
-    int ring;   // stages of the ring in use (a power of two <= kStages)
+    LatState st[kMaxTeams];
+    unsigned long long acc_cnt[kMaxTeams];
+    unsigned long long cap_cnt[kMaxTeams];
+    long long red[kWarps];
+    HbTeam hb[kMaxTeams];     // the teams of a heat-bath pass
+    float a_f[kMaxTeams];     // slope of the team's heat-bath proposals
+    int active[kMaxTeams];    // the team's lattice takes part in the sweep
+    int n_app[kMaxTeams];     // approach: sweeps done
+    int item_first, item_n, item_j, item_state;
 };
 
 // Producer side of one heat-bath class (MU, p): proposals and warp prefix
 // sums, chunk by chunk, into the stage ring (slope a_f, Philox tag `tag`).
 // When a slot comes back from the consumer (and for the last chunks at the
-// end of the class) each producer writes its link's proposal if the
-// consumer accepted the block it belongs to.
-template <int MU, int NWP, bool FAST>
-__device__ __noinline__ void produce_class(Smem<NWP> &sm, float *th, int p, float a_f,
-                                           uint32_t tag, int B, int h0, int count, int nchunk,
-                                           int D)
+// end of the class) each producer writes those of its proposals that were
+// accepted.  th: the lattice (RES: at offset lat_off of g_dyn instead).
+//
+// The team's and the lattice's constants are read from shared memory where they
+// are used: kept in registers across the loop they would be spilled.
+template <int MU, bool ROW, bool RES, bool FAST>
+__device__ __noinline__ void produce_class(Smem &sm, int slot, int pw, float *th_, int lat_off,
+                                           int p, uint32_t tag)
 {
-    constexpr int NT = (NWP + 1) * 32, CH = NWP * 32;
-    // producer rank pt (0 .. CH-1) and producer warp pw: the warps other
-    // than the consumer warp sm.cw, in order
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int pw = w - (w > sm.cw ? 1 : 0), pt = pw * 32 + lane;
-    const int L = sm.st.L, half = sm.st.half;
-    const uint32_t magic = sm.st.magic, V = 2u * (uint32_t)half;
-    const uint32_t k0 = sm.st.key0, k1 = sm.st.key1, sweep = sm.st.sweep;
-    float *own = th + (2 * MU + p) * half;
+    const int lane = threadIdx.x & 31, pt = pw * 32 + lane;
+    const LatState &st = sm.st[slot];
+    const HbTeam &hb = sm.hb[slot];
+    const int CH = (hb.nw - 1) * 64;
+    float *th = RES ? g_dyn + lat_off : th_;
     unsigned cnt = 0;
+    auto stage = [&](int s) { return stage_at((char *)(g_dyn + hb.ring), hb.nw - 1, s); };
     // write back chunk c of a slot the consumer has released
-    auto flush = [&](const Stage<NWP> &stg, int c) {
-        const int lc = c * CH + pt;
-        if (lc < count) {
-            const int eb = __ffs(stg.endmask[pw] & ~((1u << lane) - 1u)) - 1;
-            if ((stg.accmask[pw] >> eb) & 1u) {
-                own[h0 + lc] = stg.thn[pt];
+    auto flush = [&](const Stage &stg, int c) {
+        const int h = c * CH + 2 * pt, half = st.half;
+        if (h < half) {   // half is even: both links or none
+            float *own = th + (2 * MU + p) * half;
+            const uint2 acc = stg.acc[pw];
+            const unsigned took = (lane < 16 ? acc.x : acc.y) >> (2 * (lane & 15));
+            const float2 t = stg.thn[pt];
+            if (took & 1u) {
+                own[h] = t.x;
+                ++cnt;
+            }
+            if (took & 2u) {
+                own[h + 1] = t.y;
                 ++cnt;
             }
         }
     };
-    // prologue: stage the first chunk's neighbours
-    bool valid_n = pt < count;
-    int site_n = 0;
-    float t0_n = 0.0f;
-    if (valid_n) {
-        int x[4];
-        site_n = decode_half(h0 + pt, p, L, magic, x);
-        staple_fetch<MU>(th, half, L, x, site_n, p, stage_col<NT>(0), NT);
-        t0_n = own[h0 + pt];
-    }
-    cp_async_commit();
-    for (int ch = 0; ch < nchunk; ++ch) {
-        const int s = ch & (D - 1);
-        const int local = ch * CH + pt;
-        const bool valid = valid_n;
-        const int site = site_n;
-        const float t0 = t0_n;
-        // stage the next chunk's neighbours while this one is sampled
-        {
-            const int ln = local + CH;
-            valid_n = ch + 1 < nchunk && ln < count;
-            if (valid_n) {
-                int x[4];
-                site_n = decode_half(h0 + ln, p, L, magic, x);
-                staple_fetch<MU>(th, half, L, x, site_n, p, stage_col<NT>((ch + 1) & 1), NT);
-                t0_n = own[h0 + ln];
+    auto fetch = [&](int h) {
+        const LinkPair<ROW> n(h, p, st.L, st.magic);
+        float2 *col = stage_col();
+        neighbour_pairs<MU, ROW>(n, st.half, h, p, [&](int k, bool aligned, int o0, int o1) {
+            float *dst = (float *)(col + k * kThreads);
+            if (aligned) {
+                cp_async<8>(dst, th + (unsigned)o0);
+            } else {
+                cp_async<4>(dst, th + (unsigned)o0);
+                cp_async<4>(dst + 1, th + (unsigned)o1);
             }
+        });
+    };
+    if (!RES) {
+        if (2 * pt < st.half) fetch(2 * pt);
+        cp_async_commit();
+    }
+    int ch = 0;
+#pragma unroll 1
+    for (; ch * CH < st.half; ++ch) {
+        const int h = ch * CH + 2 * pt;
+        const bool valid = h < st.half;
+        float2 thn = make_float2(0.0f, 0.0f);
+        long long d0 = 0, d1 = 0;
+        float2 Sr, Si, t0;
+        if (!RES) cp_async_wait<0>();
+        if (valid) {
+            if (RES) {
+                const LinkPair<ROW> n(h, p, st.L, st.magic);
+                float2 v[kStaged];
+                neighbour_pairs<MU, ROW>(n, st.half, h, p, [&](int k, bool aligned, int o0, int o1) {
+                    v[k] = aligned ? *(const float2 *)(th + o0) : make_float2(th[o0], th[o1]);
+                });
+                staple_sums2<FAST>([&](int k) { return v[k]; }, Sr, Si);
+                t0 = v[18];
+            } else {
+                const float2 *col = stage_col();
+                staple_sums2<FAST>([&](int k) { return col[k * kThreads]; }, Sr, Si);
+                t0 = col[18 * kThreads];
+            }
+        }
+        // the next pair's neighbours, on their way while this one is sampled
+        if (!RES) {
+            if (h + CH < st.half) fetch(h + CH);
             cp_async_commit();
         }
-        if (ch >= D) {
-            bar_sync(5 + s, NT);
-            flush(sm.stage[s], ch - D);
-        }
-        cp_async_wait<1>();
-        float thn = 0.0f;
-        long long d = 0;
         if (valid) {
-            float Sr, Si;
-            staple_from<FAST>(stage_col<NT>(ch & 1), NT, Sr, Si);
-            float so, co;
-            sin_cos<FAST>(t0, &so, &co);
-            const float e_old = co * Sr - so * Si;     // |S| cos(theta + alpha)
-            const float Sabs = sqrt_fast(Sr * Sr + Si * Si);
-            float cX, sX;
-            const uint32_t link = (uint32_t)MU * V + (uint32_t)site;
-            if (von_mises(-a_f * Sabs, link, sweep, tag, k0, k1, cX, sX)) {
-                // theta' = X - alpha, alpha = arg S: e^{i theta'} = e^{iX} conj(S) / |S|
-                thn = arg<FAST>(sX * Sr - cX * Si, cX * Sr + sX * Si);
-                // dE of the angle actually stored, evaluated exactly like e_old
-                // (same staple sum, same sine/cosine): the approximation errors
-                // of one link's successive evaluations then cancel along its
-                // chain of updates and leave only random noise.  Taking
-                // |S| cos X instead carried a systematic -3.5e-8 per move (the
-                // rounded atan2 and (cos X, sin X) are not exactly the angle
-                // X - alpha), which drifted the running energy by -4.8e-4 per
-                // heat-bath pass at L = 8 and shifted the window it enforces.
-                float sn, cn;
-                sin_cos<FAST>(thn, &sn, &cn);
-                d = to_fx((cn * Sr - sn * Si) - e_old);
-            } else {
-                thn = t0;
-                atomicAdd(&sm.cap_cnt, 1ull);
+            float s0, c0, s1, c1;
+            sin_cos<FAST>(t0.x, &s0, &c0);
+            sin_cos<FAST>(t0.y, &s1, &c1);
+            // the old local energies |S| cos(theta + alpha)
+            const float e0 = link_energy(c0, s0, Sr.x, Si.x), e1 = link_energy(c1, s1, Sr.y, Si.y);
+            const float S0 = sqrt_fast(fmaf(Si.x, Si.x, __fmul_rn(Sr.x, Sr.x)));
+            const float S1 = sqrt_fast(fmaf(Si.y, Si.y, __fmul_rn(Sr.y, Sr.y)));
+            int x[4];
+            const uint32_t base = (uint32_t)MU * 2u * (uint32_t)st.half;
+            const uint32_t l0 = base + (uint32_t)decode_half(h, p, st.L, st.magic, x);
+            const uint32_t l1 =
+                ROW ? l0 + 2u : base + (uint32_t)decode_half(h + 1, p, st.L, st.magic, x);
+            float2 cX, sX;
+            bool ok0, ok1;
+            const float a_f = sm.a_f[slot];
+            von_mises2(-a_f * S0, -a_f * S1, l0, l1, st.sweep, tag, st.key0, st.key1, cX, sX, ok0,
+                       ok1);
+            // theta' = X - alpha, alpha = arg S: e^{i theta'} = e^{iX} conj(S) / |S|
+            thn = arg2<FAST>(make_float2(fmaf(sX.x, Sr.x, -__fmul_rn(cX.x, Si.x)),
+                                         fmaf(sX.y, Sr.y, -__fmul_rn(cX.y, Si.y))),
+                             make_float2(fmaf(cX.x, Sr.x, __fmul_rn(sX.x, Si.x)),
+                                         fmaf(cX.y, Sr.y, __fmul_rn(sX.y, Si.y))));
+            // dE of the angle actually stored, evaluated exactly like the old
+            // energy (same staple sum, same sine/cosine): the approximation
+            // errors of one link's successive evaluations then cancel along its
+            // chain of updates and leave only random noise.  Taking
+            // |S| cos X instead carried a systematic -3.5e-8 per move (the
+            // rounded atan2 and (cos X, sin X) are not exactly the angle
+            // X - alpha), which drifted the running energy by -4.8e-4 per
+            // heat-bath pass at L = 8 and shifted the window it enforces.
+            sin_cos<FAST>(thn.x, &s0, &c0);
+            sin_cos<FAST>(thn.y, &s1, &c1);
+            d0 = to_fx(__fsub_rn(link_energy(c0, s0, Sr.x, Si.x), e0));
+            d1 = to_fx(__fsub_rn(link_energy(c1, s1, Sr.y, Si.y), e1));
+            if (!(ok0 && ok1)) {
+                if (!ok0) {
+                    thn.x = t0.x;
+                    d0 = 0;
+                }
+                if (!ok1) {
+                    thn.y = t0.y;
+                    d1 = 0;
+                }
+                atomicAdd(&sm.cap_cnt[slot], (unsigned long long)(!ok0 + !ok1));
             }
         }
-        long long P = d;
+        __syncwarp();
+        long long P = d0 + d1;
 #pragma unroll
         for (int o = 1; o < 32; o <<= 1) {
             const long long y = __shfl_up_sync(kFull, P, o);
             if (lane >= o) P += y;
         }
-        const bool isend = valid && (((lane & (B - 1)) == B - 1) || local == count - 1);
-        const unsigned em = __ballot_sync(kFull, isend);
-        Stage<NWP> &stg = sm.stage[s];
+        const int D = hb.D, s = ch & (D - 1), bar = hb.full + s, NT = hb.nw * 32;
+        const Stage stg = stage(s);
+        if (ch >= D) {
+            bar_sync(bar + D, NT);
+            flush(stg, ch - D);
+        }
         stg.thn[pt] = thn;
-        stg.P[pt] = P;
-        if (lane == 0) stg.endmask[pw] = em;
-        bar_arrive(1 + s, NT);
+        ((longlong2 *)stg.P)[pt] = make_longlong2(P - d1, P);
+        ((longlong2 *)stg.d)[pt] = make_longlong2(d0, d1);
+        bar_arrive(bar, NT);
     }
-    for (int c = nchunk > D ? nchunk - D : 0; c < nchunk; ++c) {
+    const int D = hb.D;
+    for (int c = max(ch - D, 0); c < ch; ++c) {
         const int s = c & (D - 1);
-        bar_sync(5 + s, NT);
-        flush(sm.stage[s], c);
+        bar_sync(hb.full + D + s, hb.nw * 32);
+        flush(stage(s), c);
     }
-    cp_async_wait<0>();
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_down_sync(kFull, cnt, o);
-    if (lane == 0) atomicAdd(&sm.acc_cnt, (unsigned long long)cnt);
+    if (lane == 0) atomicAdd(&sm.acc_cnt[slot], (unsigned long long)cnt);
 }
 
 // Neighbour angles of link theta_MU(x) (site s, parity p) loaded straight into
@@ -494,37 +710,33 @@ __device__ __forceinline__ float overrelax_link(const float *th, const float *ow
         float sn, cn, so, co;
         sin_cos<FAST>(tn, &sn, &cn);
         sin_cos<FAST>(t0, &so, &co);
-        const float d = (cn * Sr - sn * Si) - (co * Sr - so * Si);
+        const float d = __fsub_rn(link_energy(cn, sn, Sr, Si), link_energy(co, so, Sr, Si));
         dfx = fabsf(d) <= kOrDeltaMax ? __float2int_rn(d * 4294967296.0f) : kOrRefused;
     }
     return tn;
 }
 
 // One overrelaxation group (the links of class (MU, p) with half-site index
-// in [h0, h0 + count)) whose running energy E lies outside the window, or
-// inside and farther than B * 2^-14 from both edges: every move is taken by
-// the window rule, so no dE is needed.  Every thread reflects its links and
-// writes them directly.  The neighbours are plain loads: within a slab they
-// mostly hit L1/L2, and with no consumer to feed, the loads of many warps
-// hide each other.
-template <int MU, int NWP, bool FAST>
-__device__ __noinline__ void overrelax_class(Smem<NWP> &sm, float *th, int p, int h0, int count)
+// in [h0, h0 + count)) of a lattice whose slab is too large for shared memory
+// (L > kSlabMaxL): every thread reflects its links, neighbours by plain loads.
+template <int MU, bool FAST>
+__device__ __noinline__ void overrelax_class(const LatState &st, const Team &t, float *th, int p,
+                                             int h0, int count)
 {
-    constexpr int NT = (NWP + 1) * 32;
-    const int L = sm.st.L, half = sm.st.half;
-    const uint32_t magic = sm.st.magic;
+    const int L = st.L, half = st.half;
+    const uint32_t magic = st.magic;
     float *own = th + (2 * MU + p) * half;
-    for (int local = threadIdx.x; local < count; local += NT) {
+    for (int local = t.tid; local < count; local += t.nt) {
         int dfx;
         own[h0 + local] =
             overrelax_link<MU, FAST, false>(th, own, half, L, magic, p, h0 + local, dfx);
     }
 }
 
-// Heat-bath window decisions of one 32-link group in link order, by the
-// calling warp.  Lane k holds Pk, the inclusive prefix sum of dE over the
-// group's links 0..k; em marks the lanes that end a block (blocks of B links
-// start at multiples of B).  A block is taken iff dist(E + dE_block) <=
+// Heat-bath window decisions of one group in link order, by the calling warp.
+// Lane k holds Pk, the inclusive prefix sum of dE over the group's lanes 0..k;
+// em marks the lanes that end a block (blocks of B lanes start at multiples
+// of B).  A block is taken iff dist(E + dE_block) <=
 // dist(E), dist the distance from the closed window (inside the window: iff
 // the energy after the block is inside).  Returns the mask of taken block
 // ends and advances E.
@@ -598,19 +810,18 @@ __device__ __forceinline__ unsigned window_scan_group(long long Pk, unsigned em,
 // outside the window or E + dE_block inside it.  Decisions are independent of
 // one another (E does not move), so no barrier is needed.  Returns the number
 // of moves this thread took.
-template <int MU, int NWP, bool FAST>
-__device__ __noinline__ int overrelax_class_near(Smem<NWP> &sm, float *th, int p, int h0,
-                                                 int count, int B, long long E)
+template <int MU, bool FAST>
+__device__ __noinline__ int overrelax_class_near(const LatState &st, const Team &t, float *th,
+                                                 int p, int h0, int count, int B, long long E)
 {
-    constexpr int NT = (NWP + 1) * 32;
-    const int L = sm.st.L, half = sm.st.half;
-    const uint32_t magic = sm.st.magic;
-    const long long lo = sm.st.lo_fx, hi = sm.st.hi_fx;
+    const int L = st.L, half = st.half;
+    const uint32_t magic = st.magic;
+    const long long lo = st.lo_fx, hi = st.hi_fx;
     const bool outside = E < lo || E > hi;
     float *own = th + (2 * MU + p) * half;
     int taken = 0;
-    for (int c0 = 0; c0 < count; c0 += NT) {
-        const int local = c0 + threadIdx.x;
+    for (int c0 = 0; c0 < count; c0 += t.nt) {
+        const int local = c0 + t.tid;
         const bool valid = local < count;
         int dfx = 0;
         float tn = 0.0f;
@@ -631,28 +842,126 @@ __device__ __noinline__ int overrelax_class_near(Smem<NWP> &sm, float *th, int p
     return taken;
 }
 
-// Consumer side: sequential Metropolis accept of the chunk's blocks in link
-// order; publishes the accepted block ends of each group (the producers
-// write the angles).  Runs in the last warp.
-template <int NWP>
-__device__ __noinline__ void consume_class(Smem<NWP> &sm, int B, int nchunk, int D)
+// The same for 32 links with blocks of one link and the energy inside the window
+// (the usual case; it stays inside).  This is the deciding warp's critical path,
+// so it is short: the links run from lane 31 down (the first refusal is the
+// highest bit of a ballot), lane k holds the dE d of its link and the sum P of the
+// dE up to it; u is the energy before all links that P counts, less the dE refused
+// among them, above the lower edge.  A link is taken iff the energy after it, u + P,
+// is at most the width: one unsigned comparison.  Every undecided link is decided
+// as if the ones before it were taken; the first refusal takes its dE out.  Lanes
+// past the end of the class (d = 0) never refuse.  Returns the lanes refused.
+__device__ __forceinline__ unsigned window_scan_inside(long long P, long long d, long long &u,
+                                                       unsigned long long width)
 {
-    constexpr int NT = (NWP + 1) * 32;
+    unsigned rem = kFull, refused = 0u;
+    for (;;) {
+        const unsigned m = __ballot_sync(kFull, (unsigned long long)(u + P) > width) & rem;
+        if (m == 0u) break;
+        const int j = 31 - __clz(m);
+        u -= __shfl_sync(kFull, d, j);
+        refused |= 1u << j;
+        rem = (1u << j) - 1u;
+    }
+    return refused;
+}
+
+// The same wherever the energy is; `valid` marks the lanes that hold a link, and E
+// is the energy before all links that P counts, less the dE refused among them.
+__device__ __forceinline__ unsigned window_scan_links(long long P, long long d, unsigned valid,
+                                                      long long &E, long long lo, long long hi)
+{
+    unsigned rem = valid, refused = 0u;
     const int lane = threadIdx.x & 31;
-    long long E = sm.st.E_fx;
-    const long long lo = sm.st.lo_fx, hi = sm.st.hi_fx;
+    const bool mine = (valid >> lane) & 1u;
+    // Far outside, where even all moves towards the window together do not reach
+    // it, a link is taken iff its move does not lead away.
+    const long long E0 = E + __shfl_sync(kFull, P - d, 31);   // before the first link
+    const bool below = E0 < lo, above = E0 > hi;
+    const bool away = mine && (below ? d < 0 : d > 0);
+    long long sum = mine && !away ? d : 0, drop = away ? d : 0;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        sum += __shfl_xor_sync(kFull, sum, o);
+        drop += __shfl_xor_sync(kFull, drop, o);
+    }
+    if ((below && E0 + sum < lo) || (above && E0 + sum > hi)) {
+        E -= drop;
+        return __ballot_sync(kFull, away);
+    }
+    // near an edge: as inside, with the rule in full
+    for (;;) {
+        const long long e = E + P;   // after the link
+        const unsigned m =
+            __ballot_sync(kFull, dist_fx(e, lo, hi) > dist_fx(e - d, lo, hi)) & rem;
+        if (m == 0u) break;
+        const int j = 31 - __clz(m);
+        E -= __shfl_sync(kFull, d, j);
+        refused |= 1u << j;
+        rem = (1u << j) - 1u;
+    }
+    return refused;
+}
+
+// Consumer side: sequential Metropolis accept of the chunk's blocks in link
+// order; publishes the accepted links of each group (the producers write the
+// angles).  Runs in one of the team's warps.
+__device__ __noinline__ void consume_class(LatState &st, const HbTeam &hb, int B)
+{
+    const int lane = threadIdx.x & 31, nwp = hb.nw - 1, D = hb.D, NT = hb.nw * 32;
+    const int half = st.half, CH = nwp * 64, nchunk = (half + CH - 1) / CH;
+    long long E = st.E_fx;
+    const long long lo = st.lo_fx, hi = st.hi_fx;
     for (int ch = 0; ch < nchunk; ++ch) {
         const int s = ch & (D - 1);
-        bar_sync(1 + s, NT);
-        Stage<NWP> &stg = sm.stage[s];
-        for (int g = 0; g < NWP; ++g) {
-            const unsigned acc =
-                window_scan_group(stg.P[g * 32 + lane], stg.endmask[g], B, E, lo, hi);
-            if (lane == 0) stg.accmask[g] = acc;
+        bar_sync(hb.full + s, NT);
+        const Stage stg = stage_at((char *)(g_dyn + hb.ring), nwp, s);
+        const int left = half - ch * CH;   // links of the class from this chunk on
+        if (B == 1) {
+            // 32 links at a time, the two halves of a group after another
+            const int groups = min(nwp, (left + 63) >> 6);
+            const long long *Pp = stg.P + 31 - lane, *dp = stg.d + 31 - lane;
+            long long P0 = Pp[0], P1 = Pp[32], d0 = dp[0], d1 = dp[32], sum = stg.P[63];
+            for (int g = 0; g < groups; ++g) {
+                // the next group's, on their way during the scan
+                const int nx = min(g + 1, groups - 1) * 64;
+                const long long nP0 = Pp[nx], nP1 = Pp[nx + 32], nd0 = dp[nx], nd1 = dp[nx + 32],
+                                nsum = stg.P[nx + 63];
+                unsigned r0, r1;
+                if (E >= lo && E <= hi) {
+                    long long u = E - lo;
+                    r0 = window_scan_inside(P0, d0, u, (unsigned long long)(hi - lo));
+                    r1 = window_scan_inside(P1, d1, u, (unsigned long long)(hi - lo));
+                    E = lo + u;
+                } else {
+                    const int n0 = min(32, left - g * 64), n1 = min(32, left - g * 64 - 32);
+                    r0 = window_scan_links(P0, d0, kFull << (32 - n0), E, lo, hi);
+                    r1 = n1 > 0 ? window_scan_links(P1, d1, kFull << (32 - n1), E, lo, hi) : 0u;
+                }
+                E += sum;
+                if (lane == 0) stg.acc[g] = make_uint2(__brev(~r0), __brev(~r1));
+                P0 = nP0, P1 = nP1, d0 = nd0, d1 = nd1, sum = nsum;
+            }
+        } else {
+            for (int g = 0; g < nwp; ++g) {
+                const int nl = min(64, left - g * 64) >> 1;   // lanes, two links each
+                if (nl <= 0) break;
+                // blocks of B links end at second links: blocks of B / 2 lanes
+                const int Bl = B >> 1;
+                const bool isend = lane < nl && ((lane & (Bl - 1)) == Bl - 1 || lane == nl - 1);
+                const unsigned em = __ballot_sync(kFull, isend);
+                const unsigned ends =
+                    window_scan_group(stg.P[g * 64 + 2 * lane + 1], em, Bl, E, lo, hi);
+                const int end = min(lane | (Bl - 1), nl - 1);   // of this lane's block
+                const unsigned took = __ballot_sync(kFull, lane < nl && ((ends >> end) & 1u));
+                const unsigned x = __ballot_sync(kFull, (took >> (lane >> 1)) & 1u);
+                const unsigned y = __ballot_sync(kFull, (took >> (16 + (lane >> 1))) & 1u);
+                if (lane == 0) stg.acc[g] = make_uint2(x, y);
+            }
         }
-        bar_arrive(5 + s, NT);
+        bar_arrive(hb.full + D + s, NT);
     }
-    if (lane == 0) sm.st.E_fx = E;
+    if (lane == 0) st.E_fx = E;
 }
 
 // ln rho~ of the multicanonical weight at the fixed-point energy E: the
@@ -667,38 +976,40 @@ __device__ __forceinline__ double muca_lnrho(const KernelArgs &a, long long E_fx
 }
 
 // Consumer side of a multicanonical heat-bath class (Sec. 2.6): the links
-// of each 32-link group are taken in link order by Metropolis-Hastings for
-// the weight 1/rho~ with the proposal at slope a0, i.e. with probability
+// are taken in link order by Metropolis-Hastings for the weight 1/rho~ with
+// the proposal at slope a0, i.e. with probability
 // min(1, exp(a0 dE - (ln rho~(E + dE) - ln rho~(E)))), E the running energy
 // before the link; the uniform comes from Philox counter (link, sweep, 12, 0).
-// Speculatively every remaining link is decided as if all earlier ones were
-// taken; the first refusal (one ballot) fixes the links before it, its dE is
-// dropped and the rest is decided again.  Blocks of one link.
-template <int NWP>
-__device__ __noinline__ void consume_class_muca(Smem<NWP> &sm, int nchunk, int mu, int p,
-                                                const KernelArgs &args, int D)
+// 32 links at a time (half a 64-link group): speculatively every remaining
+// link is decided as if all earlier ones were taken; the first refusal (one
+// ballot) fixes the links before it, its dE is dropped and the rest is decided
+// again.  Blocks of one link.
+__device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb, int mu, int p,
+                                                const KernelArgs &args)
 {
-    constexpr int NT = (NWP + 1) * 32, CH = NWP * 32;
-    const int lane = threadIdx.x & 31;
-    const int L = sm.st.L, half = sm.st.half;
-    const uint32_t magic = sm.st.magic, V = 2u * (uint32_t)half;
-    const uint32_t k0 = sm.st.key0, k1 = sm.st.key1, sweep = sm.st.sweep;
+    const int lane = threadIdx.x & 31, nwp = hb.nw - 1, CH = nwp * 64, D = hb.D, NT = hb.nw * 32;
+    const int L = st.L, half = st.half, nchunk = (half + CH - 1) / CH;
+    const uint32_t magic = st.magic, V = 2u * (uint32_t)half;
+    const uint32_t k0 = st.key0, k1 = st.key1, sweep = st.sweep;
     const double a0 = args.muca_a0;
-    long long E = sm.st.E_fx;
+    long long E = st.E_fx;
     for (int ch = 0; ch < nchunk; ++ch) {
         const int s = ch & (D - 1);
-        bar_sync(1 + s, NT);
-        Stage<NWP> &stg = sm.stage[s];
-        for (int g = 0; g < NWP; ++g) {
-            const unsigned em = stg.endmask[g];
+        bar_sync(hb.full + s, NT);
+        const Stage stg = stage_at((char *)(g_dyn + hb.ring), nwp, s);
+        for (int g = 0; g < 2 * nwp; ++g) {
+            const int h = ch * CH + g * 32 + lane, nval = min(32, half - (ch * CH + g * 32));
+            if (nval <= 0) break;
+            const long long *Pg = stg.P + g * 32;
+            // the prefix sums run over 64 links: take the first half's out of the second's
+            const long long off = (g & 1) ? Pg[-1] : 0ll;
+            const long long Pk = Pg[lane] - off, dk = stg.d[g * 32 + lane];
+            const unsigned em = nval >= 32 ? kFull : (1u << nval) - 1u;
             unsigned rem = em, acc = 0u;
-            const long long Pk = stg.P[g * 32 + lane];
-            const long long Pprev = __shfl_up_sync(kFull, Pk, 1);
-            const long long dk = lane > 0 ? Pk - Pprev : Pk;
             double u = 1.0;
             if ((em >> lane) & 1u) {
                 int x[4];
-                const int site = decode_half(ch * CH + g * 32 + lane, p, L, magic, x);
+                const int site = decode_half(h, p, L, magic, x);
                 const U4 w = philox4x32_10((uint32_t)mu * V + (uint32_t)site, sweep, kTagMuca, 0u,
                                            k0, k1);
                 u = (double)u01(w.x);
@@ -723,42 +1034,390 @@ __device__ __noinline__ void consume_class_muca(Smem<NWP> &sm, int nchunk, int m
                 R += __shfl_sync(kFull, dk, j);
                 rem &= ~((2u << j) - 1u);
             }
-            if (em != 0u) E += __shfl_sync(kFull, Pk, 31 - __clz(em)) - R;
-            if (lane == 0) stg.accmask[g] = acc;
+            E += __shfl_sync(kFull, Pk, nval - 1) - R;
+            if (lane == 0) ((unsigned *)(stg.acc + (g >> 1)))[g & 1] = acc;
         }
-        bar_arrive(5 + s, NT);
+        bar_arrive(hb.full + D + s, NT);
     }
-    if (lane == 0) sm.st.E_fx = E;
+    if (lane == 0) st.E_fx = E;
 }
 
-// One pass over the selected classes (mu = 0..3, parity 0,1).  Heat-bath:
-// class by class over the whole lattice.  Overrelaxation: slab by slab of the
-// last coordinate (x3 = t, the h range [t S, (t+1) S) of every class array,
-// S = L^3 / 2) and the classes within each slab, each group under the window
-// rule of the running energy (windowed false: no window, every reflection
-// is taken -- the multicanonical run).
-template <int NWP, bool FAST>
-__device__ void run_pass(Smem<NWP> &sm, float *th, int kind, float a_f, uint32_t tag, int B,
-                         int class_mask, const KernelArgs *muca = nullptr, bool windowed = true)
+// ---------------------------------------------------------------------------
+// Overrelaxation pass with the current slab in shared memory.
+//
+// The pass goes slab by slab of x3, in each slab class by class, so every class
+// reads the same 8 class arrays of the slab (4 L^3 angles) again: they are
+// copied to shared memory once per slab (16 L^3 bytes, 128 KB at L = 20) and
+// the classes read 13 to 14 of a link's 18 neighbours there; the others lie in
+// the slabs before and after and are plain loads (neither slab changes during
+// this one).  New angles go to shared memory and to global memory.
+//
+// A thread reflects two links at a time, so the index arithmetic and (with
+// rows of even length, ROW) the loads serve two: links k, k + 1 of one x0 row
+// (one 8-byte load each), or, where the half row L / 2 is odd, the links at x2
+// and x2 + L / 2.  Threads map to (x2 plane, x1, k) and step over planes, so
+// only x2 changes from one unit of a thread to the next.
+// ---------------------------------------------------------------------------
+constexpr int kSlabMaxL = 24;       // 16 * 24^3 bytes = 216 KB
+constexpr int kResidentMaxL = 10;   // 16 * 10^4 bytes = 156 KB
+
+struct SlabGeo {
+    int L, Lh, S1, S, half, SH;   // side, half row, plane, slab, class array, half slab (floats)
+    int F, nit, planes;           // planes per iteration, iterations, planes in all
+    int x2, h;                    // the thread's first plane (beyond all: idle) and link
+    int d1p, d1m, rdn, rup, par;  // x1 neighbours, x0 wraps, parity of x1
+};
+
+template <bool ROW>
+__device__ __forceinline__ SlabGeo slab_geo(int L, int nt, int tid)
 {
-    constexpr int NT = (NWP + 1) * 32, CH = NWP * 32;
-    if (threadIdx.x == 0) sm.acc_cnt = 0ull;
-    __syncthreads();
-    const int half = sm.st.half, L = sm.st.L;
-    const int D = sm.ring;   // stages of the producer/consumer ring in use: 1, 2 or 4
-    if (kind == 1) {
-        // Overrelaxation: slab by slab (x3), all classes within a slab, so the
-        // neighbours a slab's staples read are still in L2 from the class before.
-        const int S = half / L;
-        const long long lo = windowed ? sm.st.lo_fx : -(1ll << 62);
-        const long long hi = windowed ? sm.st.hi_fx : (1ll << 62);
-        // a block's |dE| is below B 2^-14, so no block can be refused unless E
-        // is inside the window and within that of an edge
-        const long long bound = (long long)B * kOrDeltaMaxFx;
-        const long long E = sm.st.E_fx;   // the running energy; overrelaxation leaves it
-        const bool free_all = E < lo || E > hi || (E - bound >= lo && E + bound <= hi);
-        int taken = 0;              // moves taken by this thread in near-edge groups
-        unsigned long long n_free = 0;
+    SlabGeo g;
+    g.L = L;
+    g.Lh = L >> 1;
+    g.S1 = L * g.Lh;
+    g.S = g.S1 * L;
+    g.half = g.S * L;
+    g.SH = g.S >> 1;
+    g.planes = ROW ? L : g.Lh;
+    const int pr = ROW ? L >> 2 : g.Lh, pp = pr * L;   // pairs per row, per plane
+    int f = nt / pp;
+    f = f > g.planes ? g.planes : (f < 1 ? 1 : f);
+    g.nit = (g.planes + f - 1) / f;
+    g.F = (g.planes + g.nit - 1) / g.nit;              // the same number of iterations, evenly
+    const int pl = tid / pp, r = tid - pl * pp, x1 = r / pr, k = (r - x1 * pr) * (ROW ? 2 : 1);
+    g.x2 = pl < g.F ? pl : 1 << 20;
+    g.h = pl * g.S1 + x1 * g.Lh + k;
+    g.d1p = x1 == L - 1 ? -(L - 1) * g.Lh : g.Lh;
+    g.d1m = x1 == 0 ? (L - 1) * g.Lh : -g.Lh;
+    g.rdn = k == 0 ? g.Lh - 1 : -1;
+    g.rup = ROW ? (k + 2 == g.Lh ? 2 - g.Lh : 2) : (k == g.Lh - 1 ? 1 - g.Lh : 1);
+    g.par = x1 & 1;
+    return g;
+}
+
+// x0 neighbours of a unit.  A link at x0 = 2 k + b has its neighbour x0 + 1 at
+// half row position k + b and x0 - 1 at k + b - 1.  ROW: r0, r1, r2 are the
+// positions -1 + b, b, 1 + b relative to the first link (wrapped), so x0 + 1 of
+// the pair is (r1, r2), x0 - 1 is (r0, r1).  Otherwise r0, r1 (first link) and
+// r2, r3 (second, of the other parity) are x0 + 1 and x0 - 1.
+template <bool ROW>
+struct X0Off {
+    int r0, r1, r2, r3;
+    __device__ __forceinline__ X0Off(const SlabGeo &g, int x2, int pt)
+    {
+        const int b = (pt + g.par + x2) & 1;
+        if (ROW) {
+            r0 = b ? 0 : g.rdn;
+            r1 = b;
+            r2 = b ? g.rup : 1;
+            r3 = 0;
+        } else {
+            r0 = b ? g.rup : 0;
+            r1 = b ? 0 : g.rdn;
+            r2 = b ? 0 : g.rup;
+            r3 = b ? g.rdn : 0;
+        }
+    }
+};
+
+// The pair of angles at offsets oA (first link) and oB (second; ROW: oA + 1),
+// and of its x0 neighbours.
+template <bool ROW>
+__device__ __forceinline__ float2 pair_at(const float *a, int oA, int oB)
+{
+    if (ROW) return *(const float2 *)(a + oA);
+    return make_float2(a[oA], a[oB]);
+}
+template <bool ROW>
+__device__ __forceinline__ float2 pair_up0(const float *a, const X0Off<ROW> &x, int oA, int oB)
+{
+    if (ROW) return make_float2(a[oA + x.r1], a[oA + x.r2]);
+    return make_float2(a[oA + x.r0], a[oB + x.r2]);
+}
+template <bool ROW>
+__device__ __forceinline__ float2 pair_dn0(const float *a, const X0Off<ROW> &x, int oA, int oB)
+{
+    if (ROW) return make_float2(a[oA + x.r0], a[oA + x.r1]);
+    return make_float2(a[oA + x.r1], a[oB + x.r3]);
+}
+
+// Reflect the pair of links theta_MU of parity p at plane x2, offset h of the
+// slab; sl: the slab's class arrays in shared memory (stride S); th: the
+// lattice, tc / tp / tm its offsets of this slab, the next and the one before.
+template <int MU, bool ROW, bool FAST>
+__device__ __forceinline__ void reflect_pair(const SlabGeo &g, int x2, int h, int p, int t,
+                                             float *sl, float *th, int tc, int tp, int tm)
+{
+    const int q = p ^ 1, S = g.S, SH = g.SH, half = g.half, wr = S - g.S1;
+    const int d1p = g.d1p, d1m = g.d1m;
+    // x2 neighbours of the first link; of the second, relative to h
+    const int d2p = (ROW && x2 == g.L - 1) ? -wr : g.S1, d2m = x2 == 0 ? wr : -g.S1;
+    const int e2p = SH + (x2 == g.Lh - 1 ? -wr : g.S1), e2m = SH - g.S1;
+    const X0Off<ROW> x(g, x2, p + t);
+    auto at = [&](int nu, int par, int dA, int dB) {
+        return pair_at<ROW>(sl, h + (2 * nu + par) * S + dA, h + (2 * nu + par) * S + dB);
+    };
+    auto up0 = [&](int nu, int par, int dA, int dB) {
+        return pair_up0<ROW>(sl, x, h + (2 * nu + par) * S + dA, h + (2 * nu + par) * S + dB);
+    };
+    auto dn0 = [&](int nu, int par, int dA, int dB) {
+        return pair_dn0<ROW>(sl, x, h + (2 * nu + par) * S + dA, h + (2 * nu + par) * S + dB);
+    };
+    // the same in another slab (global memory, at offset ts)
+    auto gat = [&](int ts, int nu, int par, int dA, int dB) {
+        return pair_at<ROW>(th, h + (2 * nu + par) * half + ts + dA,
+                            h + (2 * nu + par) * half + ts + dB);
+    };
+    float2 g0, g1, g2, g3, g4, g5;
+    if (MU < 3) {
+        g0 = gat(tp, MU, q, 0, SH);      // theta_mu(x+3)
+        g1 = gat(tm, MU, q, 0, SH);      // theta_mu(x-3)
+        g2 = gat(tm, 3, q, 0, SH);       // theta_3(x-3)
+        const int o = h + (6 + p) * half + tm;   // theta_3(x-3+mu)
+        g3 = MU == 0   ? pair_up0<ROW>(th, x, o, o + SH)
+             : MU == 1 ? pair_at<ROW>(th, o + d1p, o + SH + d1p)
+                       : pair_at<ROW>(th, o + d2p, o + e2p);
+        g4 = g5 = g3;
+    } else {
+        g0 = gat(tp, 0, q, 0, SH);       // theta_nu(x+3), theta_nu(x-nu+3) for nu = 0, 1, 2
+        const int o = h + p * half + tp;
+        g1 = pair_dn0<ROW>(th, x, o, o + SH);
+        g2 = gat(tp, 1, q, 0, SH);
+        g3 = gat(tp, 1, p, d1m, SH + d1m);
+        g4 = gat(tp, 2, q, 0, SH);
+        g5 = gat(tp, 2, p, d2m, e2m);
+    }
+    float2 Sr = make_float2(0.0f, 0.0f), Si = Sr;
+    const float2 t0 = at(MU, p, 0, SH);
+#pragma unroll
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == MU) continue;
+        // a1 = theta_nu(x+mu), a2 = theta_mu(x+nu), a3 = theta_nu(x),
+        // b1 = theta_nu(x-nu+mu), b2 = theta_mu(x-nu), b3 = theta_nu(x-nu)
+        float2 a1, a2, a3, b1, b2, b3;
+        a3 = at(nu, p, 0, SH);
+        if (MU == 0) a1 = up0(nu, q, 0, SH);
+        else if (MU == 1) a1 = at(nu, q, d1p, d1p + SH);
+        else if (MU == 2) a1 = at(nu, q, d2p, e2p);
+        else a1 = nu == 0 ? g0 : nu == 1 ? g2 : g4;
+        if (nu == 0) {
+            a2 = up0(MU, q, 0, SH);
+            b2 = dn0(MU, q, 0, SH);
+            b3 = dn0(0, q, 0, SH);
+            if (MU == 1) b1 = dn0(0, p, d1p, d1p + SH);
+            else if (MU == 2) b1 = dn0(0, p, d2p, e2p);
+            else b1 = g1;
+        } else if (nu == 1) {
+            a2 = at(MU, q, d1p, d1p + SH);
+            b2 = at(MU, q, d1m, d1m + SH);
+            b3 = at(1, q, d1m, d1m + SH);
+            if (MU == 0) b1 = up0(1, p, d1m, d1m + SH);
+            else if (MU == 2) b1 = at(1, p, d2p + d1m, e2p + d1m);
+            else b1 = g3;
+        } else if (nu == 2) {
+            a2 = at(MU, q, d2p, e2p);
+            b2 = at(MU, q, d2m, e2m);
+            b3 = at(2, q, d2m, e2m);
+            if (MU == 0) b1 = up0(2, p, d2m, e2m);
+            else if (MU == 1) b1 = at(2, p, d2m + d1p, e2m + d1p);
+            else b1 = g5;
+        } else {
+            a2 = g0;
+            b2 = g1;
+            b3 = g2;
+            b1 = g3;
+        }
+        // the staple sums of both links, formed exactly as in staple_from
+        const float2 pf = sub2(sub2(a1, a2), a3), pb = sub2(sub2(b3, b1), b2);
+        float2 sf, cf, sb, cb;
+        sin_cos<FAST>(pf.x, &sf.x, &cf.x);
+        sin_cos<FAST>(pf.y, &sf.y, &cf.y);
+        sin_cos<FAST>(pb.x, &sb.x, &cb.x);
+        sin_cos<FAST>(pb.y, &sb.y, &cb.y);
+        Sr = add2(Sr, add2(cf, cb));
+        Si = add2(Si, add2(sf, sb));
+    }
+    const float2 al = arg2<FAST>(Si, Sr);
+    float2 tn;
+    tn.x = wrap_angle(-t0.x - 2.0f * al.x);
+    tn.y = wrap_angle(-t0.y - 2.0f * al.y);
+    const int so = h + (2 * MU + p) * S, go = h + (2 * MU + p) * half + tc;
+    if (ROW) {
+        *(float2 *)(sl + so) = tn;
+        *(float2 *)(th + go) = tn;
+    } else {
+        sl[so] = tn.x;
+        sl[so + SH] = tn.y;
+        th[go] = tn.x;
+        th[go + SH] = tn.y;
+    }
+}
+
+// The two classes of direction MU in one slab.
+template <int MU, bool ROW, bool FAST>
+__device__ __forceinline__ void reflect_dir(const SlabGeo &g, const Team &tm_, int t, int mask,
+                                            float *sl, float *th, int tc, int tp, int tm)
+{
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p) {
+        if (!((mask >> (2 * MU + p)) & 1)) continue;
+        int x2 = g.x2, h = g.h;
+#pragma unroll 1
+        for (int i = 0; i < g.nit; ++i) {
+            if (x2 < g.planes) reflect_pair<MU, ROW, FAST>(g, x2, h, p, t, sl, th, tc, tp, tm);
+            x2 += g.F;
+            h += g.F * g.S1;
+        }
+        tm_.sync();   // the next class reads the angles written here
+    }
+}
+
+// The whole pass of the team's lattice: every reflection is taken (see
+// overrelax_pass).  slab_off: the team's slab in g_dyn.  The team shrinks to
+// the warps that hold a link; the others return.
+template <bool ROW, bool FAST>
+__device__ __noinline__ void reflect_slabs(Team team, int L_, float *th_, int slab_off, int mask)
+{
+    const int L = uniform(L_);
+    float *th = (float *)__shfl_sync(kFull, (unsigned long long)th_, 0);
+    float *sl = g_dyn + uniform(slab_off);
+    const SlabGeo g = slab_geo<ROW>(L, team.nt, team.tid);
+    const int need = (g.F * (ROW ? L >> 2 : g.Lh) * L + 31) >> 5;
+    if (team.w >= need) return;
+    team.nw = need < team.nw ? need : team.nw;
+    team.nt = team.nw * 32;
+    const int S = g.S, half = g.half;
+#pragma unroll 1
+    for (int t = 0; t < L; ++t) {
+        const int tc = t * S, tp = (t == L - 1 ? 0 : t + 1) * S, tm = (t == 0 ? L - 1 : t - 1) * S;
+        // S = L^3 / 2 is a multiple of 4 floats for even L, as are all offsets
+#pragma unroll 1
+        for (int a = 0; a < 8; ++a)
+            for (int i = 4 * team.tid; i < S; i += 4 * team.nt)
+                cp_async16(sl + a * S + i, th + tc + a * half + i);
+        cp_async_commit();
+        // the next slab on its way from HBM to L2
+#pragma unroll 1
+        for (int a = 0; a < 8; ++a)
+            for (int i = 32 * team.tid; i < S; i += 32 * team.nt)
+                asm volatile("prefetch.global.L2 [%0];" ::"l"(th + tp + a * half + i));
+        cp_async_wait<0>();
+        team.sync();
+        reflect_dir<0, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<1, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<2, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<3, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Overrelaxation pass of a lattice that is in shared memory as a whole.  A
+// class of a slab has at most as many links as the team has threads, so the
+// pass is a chain of 8 L short steps, and the time is the step's latency: one
+// link per thread, the side a compile-time constant (every class array and wrap
+// an immediate of the load), the thread's place in the slab worked out once.
+// ---------------------------------------------------------------------------
+template <int MU, int L, bool FAST>
+__device__ __forceinline__ void reflect_resident(float *l, int p, int up0, int dn0, int d1p,
+                                                 int d1m, int d2p, int d2m, int d3p, int d3m)
+{
+    // l: the link's half site in class array 0; up / dn: half-site distances to
+    // x + nu, x - nu
+    constexpr int half = L * L * L * L / 2;
+    const int up[4] = {up0, d1p, d2p, d3p}, dn[4] = {dn0, d1m, d2m, d3m};
+    float *lp = l + p * half;               // arrays of parity p at 2 nu half
+    const float *lq = l + (p ^ 1) * half;   // of the other parity
+    const float t0 = lp[2 * MU * half];
+    float v[18];
+    int j = 0;
+#pragma unroll
+    for (int nu = 0; nu < 4; ++nu) {
+        if (nu == MU) continue;
+        v[6 * j + 0] = lq[2 * nu * half + up[MU]];
+        v[6 * j + 1] = lq[2 * MU * half + up[nu]];
+        v[6 * j + 2] = lp[2 * nu * half];
+        v[6 * j + 3] = lp[2 * nu * half + dn[nu] + up[MU]];
+        v[6 * j + 4] = lq[2 * MU * half + dn[nu]];
+        v[6 * j + 5] = lq[2 * nu * half + dn[nu]];
+        ++j;
+    }
+    float Sr, Si;
+    staple_sum_regs<FAST>(v, Sr, Si);
+    lp[2 * MU * half] = wrap_angle(-t0 - 2.0f * arg<FAST>(Si, Sr));
+}
+
+template <int L, bool FAST>
+__device__ __noinline__ void reflect_lattice(Team team, int lat_off, int mask)
+{
+    constexpr int Lh = L / 2, S1 = L * Lh, S = S1 * L, nw = (S + 31) / 32;
+    if (team.w >= nw) return;
+    const int h = team.tid;
+    const bool mine = h < S;
+    const int row = h / Lh, k = h - row * Lh, x2 = row / L, x1 = row - x2 * L;
+    const int d1p = x1 == L - 1 ? Lh - S1 : Lh, d1m = x1 == 0 ? S1 - Lh : -Lh;
+    const int d2p = x2 == L - 1 ? S1 - S : S1, d2m = x2 == 0 ? S - S1 : -S1;
+    const int dn = k == 0 ? Lh - 1 : -1, up = k == Lh - 1 ? 1 - Lh : 1;
+    float *l = g_dyn + lat_off + h;
+#pragma unroll 1
+    for (int t = 0; t < L; ++t, l += S) {
+        const int d3p = t == L - 1 ? S - S * L : S, d3m = t == 0 ? S * L - S : -S;
+        const int c = (x1 + x2 + t) & 1;
+#define LLR_CLASS(MU)                                                                            \
+    _Pragma("unroll 1") for (int p = 0; p < 2; ++p)                                              \
+    {                                                                                            \
+        if (!((mask >> (2 * MU + p)) & 1)) continue;                                             \
+        const bool odd = p ^ c; /* x0 = 2 k + odd */                                             \
+        if (mine)                                                                                \
+            reflect_resident<MU, L, FAST>(l, p, odd ? up : 0, odd ? 0 : dn, d1p, d1m, d2p, d2m,  \
+                                          d3p, d3m);                                             \
+        bar_sync(team.bar, nw * 32); /* the next class reads the angles written here */          \
+    }
+        LLR_CLASS(0)
+        LLR_CLASS(1)
+        LLR_CLASS(2)
+        LLR_CLASS(3)
+#undef LLR_CLASS
+    }
+}
+
+// One overrelaxation pass of a lattice by a team, over the selected classes,
+// slab by slab of the last coordinate (x3 = t, the h range [t S, (t+1) S) of
+// every class array, S = L^3 / 2) and the classes within each slab, under the
+// window rule of the running energy (windowed false: no window, every
+// reflection is taken -- the multicanonical run).
+template <bool FAST>
+__device__ __noinline__ void overrelax_pass(Smem &sm, int slot, const Team &team, float *th,
+                                            int slab_off, bool res, int B, int class_mask,
+                                            bool windowed)
+{
+    const LatState &st = sm.st[slot];
+    const int half = st.half, L = st.L, S = half / L;
+    const long long lo = windowed ? st.lo_fx : -(1ll << 62);
+    const long long hi = windowed ? st.hi_fx : (1ll << 62);
+    // a block's |dE| is below B 2^-14, so no block can be refused unless E is
+    // inside the window and within that of an edge
+    const long long bound = (long long)B * kOrDeltaMaxFx;
+    const long long E = st.E_fx;   // the running energy; overrelaxation leaves it
+    const bool free_all = E < lo || E > hi || (E - bound >= lo && E + bound <= hi);
+    // the pairs of one unit plane (L^2 / 4, or L^2 / 2 for odd half rows) need a thread each
+    const bool in_slabs =
+        free_all && (res || (L <= kSlabMaxL && L * L <= ((L & 3) == 0 ? 4 : 2) * team.nt));
+    if (in_slabs && res) {
+        switch (L) {
+            case 2: reflect_lattice<2, FAST>(team, slab_off, class_mask); break;
+            case 4: reflect_lattice<4, FAST>(team, slab_off, class_mask); break;
+            case 6: reflect_lattice<6, FAST>(team, slab_off, class_mask); break;
+            case 8: reflect_lattice<8, FAST>(team, slab_off, class_mask); break;
+            default: reflect_lattice<10, FAST>(team, slab_off, class_mask); break;
+        }
+    } else if (in_slabs) {
+        if ((L & 3) == 0)
+            reflect_slabs<true, FAST>(team, L, th, slab_off, class_mask);
+        else
+            reflect_slabs<false, FAST>(team, L, th, slab_off, class_mask);
+    }
+    int taken = 0;              // moves taken by this thread in near-edge groups
+    if (!in_slabs) {
 #pragma unroll 1
         for (int t = 0; t < L; ++t) {
 #pragma unroll 1
@@ -767,64 +1426,154 @@ __device__ void run_pass(Smem<NWP> &sm, float *th, int kind, float a_f, uint32_t
                 const int p = cls & 1;
                 if (free_all) {
                     switch (cls >> 1) {
-                        case 0: overrelax_class<0, NWP, FAST>(sm, th, p, t * S, S); break;
-                        case 1: overrelax_class<1, NWP, FAST>(sm, th, p, t * S, S); break;
-                        case 2: overrelax_class<2, NWP, FAST>(sm, th, p, t * S, S); break;
-                        default: overrelax_class<3, NWP, FAST>(sm, th, p, t * S, S); break;
+                        case 0: overrelax_class<0, FAST>(st, team, th, p, t * S, S); break;
+                        case 1: overrelax_class<1, FAST>(st, team, th, p, t * S, S); break;
+                        case 2: overrelax_class<2, FAST>(st, team, th, p, t * S, S); break;
+                        default: overrelax_class<3, FAST>(st, team, th, p, t * S, S); break;
                     }
-                    n_free += (unsigned long long)S;
                 } else {
                     switch (cls >> 1) {
-                        case 0: taken += overrelax_class_near<0, NWP, FAST>(sm, th, p, t * S, S, B, E); break;
-                        case 1: taken += overrelax_class_near<1, NWP, FAST>(sm, th, p, t * S, S, B, E); break;
-                        case 2: taken += overrelax_class_near<2, NWP, FAST>(sm, th, p, t * S, S, B, E); break;
-                        default: taken += overrelax_class_near<3, NWP, FAST>(sm, th, p, t * S, S, B, E); break;
+                        case 0: taken += overrelax_class_near<0, FAST>(st, team, th, p, t * S, S, B, E); break;
+                        case 1: taken += overrelax_class_near<1, FAST>(st, team, th, p, t * S, S, B, E); break;
+                        case 2: taken += overrelax_class_near<2, FAST>(st, team, th, p, t * S, S, B, E); break;
+                        default: taken += overrelax_class_near<3, FAST>(st, team, th, p, t * S, S, B, E); break;
                     }
                 }
-                __syncthreads();   // the next group reads the angles written here
+                team.sync();   // the next group reads the angles written here
             }
         }
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) taken += __shfl_down_sync(kFull, taken, o);
-        if ((threadIdx.x & 31) == 0 && taken) atomicAdd(&sm.acc_cnt, (unsigned long long)taken);
-        if (threadIdx.x == 0 && n_free) atomicAdd(&sm.acc_cnt, n_free);
-        (void)NT;
+        if ((threadIdx.x & 31) == 0 && taken)
+            atomicAdd(&sm.acc_cnt[slot], (unsigned long long)taken);
+    }
+    if (team.tid == 0 && free_all)
+        atomicAdd(&sm.acc_cnt[slot], (unsigned long long)__popc(class_mask & 0xFF) *
+                                         (unsigned long long)half);
+}
+
+// What the phases of a sweep need of the launch.
+struct Phase {
+    int teams, tw;        // lattices a CTA works on, warps per lattice
+    int nl;               // lattices of this item (<= teams)
+    int or_teams;         // lattices in overrelaxation at a time (their slabs in shared memory)
+    int slab;             // floats of shared memory per slab (res: per lattice)
+    bool res;             // the item's lattices are in shared memory as a whole
+    int ring;             // offset of the heat-bath rings in g_dyn (floats)
+    int D;                // ring stages
+
+    // the links of lattice `slot` of the item
+    __device__ __forceinline__ float *links(const Smem &sm, const KernelArgs &args, int slot) const
+    {
+        return res ? g_dyn + slot * slab : args.theta + sm.st[slot].off;
+    }
+};
+
+// One class of a heat-bath pass by the team's producers.
+template <int MU, bool FAST>
+__device__ __forceinline__ void produce(Smem &sm, const Phase &ph, int slot, int pw, float *th,
+                                        int p, uint32_t tag)
+{
+    const bool row = (sm.st[slot].L & 3) == 0;
+    const int off = slot * ph.slab;
+    if (ph.res) {
+        if (row)
+            produce_class<MU, true, true, FAST>(sm, slot, pw, th, off, p, tag);
+        else
+            produce_class<MU, false, true, FAST>(sm, slot, pw, th, off, p, tag);
     } else {
-        // Heat-bath: one class at a time over the whole lattice, so the
-        // producer/consumer pipeline drains once per class.
-        const int nchunk = (half + CH - 1) / CH;
-        const bool consumer = (threadIdx.x >> 5) == sm.cw;
+        if (row)
+            produce_class<MU, true, false, FAST>(sm, slot, pw, th, off, p, tag);
+        else
+            produce_class<MU, false, false, FAST>(sm, slot, pw, th, off, p, tag);
+    }
+}
+
+// Heat-bath pass of every active lattice of the item, each by its team, one
+// class at a time over the whole lattice, so the producer/consumer pipeline
+// drains once per class.  kind 0: window rule, 2: multicanonical.
+template <bool FAST>
+__device__ __noinline__ void heatbath_phase(Smem &sm, const Phase &ph, const KernelArgs &args,
+                                            int kind, uint32_t tag, int B, int class_mask)
+{
+    if (threadIdx.x < ph.nl) {
+        const int k = threadIdx.x;
+        sm.acc_cnt[k] = 0ull;
+        HbTeam &hb = sm.hb[k];
+        hb.nw = min(ph.tw, 1 + (sm.st[k].half + 63) / 64);   // no more producers than groups
+        // the consumers of different teams on different quarters of the SM
+        hb.cw = hb.nw - 1;
+        for (int c = hb.nw - 1; c >= max(0, hb.nw - 4); --c)
+            if (((k * ph.tw + c) & 3) == 3 - (k & 3)) hb.cw = c;
+        hb.D = ph.D;
+        hb.ring = ph.ring + k * ph.D * (ph.tw - 1) * (kStageGroupBytes / 4);
+        hb.full = 1 + 2 * ph.D * k;
+    }
+    __syncthreads();
+    const int warp = threadIdx.x >> 5, slot = warp / ph.tw, w = warp - slot * ph.tw;
+    if (slot < ph.nl && sm.active[slot]) {
+        LatState &st = sm.st[slot];
+        const int nw = sm.hb[slot].nw, cw = sm.hb[slot].cw;
+        if (w < nw) {
+            float *th = args.theta + st.off;
+            const bool consumer = w == cw;
+            const int pw = w - (w > cw ? 1 : 0);   // rank among the producers
 #pragma unroll 1
-        for (int cls = 0; cls < 8; ++cls) {
-            if (!((class_mask >> cls) & 1)) continue;
-            const int mu = cls >> 1, p = cls & 1;
-            if (consumer) {
-                if (kind == 2)
-                    consume_class_muca<NWP>(sm, nchunk, mu, p, *muca, D);
-                else
-                    consume_class<NWP>(sm, B, nchunk, D);
-            } else {
-                switch (mu) {
-                    case 0: produce_class<0, NWP, FAST>(sm, th, p, a_f, tag, B, 0, half, nchunk, D); break;
-                    case 1: produce_class<1, NWP, FAST>(sm, th, p, a_f, tag, B, 0, half, nchunk, D); break;
-                    case 2: produce_class<2, NWP, FAST>(sm, th, p, a_f, tag, B, 0, half, nchunk, D); break;
-                    default: produce_class<3, NWP, FAST>(sm, th, p, a_f, tag, B, 0, half, nchunk, D); break;
+            for (int cls = 0; cls < 8; ++cls) {
+                if (!((class_mask >> cls) & 1)) continue;
+                const int mu = cls >> 1, p = cls & 1;
+                if (consumer) {
+                    if (kind == 2)
+                        consume_class_muca(st, sm.hb[slot], mu, p, args);
+                    else
+                        consume_class(st, sm.hb[slot], B);
+                } else {
+                    switch (mu) {
+                        case 0: produce<0, FAST>(sm, ph, slot, pw, th, p, tag); break;
+                        case 1: produce<1, FAST>(sm, ph, slot, pw, th, p, tag); break;
+                        case 2: produce<2, FAST>(sm, ph, slot, pw, th, p, tag); break;
+                        default: produce<3, FAST>(sm, ph, slot, pw, th, p, tag); break;
+                    }
                 }
+                // the next class reads the angles written here
+                bar_sync(sm.hb[slot].full, nw * 32);
             }
-            __syncthreads();   // the next class reads the angles written here
         }
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        const unsigned long long n =
-            (unsigned long long)__popc(class_mask & 0xFF) * (unsigned long long)half;
-        if (kind != 1) {
-            sm.st.hb_acc += sm.acc_cnt;
-            sm.st.hb_tot += n;
-        } else {
-            sm.st.or_acc += sm.acc_cnt;
-            sm.st.or_tot += n;
+    if (threadIdx.x < ph.nl && sm.active[threadIdx.x]) {
+        LatState &st = sm.st[threadIdx.x];
+        st.hb_acc += sm.acc_cnt[threadIdx.x];
+        st.hb_tot += (unsigned long long)__popc(class_mask & 0xFF) * (unsigned long long)st.half;
+    }
+    __syncthreads();
+}
+
+// Overrelaxation pass of every active lattice of the item, or_teams of them at a
+// time, each by its share of the warps.
+template <bool FAST>
+__device__ __noinline__ void overrelax_phase(Smem &sm, const Phase &ph, const KernelArgs &args,
+                                             int B, int class_mask, bool windowed)
+{
+    if (threadIdx.x < kMaxTeams) sm.acc_cnt[threadIdx.x] = 0ull;
+    __syncthreads();
+    const int tw = kWarps / ph.or_teams, warp = threadIdx.x >> 5, k = warp / tw;
+    if (k < ph.or_teams) {
+        const Team t{warp - k * tw, tw, (int)threadIdx.x - k * tw * 32, tw * 32, 1 + k};
+        for (int slot = k; slot < ph.nl; slot += ph.or_teams) {
+            if (!sm.active[slot]) continue;
+            overrelax_pass<FAST>(sm, slot, t, ph.links(sm, args, slot),
+                                 (ph.res ? slot : k) * ph.slab, ph.res, B, class_mask, windowed);
+            // a pass may end with some of the team's warps only, and the next
+            // lattice's slab takes this one's place
+            bar_sync(8 + k, t.nt);
         }
+    }
+    __syncthreads();
+    if (threadIdx.x < ph.nl && sm.active[threadIdx.x]) {
+        LatState &st = sm.st[threadIdx.x];
+        st.or_acc += sm.acc_cnt[threadIdx.x];
+        st.or_tot += (unsigned long long)__popc(class_mask & 0xFF) * (unsigned long long)st.half;
     }
     __syncthreads();
 }
@@ -905,19 +1654,18 @@ __device__ __forceinline__ float plaquette_cos(float a, float b, float c, float 
     return cos_unbiased(hi, lo);
 }
 
-// Fresh energy of the CTA's lattice in fixed point: sum over the 6 V
-// plaquettes, exact int64 accumulation and reduction.  Valid in thread 0.
-template <int NWP>
-__device__ __noinline__ long long fresh_energy_fx(Smem<NWP> &sm, const float *th)
+// Fresh energy of the team's lattice in fixed point: sum over the 6 V
+// plaquettes, exact int64 accumulation and reduction.  Valid in the team's thread 0.
+__device__ __noinline__ long long fresh_energy_fx(const LatState &st_, const Team &team,
+                                                  long long *red, const float *th)
 {
-    constexpr int NT = (NWP + 1) * 32;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int L = sm.st.L, half = sm.st.half;
-    const uint32_t magic = sm.st.magic;
+    const int tid = team.tid, lane = tid & 31;
+    const int L = uniform(st_.L), half = uniform(st_.half);
+    const uint32_t magic = uniform(st_.magic);
     const int V = 2 * half;
     const int st[4] = {1, L, L * L, L * L * L};
     long long acc = 0;
-    for (int s = tid; s < V; s += NT) {
+    for (int s = tid; s < V; s += team.nt) {
         int x[4];
         const int q = (int)__umulhi((uint32_t)s, magic);
         x[0] = s - q * L;
@@ -946,43 +1694,53 @@ __device__ __noinline__ long long fresh_energy_fx(Smem<NWP> &sm, const float *th
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
-    if (lane == 0) sm.red[warp] = acc;
-    __syncthreads();
+    if (lane == 0) red[team.w] = acc;
+    team.sync();
     long long tot = 0;
     if (tid == 0)
-        for (int w = 0; w < NWP + 1; ++w) tot += sm.red[w];
-    __syncthreads();
+        for (int w = 0; w < team.nw; ++w) tot += red[w];
     return tot;
 }
 
-// Resync after a composite sweep; thread 0 updates the state.
-template <int NWP>
-__device__ void end_of_sweep(Smem<NWP> &sm, const float *th, bool measure)
+// Fresh energies of the active lattices of the item, each by its team, into
+// the tracked energy.  resync: at the end of a composite sweep, which records
+// the drift, counts the sweep and measures.
+__device__ __noinline__ void energy_phase(Smem &sm, const Phase &ph, const KernelArgs &args,
+                                          bool resync, bool measure)
 {
-    const long long fresh = fresh_energy_fx<NWP>(sm, th);
-    if (threadIdx.x == 0) {
-        const double drift = fabs((double)(sm.st.E_fx - fresh) * kInvFx);
-        if (drift > sm.st.max_drift) sm.st.max_drift = drift;
-        sm.st.E_fx = fresh;
-        sm.st.sweep += 1u;
-        sm.st.sweeps_done += 1ull;
-        if (measure) {
-            const double dEm = (double)fresh * kInvFx - (sm.st.E_lo + 0.5 * sm.st.dE);
-            sm.st.sum_dE += dEm;
-            sm.st.sum_dE2 += dEm * dEm;
-            sm.st.n_meas += 1;
+    const int warp = threadIdx.x >> 5, slot = warp / ph.tw;
+    if (slot < ph.nl && sm.active[slot]) {
+        const Team t{warp - slot * ph.tw, ph.tw, (int)threadIdx.x - slot * ph.tw * 32, ph.tw * 32,
+                     1 + slot};
+        LatState &st = sm.st[slot];
+        const long long fresh = fresh_energy_fx(st, t, sm.red + slot * ph.tw, ph.links(sm, args, slot));
+        if (t.tid == 0) {
+            if (resync) {
+                const double drift = fabs((double)(st.E_fx - fresh) * kInvFx);
+                if (drift > st.max_drift) st.max_drift = drift;
+                st.sweep += 1u;
+                st.sweeps_done += 1ull;
+                if (measure) {
+                    const double dEm = (double)fresh * kInvFx - (st.E_lo + 0.5 * st.dE);
+                    st.sum_dE += dEm;
+                    st.sum_dE2 += dEm * dEm;
+                    st.n_meas += 1;
+                }
+            }
+            st.E_fx = fresh;
         }
     }
     __syncthreads();
 }
 
-template <int NWP, bool FAST>
-__device__ void composite_sweep(Smem<NWP> &sm, float *th, float a_f, uint32_t tag, int n_or,
-                                int B, bool measure)
+template <bool FAST>
+__device__ void composite_sweep(Smem &sm, const Phase &ph, const KernelArgs &args, uint32_t tag,
+                                bool measure)
 {
-    run_pass<NWP, FAST>(sm, th, 0, a_f, tag, B, 0xFF);
-    for (int k = 0; k < n_or; ++k) run_pass<NWP, FAST>(sm, th, 1, a_f, tag, B, 0xFF);
-    end_of_sweep<NWP>(sm, th, measure);
+    heatbath_phase<FAST>(sm, ph, args, 0, tag, args.block, 0xFF);
+    for (int k = 0; k < args.n_or; ++k)
+        overrelax_phase<FAST>(sm, ph, args, args.block, 0xFF, true);
+    energy_phase(sm, ph, args, true, measure);
 }
 
 __device__ __forceinline__ unsigned long long global_ns()
@@ -1018,48 +1776,66 @@ __device__ __noinline__ void rm_update(LatState &st, const KernelArgs &args, int
     if (args.hist) args.hist[(size_t)step * (size_t)args.n_lat + (size_t)lat] = a_new;
 }
 
-// Resident CTAs per SM the register budget is held to: 512 threads x 2 (64
-// registers); 128 threads x 6, 160 threads x 5, 192 threads x 4 and 256
-// threads x 3 (80 registers).
-template <int NWP>
-constexpr int min_ctas()
+// The item's lattices into shared memory (in) and back to global memory.
+__device__ __noinline__ void copy_lattices(const Smem &sm, const Phase &ph, const KernelArgs &args,
+                                           bool in)
 {
-    return NWP == 3 ? 6 : NWP == 4 ? 5 : NWP == 5 ? 4 : NWP == 7 ? 3 : 2;
+    for (int slot = 0; slot < ph.nl; ++slot) {
+        float *g = args.theta + sm.st[slot].off, *l = g_dyn + slot * ph.slab;
+        const int n = 8 * sm.st[slot].half;   // a multiple of 4, lattices 128-byte aligned
+        for (int i = 4 * threadIdx.x; i < n; i += 4 * kThreads) {
+            if (in)
+                cp_async16(l + i, g + i);
+            else
+                *(float4 *)(g + i) = *(const float4 *)(l + i);
+        }
+    }
+    if (in) {
+        cp_async_commit();
+        cp_async_wait<0>();
+    }
+    __syncthreads();
 }
 
-template <int NWP, bool FAST>
-__global__ void __launch_bounds__((NWP + 1) * 32, min_ctas<NWP>()) llr_kernel(KernelArgs args)
+// One CTA per SM.  Work items are (composite sweep j, group of up to `teams`
+// lattices); the lattices of a group advance together, phase by phase.
+template <bool FAST>
+__global__ void __launch_bounds__(kThreads, 1) llr_kernel(const __grid_constant__ KernelArgs args)
 {
-    __shared__ Smem<NWP> sm;
+    __shared__ Smem sm;
     const int tid = threadIdx.x;
     const bool multi =
         args.program == kProgSweeps || args.program == kProgRM || args.program == kProgMuca;
     const int per_lat = multi ? args.n_therm + args.n_meas : 1;
-    const unsigned n_items = (unsigned)args.n_lat * (unsigned)per_lat;
+    Phase ph;
+    ph.teams = args.teams;
+    ph.tw = kWarps / args.teams;
+    ph.or_teams = args.or_teams;
+    ph.slab = args.slab;
+    ph.res = args.resident != 0;
+    ph.ring = args.ring_off;
+    ph.D = args.ring;
+    const unsigned n_groups = (unsigned)((args.n_lat + args.teams - 1) / args.teams);
+    const unsigned n_items = n_groups * (unsigned)per_lat;
     unsigned *err = args.sync;
     unsigned *counter = args.sync + 1;
     unsigned *done = args.sync + 2;
-    if (tid == 0) {
-        sm.cw = NWP;   // the consumer warp of a heat-bath pass: the last
-        sm.ring = (args.ring == 1 || args.ring == 2) ? args.ring : kStages;
-    }
-    __syncthreads();
     for (;;) {
         if (tid == 0) {
             const unsigned i = atomicAdd(counter, 1u);
             int state = 0;
             if (i < n_items) {
-                const int j = (int)(i / (unsigned)args.n_lat);
-                const int slot = (int)(i % (unsigned)args.n_lat);
+                const int j = (int)(i / n_groups);
+                const unsigned grp = i % n_groups;
                 state = 1;
                 if (j > 0) {
-                    // sweep j-1 of this lattice was dequeued earlier by a running
+                    // sweep j-1 of this group was dequeued earlier by a running
                     // CTA; wait for it, but never longer than wait_limit_ns.  Once
                     // any wait has run out (the error word is set; it stays set
                     // until the host reads it), an item that would wait skips at
                     // once: the sweep before it may never come.
                     const unsigned long long t0 = global_ns();
-                    while (ld_acquire(done + slot) < (unsigned)j) {
+                    while (ld_acquire(done + grp) < (unsigned)j) {
                         if (ld_acquire(err) != 0u) {
                             state = 2;
                             break;
@@ -1072,117 +1848,129 @@ __global__ void __launch_bounds__((NWP + 1) * 32, min_ctas<NWP>()) llr_kernel(Ke
                         __nanosleep(256);
                     }
                 }
-                sm.item_lat = slot;
+                sm.item_first = (int)grp * args.teams;
+                sm.item_n = min(args.teams, args.n_lat - (int)grp * args.teams);
                 sm.item_j = j;
-                if (state == 1) sm.st = args.lats[args.order ? args.order[slot] : slot];
             }
             sm.item_state = state;
-            sm.cap_cnt = 0ull;
         }
         __syncthreads();
         const int state = sm.item_state;
         if (state == 0) break;
         if (state == 2) {
             __syncthreads();
-            continue;   // timed out: leave this lattice alone, the host reads the error word
+            continue;   // timed out: leave these lattices alone, the host reads the error word
         }
-        const int slot = sm.item_lat, j = sm.item_j;
-        const int lat = args.order ? args.order[slot] : slot;
-        float *th = args.theta + sm.st.off;
+        const int j = sm.item_j;
+        ph.nl = sm.item_n;
+        // thread k < nl looks after lattice k of the item
+        const bool mine = tid < ph.nl;
+        int lat = 0;
+        if (mine) {
+            const int slot = sm.item_first + tid;
+            lat = args.order ? args.order[slot] : slot;
+            sm.st[tid] = args.lats[lat];
+            LatState &st = sm.st[tid];
+            sm.cap_cnt[tid] = 0ull;
+            sm.active[tid] = 1;
+            if (args.program == kProgSweeps || args.program == kProgRM ||
+                args.program == kProgBegin) {
+                if (j == 0) {
+                    if (args.a_in) st.a = args.a_in[lat];
+                    st.sum_dE = 0.0;
+                    st.sum_dE2 = 0.0;
+                    st.n_meas = 0;
+                }
+            } else if (args.program == kProgPass && args.a_in) {
+                st.a = args.a_in[lat];
+            }
+            const bool muca = args.program == kProgMuca ||
+                              (args.program == kProgPass && args.pass_kind == 2);
+            sm.a_f[tid] = muca ? (float)args.muca_a0 : (float)st.a;
+            sm.n_app[tid] = 0;
+        }
+        __syncthreads();
+        if (ph.res) copy_lattices(sm, ph, args, true);
 
         switch (args.program) {
             case kProgSweeps:
             case kProgRM: {
-                if (j == 0 && tid == 0) {
-                    if (args.a_in) sm.st.a = args.a_in[lat];
-                    sm.st.sum_dE = 0.0;
-                    sm.st.sum_dE2 = 0.0;
-                    sm.st.n_meas = 0;
-                }
-                __syncthreads();
-                const float a_f = (float)sm.st.a;
-                composite_sweep<NWP, FAST>(sm, th, a_f, kTagSweep, args.n_or, args.block,
-                                           args.measure && j >= args.n_therm);
-                if (j == per_lat - 1 && tid == 0) {
+                composite_sweep<FAST>(sm, ph, args, kTagSweep, args.measure && j >= args.n_therm);
+                if (j == per_lat - 1 && mine) {
                     if (args.program == kProgRM)
-                        rm_update(sm.st, args, lat);
+                        rm_update(sm.st[tid], args, lat);
                     else if (args.mean_out)
-                        args.mean_out[lat] = sm.st.sum_dE;
+                        args.mean_out[lat] = sm.st[tid].sum_dE;
                 }
                 break;
             }
             case kProgApproach: {
-                int n = 0;
                 for (;;) {
-                    const long long E = sm.st.E_fx;   // uniform after the last barrier
-                    if (dist_fx(E, sm.st.lo_fx, sm.st.hi_fx) == 0) break;
-                    if (n >= args.max_approach) {
-                        if (tid == 0) sm.st.status = -3;   // LLR_ERR_WINDOW
-                        break;
+                    bool go = false;
+                    if (mine) {
+                        LatState &st = sm.st[tid];
+                        go = dist_fx(st.E_fx, st.lo_fx, st.hi_fx) != 0;
+                        if (go && sm.n_app[tid] >= args.max_approach) {
+                            st.status = -3;   // LLR_ERR_WINDOW
+                            go = false;
+                        }
+                        sm.active[tid] = go;
+                        sm.a_f[tid] = (float)(st.E_fx < st.lo_fx ? -args.beta_up : -args.beta_dn);
+                        sm.n_app[tid] += go;
                     }
-                    const float a_f = (float)(E < sm.st.lo_fx ? -args.beta_up : -args.beta_dn);
-                    composite_sweep<NWP, FAST>(sm, th, a_f, kTagApproach, args.n_or, args.block,
-                                               false);
-                    ++n;
+                    if (!__syncthreads_or(go)) break;
+                    composite_sweep<FAST>(sm, ph, args, kTagApproach, false);
                 }
-                if (tid == 0 && args.approach_sweeps) args.approach_sweeps[lat] = n;
+                if (mine && args.approach_sweeps) args.approach_sweeps[lat] = sm.n_app[tid];
                 break;
             }
-            case kProgResync: {
-                const long long fresh = fresh_energy_fx<NWP>(sm, th);
-                if (tid == 0) sm.st.E_fx = fresh;
+            case kProgResync:
+                energy_phase(sm, ph, args, false, false);
                 break;
-            }
             case kProgPass: {
-                if (tid == 0 && args.a_in) sm.st.a = args.a_in[lat];
-                __syncthreads();
                 if (args.pass_kind == 2)   // multicanonical heat-bath pass at slope a0
-                    run_pass<NWP, FAST>(sm, th, 2, (float)args.muca_a0, kTagSweep, 1,
-                                        args.class_mask, &args);
+                    heatbath_phase<FAST>(sm, ph, args, 2, kTagSweep, 1, args.class_mask);
                 else if (args.pass_kind == 3)   // the end of a composite sweep
-                    end_of_sweep<NWP>(sm, th, false);
+                    energy_phase(sm, ph, args, true, false);
+                else if (args.pass_kind == 1)
+                    overrelax_phase<FAST>(sm, ph, args, args.block, args.class_mask, true);
                 else
-                    run_pass<NWP, FAST>(sm, th, args.pass_kind, (float)sm.st.a, kTagSweep,
-                                        args.block, args.class_mask);
+                    heatbath_phase<FAST>(sm, ph, args, 0, kTagSweep, args.block, args.class_mask);
                 break;
             }
             case kProgMuca: {
                 // one multicanonical composite sweep (Sec. 2.6): heat-bath pass
                 // for the weight 1/rho~, n_or overrelaxation passes (they keep
                 // E, so every weight of E takes them), resync, energy history
-                run_pass<NWP, FAST>(sm, th, 2, (float)args.muca_a0, kTagSweep, 1, 0xFF, &args);
+                heatbath_phase<FAST>(sm, ph, args, 2, kTagSweep, 1, 0xFF);
                 for (int k = 0; k < args.n_or; ++k)
-                    run_pass<NWP, FAST>(sm, th, 1, 0.0f, kTagSweep, 1, 0xFF, nullptr, false);
-                end_of_sweep<NWP>(sm, th, false);
-                if (tid == 0 && args.e_hist)
+                    overrelax_phase<FAST>(sm, ph, args, 1, 0xFF, false);
+                energy_phase(sm, ph, args, true, false);
+                if (mine && args.e_hist)
                     args.e_hist[(size_t)j * (size_t)args.n_lat + (size_t)lat] =
-                        (double)sm.st.E_fx * kInvFx;
-                break;
-            }
-            case kProgBegin: {
-                if (tid == 0) {
-                    if (args.a_in) sm.st.a = args.a_in[lat];
-                    sm.st.sum_dE = 0.0;
-                    sm.st.sum_dE2 = 0.0;
-                    sm.st.n_meas = 0;
-                }
+                        (double)sm.st[tid].E_fx * kInvFx;
                 break;
             }
             case kProgFinish:
-                end_of_sweep<NWP>(sm, th, args.measure != 0);
+                energy_phase(sm, ph, args, true, args.measure != 0);
                 break;
             case kProgUpdate:
-                if (tid == 0) rm_update(sm.st, args, lat);
+                if (mine) rm_update(sm.st[tid], args, lat);
                 break;
             default:
                 break;
         }
         __syncthreads();
-        if (tid == 0) {
-            sm.st.caps += sm.cap_cnt;
-            args.lats[lat] = sm.st;
+        if (ph.res) copy_lattices(sm, ph, args, false);
+        if (mine) {
+            sm.st[tid].caps += sm.cap_cnt[tid];
+            args.lats[lat] = sm.st[tid];
             __threadfence();
-            st_release(done + slot, (unsigned)(j + 1));
+        }
+        __syncthreads();
+        if (tid == 0) {
+            __threadfence();
+            st_release(done + (unsigned)(sm.item_first / args.teams), (unsigned)(j + 1));
         }
         __syncthreads();
     }
@@ -1277,57 +2065,95 @@ __global__ void from_canonical_kernel(const LatState *lat, float *theta, const f
     }
 }
 
-// Dynamic shared memory of one kernel variant: the two stage column sets.
-template <int NWP>
-constexpr size_t stage_bytes() { return 2u * kStaged * (NWP + 1) * 32 * sizeof(float); }
+// Shared memory an SM gives to one CTA (227 KB) less the kernel's static part.
+constexpr size_t kDynMax = 227 * 1024 - ((sizeof(Smem) + 127) / 128) * 128;
 
-// Resident CTAs of one kernel variant under a shared-memory carve-out
-// preference (carveout: percent of the unified L1/shared storage, or -1 for
-// the driver's default).  Queried once per process, device and carve-out; the
-// query also sets the variant's dynamic shared memory limit and carve-out (a
-// property of the kernel function in this process, so the last configured
-// carve-out of a variant applies to every handle that launches it).
-template <int NWP, bool FAST>
-int resident_ctas(int carveout)
+constexpr size_t slab_bytes(int L) { return 16u * (size_t)L * L * L; }
+constexpr size_t lattice_bytes(int L) { return slab_bytes(L) * (size_t)L; }
+static_assert(slab_bytes(kSlabMaxL) <= kDynMax, "the largest slab fits");
+
+// SMs of the current device, with the kernel's shared-memory limit and
+// carve-out preference (percent of the unified L1/shared storage, or -1 for
+// the driver's default) set.  Queried once per process, device and carve-out;
+// the carve-out is a property of the kernel function in this process, so the
+// last one configured applies to every handle that launches it.
+template <bool FAST>
+int prepare_kernel(int carveout)
 {
-    static int cached[64][4] = {};
+    static int sms[64] = {};
     static int applied[64] = {};   // carve-out index + 1 last applied per device
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 64) dev = 0;
     const int ci = carveout < 0 ? 0 : carveout <= 50 ? 1 : carveout <= 75 ? 2 : 3;
     if (applied[dev] != ci + 1) {
-        cudaFuncSetAttribute(llr_kernel<NWP, FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)stage_bytes<NWP>());
+        cudaFuncSetAttribute(llr_kernel<FAST>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)kDynMax);
         const int pct = ci == 0 ? (int)cudaSharedmemCarveoutDefault : ci == 1 ? 50 : ci == 2 ? 75 : 100;
-        cudaFuncSetAttribute(llr_kernel<NWP, FAST>, cudaFuncAttributePreferredSharedMemoryCarveout,
-                             pct);
+        cudaFuncSetAttribute(llr_kernel<FAST>, cudaFuncAttributePreferredSharedMemoryCarveout, pct);
         applied[dev] = ci + 1;
     }
-    if (cached[dev][ci] == 0) {
-        int per_sm = 0, sms = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, llr_kernel<NWP, FAST>,
-                                                      (NWP + 1) * 32, stage_bytes<NWP>());
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cached[dev][ci] = (per_sm > 0 ? per_sm : 1) * (sms > 0 ? sms : 1);
+    if (sms[dev] == 0) {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
+        sms[dev] = n > 0 ? n : 1;
     }
-    return cached[dev][ci];
+    return sms[dev];
 }
 
-template <int NWP, bool FAST>
-cudaError_t launch_t(const KernelArgs &a, int carveout, cudaStream_t s, int *grid_out)
+// Lattices a CTA works on at a time.
+int choose_teams(const LaunchCfg &cfg, int n_lat, int sms)
+{
+    if (!cfg.auto_threads)
+        return cfg.threads >= 512 ? 1 : cfg.threads >= 256 ? 3 : cfg.threads >= 160 ? 4 : 6;
+    return n_lat <= sms + sms / 2 ? 1 : n_lat <= 2 * sms ? 2 : 3;
+}
+
+template <bool FAST>
+cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *grid_out)
 {
     const bool multi = a.program == kProgSweeps || a.program == kProgRM || a.program == kProgMuca;
-    const long long items = (long long)a.n_lat * (multi ? (a.n_therm + a.n_meas) : 1);
-    if (items <= 0) return cudaSuccess;
-    const long long cap = resident_ctas<NWP, FAST>(carveout);
-    const int grid = (int)(items < cap ? items : cap);
+    const int per_lat = multi ? (a.n_therm + a.n_meas) : 1;
+    if ((long long)a.n_lat * per_lat <= 0) return cudaSuccess;
+    const int sms = prepare_kernel<FAST>(cfg.carveout);
+    a.teams = choose_teams(cfg, a.n_lat, sms);
+    // 15 named barriers, two per ring stage of each team
+    const int most = a.teams == 1 ? 4 : a.teams <= 3 ? 2 : 1;
+    a.ring = cfg.ring < most ? cfg.ring : most;
+    const size_t stage1 = (size_t)a.teams * (kWarps / a.teams - 1) * kStageGroupBytes;
+    const size_t lattices = (size_t)a.teams * lattice_bytes(a.max_L);
+    // a lattice may be resident if a team of the overrelaxation pass has a
+    // thread for each of the L^3 / 2 links of a slab's class
+    const int or_most = std::min(a.teams, 3);
+    a.resident = a.max_L <= kResidentMaxL && lattices + stage1 <= kDynMax &&
+                 a.max_L * a.max_L * a.max_L / 2 <= kWarps / or_most * 32;
+    while (a.resident && lattices + stage1 * a.ring > kDynMax) a.ring >>= 1;
+    size_t rings = stage1 * a.ring;
+    size_t dyn;
+    if (a.resident) {
+        a.or_teams = or_most;
+        a.slab = (int)(lattice_bytes(a.max_L) / sizeof(float));
+        a.ring_off = (int)(lattices / sizeof(float));
+        dyn = lattices + rings;
+    } else {
+        const size_t slab = a.slab_L > 0 ? slab_bytes(a.slab_L) : 0;
+        const size_t stage = (size_t)kStaged * kThreads * sizeof(float2);
+        while (a.ring > 1 && stage + stage1 * a.ring > kDynMax) a.ring >>= 1;
+        rings = stage1 * a.ring;
+        a.or_teams = or_most;
+        while (a.or_teams > 1 && slab * a.or_teams > kDynMax) --a.or_teams;
+        a.slab = (int)(slab / sizeof(float));
+        a.ring_off = (int)(stage / sizeof(float));
+        dyn = std::max(stage + rings, slab * a.or_teams);
+    }
+    const long long items = (long long)((a.n_lat + a.teams - 1) / a.teams) * per_lat;
+    const int grid = (int)(items < sms ? items : sms);
     if (grid_out) *grid_out = grid;
     // the item counter and the done counters; the error word sync[0] is left
     // alone (sticky until the host reads and clears it)
     cudaError_t e = cudaMemsetAsync(a.sync + 1, 0, sizeof(unsigned) * (size_t)(1 + a.n_lat), s);
     if (e != cudaSuccess) return e;
-    llr_kernel<NWP, FAST><<<grid, (NWP + 1) * 32, stage_bytes<NWP>(), s>>>(a);
+    llr_kernel<FAST><<<grid, kThreads, dyn, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -1335,31 +2161,14 @@ cudaError_t launch_t(const KernelArgs &a, int carveout, cudaStream_t s, int *gri
 
 void prime_launch(const LaunchCfg &cfg)
 {
-    const bool f = cfg.fast_math != 0;
-    const int c = cfg.carveout;
-    switch (cfg.threads) {
-        case 128: f ? resident_ctas<3, true>(c) : resident_ctas<3, false>(c); break;
-        case 160: f ? resident_ctas<4, true>(c) : resident_ctas<4, false>(c); break;
-        case 192: f ? resident_ctas<5, true>(c) : resident_ctas<5, false>(c); break;
-        case 512: f ? resident_ctas<15, true>(c) : resident_ctas<15, false>(c); break;
-        default: f ? resident_ctas<7, true>(c) : resident_ctas<7, false>(c); break;
-    }
+    cfg.fast_math ? prepare_kernel<true>(cfg.carveout) : prepare_kernel<false>(cfg.carveout);
 }
 
 cudaError_t launch_llr(const KernelArgs &args, const LaunchCfg &cfg, cudaStream_t s, int *grid_out)
 {
     if (args.n_lat <= 0) return cudaSuccess;
-    KernelArgs a = args;
-    a.ring = cfg.ring;
-    const bool f = cfg.fast_math != 0;
-    const int c = cfg.carveout;
-    switch (cfg.threads) {
-        case 128: return f ? launch_t<3, true>(a, c, s, grid_out) : launch_t<3, false>(a, c, s, grid_out);
-        case 160: return f ? launch_t<4, true>(a, c, s, grid_out) : launch_t<4, false>(a, c, s, grid_out);
-        case 192: return f ? launch_t<5, true>(a, c, s, grid_out) : launch_t<5, false>(a, c, s, grid_out);
-        case 512: return f ? launch_t<15, true>(a, c, s, grid_out) : launch_t<15, false>(a, c, s, grid_out);
-        default: return f ? launch_t<7, true>(a, c, s, grid_out) : launch_t<7, false>(a, c, s, grid_out);
-    }
+    return cfg.fast_math ? launch_t<true>(args, cfg, s, grid_out)
+                         : launch_t<false>(args, cfg, s, grid_out);
 }
 
 __global__ void step_increment_kernel(int *step)

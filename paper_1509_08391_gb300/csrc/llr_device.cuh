@@ -52,7 +52,7 @@ constexpr float kTwoPi = 6.28318530717958647692f;
 // Wrap to [-pi, pi).
 __device__ __forceinline__ float wrap_angle(float t)
 {
-    return t - kTwoPi * floorf((t + kPi) * (1.0f / kTwoPi));
+    return fmaf(-kTwoPi, floorf(__fmul_rn(t + kPi, 1.0f / kTwoPi)), t);
 }
 
 // sqrt(x) for x >= 0 as x times the hardware reciprocal square root (a few
@@ -75,7 +75,7 @@ __device__ __forceinline__ float arg_fast(float y, float x)
     const float ax = fabsf(x), ay = fabsf(y);
     const float mx = fmaxf(ax, ay), mn = fminf(ax, ay);
     const float t = __fdividef(mn, fmaxf(mx, 1e-30f));
-    const float u = t * t;
+    const float u = __fmul_rn(t, t);
     float p = -0.004054567310959101f;
     p = fmaf(p, u, 0.021862957626581192f);
     p = fmaf(p, u, -0.0559123270213604f);
@@ -84,10 +84,80 @@ __device__ __forceinline__ float arg_fast(float y, float x)
     p = fmaf(p, u, 0.19946566224098206f);
     p = fmaf(p, u, -0.33329859375953674f);
     p = fmaf(p, u, 0.9999993443489075f);
-    float r = t * p;
+    float r = __fmul_rn(t, p);
     r = ay > ax ? 1.57079632679489662f - r : r;
     r = x < 0.0f ? kPi - r : r;
     return copysignf(r, y);
+}
+
+// ---------------------------------------------------------------------------
+// Two float32 operations in one instruction (each rounded to nearest, exactly
+// as the scalar operation).
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ unsigned long long pack2(float2 v)
+{
+    unsigned long long r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(v.x), "f"(v.y));
+    return r;
+}
+__device__ __forceinline__ float2 unpack2(unsigned long long v)
+{
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    unsigned long long r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    unsigned long long r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(pack2(a)), "l"(pack2(b)), "l"(pack2(c)));
+    return unpack2(r);
+}
+__device__ __forceinline__ float2 both(float v)
+{
+    return make_float2(v, v);
+}
+
+// arg_fast of two vectors, with the same roundings (t P(t^2) is rounded before
+// the octant's subtraction).
+__device__ __forceinline__ float2 arg_fast2(float2 y, float2 x)
+{
+    const float ax0 = fabsf(x.x), ay0 = fabsf(y.x), ax1 = fabsf(x.y), ay1 = fabsf(y.y);
+    float2 t;
+    t.x = __fdividef(fminf(ax0, ay0), fmaxf(fmaxf(ax0, ay0), 1e-30f));
+    t.y = __fdividef(fminf(ax1, ay1), fmaxf(fmaxf(ax1, ay1), 1e-30f));
+    const float2 u = mul2(t, t);
+    float2 p = both(-0.004054567310959101f);
+    p = fma2(p, u, both(0.021862957626581192f));
+    p = fma2(p, u, both(-0.0559123270213604f));
+    p = fma2(p, u, both(0.0964219719171524f));
+    p = fma2(p, u, both(-0.1390862911939621f));
+    p = fma2(p, u, both(0.19946566224098206f));
+    p = fma2(p, u, both(-0.33329859375953674f));
+    p = fma2(p, u, both(0.9999993443489075f));
+    float2 r = mul2(t, p);
+    r.x = ay0 > ax0 ? 1.57079632679489662f - r.x : r.x;
+    r.y = ay1 > ax1 ? 1.57079632679489662f - r.y : r.y;
+    r.x = x.x < 0.0f ? kPi - r.x : r.x;
+    r.y = x.y < 0.0f ? kPi - r.y : r.y;
+    return make_float2(copysignf(r.x, y.x), copysignf(r.y, y.y));
 }
 
 // ---------------------------------------------------------------------------

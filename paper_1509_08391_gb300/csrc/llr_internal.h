@@ -57,21 +57,27 @@ struct KernelArgs {
     int muca_n;
     double muca_e0, muca_de, muca_a0;
     double *e_hist;       // kProgMuca, nullable: e_hist[sweep * n_lat + lattice] = E
-    int ring;             // stages of the heat-bath ring in use (1, 2 or 4; set at launch)
+    int max_L;            // largest L of the handle's lattices
+    int slab_L;           // largest L <= 24 of them (0: none): shared-memory slabs
+    // set at launch: lattices a CTA works on at a time; whether it holds them in
+    // shared memory as a whole; otherwise slabs in shared memory at a time; the
+    // floats of a lattice / slab; stages of the heat-bath ring and its offset
+    int teams, resident, or_teams, slab, ring, ring_off;
 };
 
 // *step += 1 (the last node of a captured Robbins-Monro step).
 cudaError_t launch_step_increment(int *step, cudaStream_t s);
 
 struct LaunchCfg {
-    int threads = 256;    // 128, 160, 192, 256 or 512: one consumer warp, the rest producers
+    bool auto_threads = true;   // until a shape is set: lattices per CTA by the batch's size
+    int threads = 256;    // most threads per lattice (128, 160, 192, 256 or 512)
     bool fast_math = true;
     int ring = 4;         // stages of the heat-bath producer/consumer ring in use: 1, 2 or 4
     int carveout = -1;    // shared-memory carve-out preference in percent, -1 = default
 };
 
-// Query (and cache) the resident-CTA count of a kernel variant; call before a
-// stream capture so the capture itself makes no occupancy queries.
+// Query (and cache) the device's SM count and set the kernel's attributes; call
+// before a stream capture so the capture itself makes no such calls.
 void prime_launch(const LaunchCfg &cfg);
 
 // Reset the work queue and launch the persistent kernel (stream ordered);
