@@ -999,12 +999,13 @@ int llr_cv_peak(int n, const double *centres, const double *a, double beta_lo, d
     if (!out || n_grid < 2 || !(beta_hi > beta_lo) || !(tol > 0.0))
         return fail(LLR_ERR_ARG, "bad peak-search arguments");
     DevBuf b;
-    LLR_CUDA(cudaMalloc(&b.p, sizeof(double) * (3 * (size_t)n + 2)));
-    double *dc = (double *)b.p, *da = dc + n, *dl = da + n, *dout = dl + n;
+    const size_t scratch = llr::cv_peak_scratch(n_grid, beta_lo, beta_hi, tol);
+    LLR_CUDA(cudaMalloc(&b.p, sizeof(double) * (3 * (size_t)n + 2 + scratch)));
+    double *dc = (double *)b.p, *da = dc + n, *dl = da + n, *dout = dl + n, *ds = dout + 2;
     LLR_CUDA(cudaMemcpy(dc, centres, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice));
     LLR_CUDA(cudaMemcpy(da, a, sizeof(double) * (size_t)n, cudaMemcpyHostToDevice));
     LLR_CUDA(llr::launch_lnrho(n, dc, da, dl, nullptr));
-    LLR_CUDA(llr::launch_cv_peak(n, dc, dl, beta_lo, beta_hi, n_grid, tol, dout, nullptr));
+    LLR_CUDA(llr::launch_cv_peak(n, dc, dl, beta_lo, beta_hi, n_grid, tol, ds, dout, nullptr));
     LLR_CUDA(cudaMemcpy(out, dout, sizeof(double) * 2, cudaMemcpyDeviceToHost));
     return LLR_OK;
 }

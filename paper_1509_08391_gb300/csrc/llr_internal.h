@@ -117,7 +117,9 @@ cudaError_t launch_observables(int n, const double *c, const double *a, int n_be
                                const double *beta, double *lnZ, double *E1, double *E2,
                                cudaStream_t s);
 cudaError_t launch_cv_peak(int n, const double *c, const double *a, double beta_lo,
-                           double beta_hi, int n_grid, double tol, double *out,
+                           double beta_hi, int n_grid, double tol, double *scratch, double *out,
+// scratch: cv_peak_scratch doubles
+size_t cv_peak_scratch(int n_grid, double beta_lo, double beta_hi, double tol);
                            cudaStream_t s);
 
 // Multicanonical reweighting kernels (Sec. 2.6, eq. (2.56)): ln rho~ of the

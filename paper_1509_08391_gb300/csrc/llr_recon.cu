@@ -10,10 +10,11 @@
 //                    with weight 1/rho~ carries exp(beta E_i + ln rho~(E_i));
 //                    tunnellings of a chain between the ends of the range
 //
-// Sizes are small (hundreds to thousands of intervals), so each quantity is
-// one CTA: a block-wide FP64 scan for ln rho, log-sum-exp reductions for the
-// observables, and a device-side grid scan + golden-section search for the
-// C_V peak.
+// Sizes are small (hundreds to thousands of intervals): one CTA scans ln rho, one
+// CTA per coupling forms the log-sum-exp observables, and the C_V peak is a grid
+// scan and a golden-section search on the device, many couplings at once.
+#include <algorithm>
+#include <cmath>
 #include <string>
 
 #include "../../include/llr.h"
@@ -131,48 +132,171 @@ __device__ double cv_at(int n, const double *c, const double *lr, double beta, d
     return e2 - e1 * e1;
 }
 
-__global__ void __launch_bounds__(kT) cv_peak_kernel(int n, const double *c, const double *lr,
+// C_V at the grid point of every block.
+__global__ void __launch_bounds__(kT) cv_grid_kernel(int n, const double *c, const double *lr,
                                                      double blo, double bhi, int n_grid,
-                                                     double tol, double *out)
+                                                     double *cv)
 {
     __shared__ double red[kT / 32];
-    int best = 0;
-    double best_cv = -INFINITY;
-    for (int i = 0; i < n_grid; ++i) {
-        const double b = n_grid > 1 ? blo + (bhi - blo) * (double)i / (double)(n_grid - 1) : blo;
-        const double v = cv_at(n, c, lr, b, red);
-        if (v > best_cv) {
-            best_cv = v;
-            best = i;
-        }
-    }
-    const double step = n_grid > 1 ? (bhi - blo) / (double)(n_grid - 1) : 0.0;
-    double lo = blo + step * (double)(best > 0 ? best - 1 : 0);
-    double hi = blo + step * (double)(best < n_grid - 1 ? best + 1 : n_grid - 1);
-    const double g = 0.6180339887498949;   // (sqrt 5 - 1) / 2
-    double x1 = hi - g * (hi - lo), x2 = lo + g * (hi - lo);
-    double f1 = cv_at(n, c, lr, x1, red), f2 = cv_at(n, c, lr, x2, red);
-    for (int it = 0; it < 200 && hi - lo > tol; ++it) {
-        if (f1 < f2) {
+    const int i = blockIdx.x;
+    const double b = n_grid > 1 ? blo + (bhi - blo) * (double)i / (double)(n_grid - 1) : blo;
+    const double v = cv_at(n, c, lr, b, red);
+    if (threadIdx.x == 0) cv[i] = v;
+}
+
+// Golden-section search on the device.  One evaluation is a chain of exps and
+// block reductions on one SM (8 us at 512 centres, mostly FP64 latency), and a
+// step needs the comparison before it, so the steps are taken several at a
+// time: a round evaluates the points of all outcomes of the next comparisons at
+// once, one block each, and the next round replays the comparisons on the
+// values found.  512 centres, 1601 grid points, tol 1e-10 (26 steps): 14.4 ms
+// with one block for everything, 0.1 ms with the grid in parallel and 5 rounds.
+constexpr int kFirstDepth = 6, kDepth = 7;            // comparisons ahead per round
+constexpr int kFirstNodes = 2 + 2 * ((1 << kFirstDepth) - 1);   // x1, x2, a tree per outcome
+constexpr int kNodes = (1 << kDepth) - 1;             // one tree: the first outcome is known
+constexpr int kMaxSteps = 200;
+
+struct Golden {
+    double lo, hi, x1, x2, f1, f2;
+    int it;
+    __device__ bool open(double tol) const { return it < kMaxSteps && hi - lo > tol; }
+    // narrow the interval by the outcome of f1 < f2; returns the new point
+    __device__ double step(bool less)
+    {
+        const double g = 0.6180339887498949;   // (sqrt 5 - 1) / 2
+        ++it;
+        if (less) {
             lo = x1;
             x1 = x2;
             f1 = f2;
             x2 = lo + g * (hi - lo);
-            f2 = cv_at(n, c, lr, x2, red);
-        } else {
-            hi = x2;
-            x2 = x1;
-            f2 = f1;
-            x1 = hi - g * (hi - lo);
-            f1 = cv_at(n, c, lr, x1, red);
+            return x2;
+        }
+        hi = x2;
+        x2 = x1;
+        f2 = f1;
+        x1 = hi - g * (hi - lo);
+        return x1;
+    }
+};
+
+// The search's state after `rounds` rounds, whose values are F[round][node]; the
+// start from the best of the grid values cv (the first of the largest).
+__device__ Golden golden_replay(const double *cv, double blo, double bhi, int n_grid, double tol,
+                                const double *F, int rounds)
+{
+    __shared__ double bv[kT / 32];
+    __shared__ int bi[kT / 32];
+    double v = -INFINITY;
+    int best = n_grid;
+    for (int i = threadIdx.x; i < n_grid; i += kT)
+        if (cv[i] > v) {
+            v = cv[i];
+            best = i;
+        }
+    for (int o = 16; o > 0; o >>= 1) {
+        const double w = __shfl_xor_sync(kFull, v, o);
+        const int j = __shfl_xor_sync(kFull, best, o);
+        if (w > v || (w == v && j < best)) {
+            v = w;
+            best = j;
         }
     }
-    const double b = 0.5 * (lo + hi);
+    if ((threadIdx.x & 31) == 0) {
+        bv[threadIdx.x >> 5] = v;
+        bi[threadIdx.x >> 5] = best;
+    }
+    __syncthreads();
+    for (int w = 0; w < kT / 32; ++w)
+        if (bv[w] > v || (bv[w] == v && bi[w] < best)) {
+            v = bv[w];
+            best = bi[w];
+        }
+    if (best == n_grid) best = 0;   // no value above -inf
+    Golden s;
+    const double step = n_grid > 1 ? (bhi - blo) / (double)(n_grid - 1) : 0.0;
+    s.lo = blo + step * (double)(best > 0 ? best - 1 : 0);
+    s.hi = blo + step * (double)(best < n_grid - 1 ? best + 1 : n_grid - 1);
+    const double g = 0.6180339887498949;
+    s.x1 = s.hi - g * (s.hi - s.lo);
+    s.x2 = s.lo + g * (s.hi - s.lo);
+    s.f1 = s.f2 = 0.0;
+    s.it = 0;
+    for (int r = 0; r < rounds; ++r, F += kFirstNodes) {
+        if (r == 0) {
+            s.f1 = F[0];
+            s.f2 = F[1];
+        }
+        const double *tree = F + (r > 0 ? 0 : s.f1 < s.f2 ? 2 + kFirstNodes / 2 - 1 : 2);
+        const int depth = r > 0 ? kDepth : kFirstDepth;
+        int node = 1;
+        for (int d = 0; d < depth && s.open(tol); ++d) {
+            const bool less = s.f1 < s.f2;
+            if (d > 0) node = 2 * node + less;
+            s.step(less);
+            (less ? s.f2 : s.f1) = tree[node - 1];
+        }
+    }
+    return s;
+}
+
+// Round `round`: block k evaluates node k.  In a tree, node 1 is the point after
+// the first comparison, nodes 2 m and 2 m + 1 those after node m's comparison
+// came out not less / less.
+__global__ void __launch_bounds__(kT) golden_round_kernel(int n, const double *c, const double *lr,
+                                                          double blo, double bhi, int n_grid,
+                                                          double tol, const double *cv,
+                                                          double *F, int round)
+{
+    __shared__ double red[kT / 32];
+    Golden s = golden_replay(cv, blo, bhi, n_grid, tol, F, round);
+    int node = blockIdx.x + 1;
+    bool less = s.f1 < s.f2;
+    double x;
+    if (round == 0 && blockIdx.x < 2) {
+        x = blockIdx.x == 0 ? s.x1 : s.x2;
+    } else {
+        if (round == 0) {
+            node = blockIdx.x - 2;
+            less = node >= kFirstNodes / 2 - 1;
+            node = node % (kFirstNodes / 2 - 1) + 1;
+        }
+        if (!s.open(tol)) return;
+        x = s.step(less);
+        for (int bit = 31 - __clz(node) - 1; bit >= 0; --bit) {
+            if (!s.open(tol)) return;   // a point the search never asks for
+            x = s.step((node >> bit) & 1);
+        }
+    }
+    const double v = cv_at(n, c, lr, x, red);
+    if (threadIdx.x == 0) F[(size_t)round * kFirstNodes + blockIdx.x] = v;
+}
+
+__global__ void __launch_bounds__(kT) golden_result_kernel(int n, const double *c, const double *lr,
+                                                           double blo, double bhi, int n_grid,
+                                                           double tol, const double *cv,
+                                                           const double *F, int rounds,
+                                                           double *out)
+{
+    __shared__ double red[kT / 32];
+    const Golden s = golden_replay(cv, blo, bhi, n_grid, tol, F, rounds);
+    const double b = 0.5 * (s.lo + s.hi);
     const double v = cv_at(n, c, lr, b, red);
     if (threadIdx.x == 0) {
         out[0] = b;
         out[1] = v;
     }
+}
+
+// Rounds that are sure to reach the tolerance (two steps of slack for rounding).
+int golden_rounds(double blo, double bhi, int n_grid, double tol)
+{
+    const double len = 2.0 * (bhi - blo) / (double)(n_grid - 1);
+    int steps = kMaxSteps;
+    if (tol > 0.0 && std::isfinite(len / tol))
+        steps = (int)std::min<double>(
+            kMaxSteps, std::max(0.0, std::ceil(std::log(len / tol) / 0.48121182505960347)) + 2.0);
+    return 1 + std::max(0, (steps - kFirstDepth + kDepth - 1) / kDepth);
 }
 
 // ---------------------------------------------------------------------------
@@ -338,10 +462,23 @@ cudaError_t launch_observables(int n, const double *c, const double *lr, int n_b
     return cudaGetLastError();
 }
 
-cudaError_t launch_cv_peak(int n, const double *c, const double *lr, double beta_lo,
-                           double beta_hi, int n_grid, double tol, double *out, cudaStream_t s)
+size_t cv_peak_scratch(int n_grid, double beta_lo, double beta_hi, double tol)
 {
-    cv_peak_kernel<<<1, kT, 0, s>>>(n, c, lr, beta_lo, beta_hi, n_grid, tol, out);
+    return (size_t)n_grid + (size_t)kFirstNodes * golden_rounds(beta_lo, beta_hi, n_grid, tol);
+}
+
+cudaError_t launch_cv_peak(int n, const double *c, const double *lr, double beta_lo,
+                           double beta_hi, int n_grid, double tol, double *scratch, double *out,
+                           cudaStream_t s)
+{
+    double *cv = scratch, *F = scratch + n_grid;
+    const int rounds = golden_rounds(beta_lo, beta_hi, n_grid, tol);
+    cv_grid_kernel<<<n_grid, kT, 0, s>>>(n, c, lr, beta_lo, beta_hi, n_grid, cv);
+    for (int r = 0; r < rounds; ++r)
+        golden_round_kernel<<<r > 0 ? kNodes : kFirstNodes, kT, 0, s>>>(
+            n, c, lr, beta_lo, beta_hi, n_grid, tol, cv, F, r);
+    golden_result_kernel<<<1, kT, 0, s>>>(n, c, lr, beta_lo, beta_hi, n_grid, tol, cv, F, rounds,
+                                          out);
     return cudaGetLastError();
 }
 
