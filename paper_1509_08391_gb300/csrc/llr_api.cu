@@ -25,6 +25,7 @@ struct llr_ctx {
     LatState *d_lat = nullptr;
     std::vector<LatState> h_lat;     // host copy of the static fields (geometry, window)
     double *d_a = nullptr, *d_mean = nullptr;
+    double *d_part = nullptr;        // scratch of the FP64 energies
     int *d_int = nullptr;
     float *d_links = nullptr;        // staging for llr_get/set_links
     size_t links_cap = 0;
@@ -247,6 +248,7 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
     LLR_CUDA(cudaMalloc(&h->d_lat, sizeof(LatState) * (size_t)n));
     LLR_CUDA(cudaMalloc(&h->d_a, sizeof(double) * (size_t)n));
     LLR_CUDA(cudaMalloc(&h->d_mean, sizeof(double) * (size_t)n));
+    LLR_CUDA(cudaMalloc(&h->d_part, sizeof(double) * llr::energy_parts(n)));
     LLR_CUDA(cudaMalloc(&h->d_int, sizeof(int) * (size_t)(n + 1)));
     LLR_CUDA(cudaMalloc(&h->d_sync, sizeof(unsigned) * (size_t)(n + 2)));
     LLR_CUDA(cudaMemset(h->d_sync, 0, sizeof(unsigned) * (size_t)(n + 2)));
@@ -577,7 +579,8 @@ int llr_energy(llr_handle h, double *E_out)
 {
     if (int r = check_handle(h)) return r;
     if (!E_out) return fail(LLR_ERR_ARG, "null E_out");
-    LLR_CUDA(llr::launch_energy_fp64(h->d_lat, h->d_theta, h->n, h->d_mean, h->stream));
+    LLR_CUDA(llr::launch_energy_fp64(h->d_lat, h->d_theta, h->n, h->max_half, h->d_part, h->d_mean,
+                                     h->stream));
     LLR_CUDA(cudaMemcpyAsync(E_out, h->d_mean, sizeof(double) * (size_t)h->n,
                              cudaMemcpyDeviceToHost, h->stream));
     LLR_CUDA(cudaStreamSynchronize(h->stream));
@@ -617,7 +620,8 @@ int llr_set_links(llr_handle h, int lattice, const float *in)
                              h->stream));
     LLR_CUDA(llr::launch_from_canonical(h->d_lat + lattice, h->d_theta, h->d_links, nl, h->stream));
     // tracked energy from the FP64 plaquette sum of the new angles
-    LLR_CUDA(llr::launch_energy_fp64(h->d_lat + lattice, h->d_theta, 1, h->d_mean, h->stream));
+    LLR_CUDA(llr::launch_energy_fp64(h->d_lat + lattice, h->d_theta, 1, nl / 8, h->d_part, h->d_mean,
+                                     h->stream));
     LLR_CUDA(llr::launch_set_energy(h->d_lat + lattice, h->d_mean, h->stream));
     LLR_CUDA(cudaStreamSynchronize(h->stream));
     return LLR_OK;
@@ -778,6 +782,7 @@ int llr_destroy(llr_handle h)
     cudaFree(h->d_lat);
     cudaFree(h->d_a);
     cudaFree(h->d_mean);
+    cudaFree(h->d_part);
     cudaFree(h->d_int);
     cudaFree(h->d_links);
     cudaFree(h->d_sync);

@@ -92,9 +92,11 @@ cudaError_t launch_hot_start(LatState *lats, float *theta, int n_lat, int max_ha
 // Set the tracked energy of one lattice from an FP64 energy (device scalar).
 cudaError_t launch_set_energy(LatState *lat_dev, const double *E_dev, cudaStream_t s);
 
-// FP64 fresh energies.
-cudaError_t launch_energy_fp64(const LatState *lats, const float *theta, int n_lat,
-                               double *E_out, cudaStream_t s);
+// FP64 fresh energies; part: energy_parts(n_lat) doubles of scratch, max_half the
+// largest half = V / 2 of the lattices.
+size_t energy_parts(int n_lat);
+cudaError_t launch_energy_fp64(const LatState *lats, const float *theta, int n_lat, int max_half,
+                               double *part, double *E_out, cudaStream_t s);
 
 // Canonical (mu*V + s) <-> internal layout of one lattice.
 cudaError_t launch_to_canonical(const LatState *lat_dev, const float *theta, float *out,
@@ -116,10 +118,10 @@ cudaError_t launch_lnrho(int n, const double *c, const double *a, double *out, c
 cudaError_t launch_observables(int n, const double *c, const double *a, int n_beta,
                                const double *beta, double *lnZ, double *E1, double *E2,
                                cudaStream_t s);
-cudaError_t launch_cv_peak(int n, const double *c, const double *a, double beta_lo,
-                           double beta_hi, int n_grid, double tol, double *scratch, double *out,
 // scratch: cv_peak_scratch doubles
 size_t cv_peak_scratch(int n_grid, double beta_lo, double beta_hi, double tol);
+cudaError_t launch_cv_peak(int n, const double *c, const double *a, double beta_lo,
+                           double beta_hi, int n_grid, double tol, double *scratch, double *out,
                            cudaStream_t s);
 
 // Multicanonical reweighting kernels (Sec. 2.6, eq. (2.56)): ln rho~ of the
