@@ -370,8 +370,8 @@ int llr_mlp_grad(llr_mlp_handle h, int n, const double *L, const double *e6v,
                  const double *dE6v, const double *a_target, float *grad_out, double *loss_out);
 /* Full-batch Adam (beta1 0.9, beta2 0.999, eps 1e-8) for `epochs` steps at
  * learning rate lr; standardise != 0 first sets mean/std from these inputs.
- * loss_out (nullable) gets the loss of the final parameters.  The epoch is
- * captured once in a CUDA graph and replayed. */
+ * loss_out (nullable) gets the loss of the final parameters.  All epochs run in
+ * one launch. */
 int llr_mlp_fit(llr_mlp_handle h, int n, const double *L, const double *e6v, const double *dE6v,
                 const double *a_target, int epochs, double lr, int standardise,
                 double *loss_out);

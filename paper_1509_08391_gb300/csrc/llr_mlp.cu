@@ -10,12 +10,11 @@
 //
 // Layout: one float array of parameters, W1 (3x64, row-major [in][out]),
 // b1 (64), W2 (64x64), b2, W3 (64x64), b3, W4 (64x1), b4 (1).  Activations
-// are [sample][feature].  Layers are small, so each kernel is a plain
-// thread-per-output dot product (no tensor cores: a 64-wide layer is not a
-// contraction worth them), and the sums over samples are done in a fixed
-// order (no atomics), so training is deterministic.  One training epoch
-// (features are fixed) is ~13 launches; the host captures it once in a CUDA
-// graph and replays it.
+// are [sample][feature].  Layers are small (no tensor cores: a 64-wide layer is
+// not a contraction worth them), and the sums over samples are done in a fixed
+// order (no atomics), so training is deterministic.  Training runs all its epochs
+// in one launch of a cluster of CTAs; predictions and single gradients use a
+// thread-per-output kernel per layer.
 #include <cmath>
 #include <string>
 #include <vector>
@@ -39,8 +38,8 @@ __device__ __forceinline__ float gelu(float z)
 
 __device__ __forceinline__ float gelu_grad(float z)
 {
-    return 0.5f * (1.0f + erff(z * 0.70710678118654752f)) +
-           z * expf(-0.5f * z * z) * 0.39894228040143268f;
+    const float h = 1.0f + erff(z * 0.70710678118654752f), e = z * expf(-0.5f * z * z);
+    return fmaf(0.5f, h, __fmul_rn(e, 0.39894228040143268f));
 }
 
 // Raw features (1/V, E/6V, dE/6V) standardised with mean / std.
@@ -162,25 +161,317 @@ __global__ void linear_bwd_weight_kernel(int n, int in_dim, int out_dim, const f
     }
 }
 
-// Adam (Kingma & Ba 2015) with bias correction; step count in *t.
-__global__ void adam_kernel(int np, float *P, const float *G, float *M, float *V,
-                            const int *t, float lr, float b1, float b2, float eps)
+// ---------------------------------------------------------------------------
+// Training: all epochs of a fit in one launch of a cluster of kCtas CTAs.
+//
+// An epoch is two parallel phases with a cluster barrier after each.
+//   1. Forward and backward of the samples, which only need the parameters: CTA c
+//      takes a contiguous share of the samples, in tiles of kTile, with all
+//      parameters in shared memory; activations and dZ go to global memory (L2).
+//   2. Parameter gradients and Adam: CTA c owns rows 8 c .. 8 c + 7 of W2 and W3,
+//      the first three CTAs the small tensors besides.  A thread keeps its
+//      parameters and their moments in registers for the whole training, sums
+//      its gradients over all samples (staged through shared memory, kChunk at a
+//      time) and writes the new values into every CTA's shared memory.
+// Every sum runs over the same terms in the same order as in the kernels above,
+// and the fused operations are written out as those round, so results do not
+// depend on the split, bit for bit.  Bound by shared-memory loads: four
+// samples, or four rows, per thread share a weight or a dZ.  One epoch of 120
+// samples took 70 us as 14 launches of a captured graph and takes 12 us here (1000
+// samples 262 -> 79 us), the latency of some 15 short dependent steps.
+// ---------------------------------------------------------------------------
+constexpr int kCtas = 8, kTrainThreads = 512, kTile = 16, kChunk = 128;
+constexpr int kRow = kW / kCtas;        // rows of W2, W3 owned by a CTA
+constexpr int kWs = kW + 1;             // padded row of a weight matrix
+constexpr int kHs = kW + 4;             // padded row of a sample tile (16-byte rows)
+
+struct TrainSmem {
+    float W2[kW * kWs], W3[kW * kWs];
+    float W1[kIn * kW], b1[kW], b2[kW], b3[kW], W4[kW], b4;
+    // phase 1: a tile of samples
+    float X[kTile * kIn];
+    alignas(16) float H[3][kTile * kHs];    // activations
+    alignas(16) float D[3][kTile * kHs];    // gelu'(Z), then dZ
+    float dY[kTile];
+    // phase 2: a chunk of samples
+    alignas(16) float dZ[2][kChunk * kW];   // of layers 2, 3
+    alignas(16) float A[2][kChunk * kRow];  // the owned columns of A1, A2
+    alignas(16) float E[kChunk * kW];       // CTA 1: dZ1, CTA 2: A3
+    float e[kChunk * kIn];                  // CTA 1: X, CTA 2: dY
+};
+
+__device__ __forceinline__ void cluster_sync()
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= np) return;
-    const float c1 = 1.0f - powf(b1, (float)*t);
-    const float c2 = 1.0f - powf(b2, (float)*t);
-    const float g = G[k];
-    const float m = b1 * M[k] + (1.0f - b1) * g;
-    const float v = b2 * V[k] + (1.0f - b2) * g * g;
-    M[k] = m;
-    V[k] = v;
-    P[k] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-__global__ void step_count_kernel(int *t)
+// Store v to the copy of *p in every CTA of the cluster.
+__device__ __forceinline__ void store_all(float *p, float v)
 {
-    *t += 1;
+    const unsigned a = (unsigned)__cvta_generic_to_shared(p);
+#pragma unroll
+    for (int r = 0; r < kCtas; ++r) {
+        unsigned d;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"(a), "r"(r));
+        asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(d), "f"(v) : "memory");
+    }
+}
+
+__device__ __forceinline__ void copy16(float *dst, const float *src)   // through L2 only
+{
+    const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(src) : "memory");
+}
+
+// Adam (Kingma & Ba 2015) with bias correction, c1, c2 = 1 - b^t.
+struct AdamStep {
+    float lr, b1, b2, eps, c1, c2;
+    __device__ __forceinline__ AdamStep(float lr_, float b1_, float b2_, float eps_, int t)
+        : lr(lr_), b1(b1_), b2(b2_), eps(eps_)
+    {
+        c1 = 1.0f - powf(b1, (float)t);
+        c2 = 1.0f - powf(b2, (float)t);
+    }
+    __device__ __forceinline__ void operator()(float &P, float &M, float &V, float g) const
+    {
+        M = fmaf(1.0f - b1, g, __fmul_rn(b1, M));
+        V = fmaf(__fmul_rn(1.0f - b2, g), g, __fmul_rn(b2, V));
+        P -= lr * (M / c1) / (sqrtf(V / c2) + eps);
+    }
+};
+
+// out[s][j] of a 64 x 64 layer for four samples: sum over i of in[s][i] W(i, j),
+// in the order of i, from z.
+template <class Weight>
+__device__ __forceinline__ void dot4(const float *in, Weight W, float z[4])
+{
+#pragma unroll
+    for (int i = 0; i < kW; i += 4) {
+        const float w0 = W(i), w1 = W(i + 1), w2 = W(i + 2), w3 = W(i + 3);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float4 h = *(const float4 *)(in + q * kHs + i);
+            z[q] = fmaf(h.x, w0, z[q]);
+            z[q] = fmaf(h.y, w1, z[q]);
+            z[q] = fmaf(h.z, w2, z[q]);
+            z[q] = fmaf(h.w, w3, z[q]);
+        }
+    }
+}
+
+__global__ void __cluster_dims__(kCtas, 1, 1) __launch_bounds__(kTrainThreads, 1)
+    train_kernel(int n, int epochs, const float *X, const double *T, float *A, float *dZ,
+                 float *dY, float *P, float *M, float *V, int *t, float lr, float b1, float b2,
+                 float eps)
+{
+    extern __shared__ __align__(16) char smem_raw[];
+    TrainSmem &sm = *(TrainSmem *)smem_raw;
+    const int tid = threadIdx.x, c = blockIdx.x;
+    const size_t layer = (size_t)kW * n;   // A and dZ hold layers 1, 2, 3
+
+    // all parameters into shared memory
+    for (int k = tid; k < kW * kW; k += kTrainThreads) {
+        sm.W2[(k / kW) * kWs + k % kW] = P[kOffW2 + k];
+        sm.W3[(k / kW) * kWs + k % kW] = P[kOffW3 + k];
+    }
+    for (int k = tid; k < kIn * kW; k += kTrainThreads) sm.W1[k] = P[kOffW1 + k];
+    if (tid < kW) {
+        sm.b1[tid] = P[kOffB1 + tid];
+        sm.b2[tid] = P[kOffB2 + tid];
+        sm.b3[tid] = P[kOffB3 + tid];
+        sm.W4[tid] = P[kOffW4 + tid];
+        if (tid == 0) sm.b4 = P[kOffB4];
+    }
+
+    // the parameters this thread owns: nk of them, own[q] in the parameter array
+    // and at[q] in shared memory.  Threads 0 .. 255: four rows of a column of W2
+    // (m = 0) or W3 (m = 1); the others, in the first three CTAs, the rest.
+    const int m = tid >> 7, r4 = 4 * ((tid >> 6) & 1), j = tid & 63, e = tid - 256;
+    int nk = 0, first = 0;
+    float *at = nullptr;
+    if (tid < 256) {
+        nk = 4;
+        first = (m ? kOffW3 : kOffW2) + (kRow * c + r4) * kW + j;
+        at = (m ? sm.W3 : sm.W2) + (kRow * c + r4) * kWs + j;
+    } else if (c == 0 && e < 2 * kW) {
+        nk = 1;
+        first = (e < kW ? kOffB2 : kOffB3 - kW) + e;
+        at = e < kW ? sm.b2 + e : sm.b3 + e - kW;
+    } else if (c == 1) {
+        nk = 1;   // W1, b1 are adjacent
+        first = kOffW1 + e;
+        at = e < kIn * kW ? sm.W1 + e : sm.b1 + e - kIn * kW;
+    } else if (c == 2 && e <= kW) {
+        nk = 1;   // W4, b4 are adjacent
+        first = kOffW4 + e;
+        at = e < kW ? sm.W4 + e : &sm.b4;
+    }
+    float p[4] = {0, 0, 0, 0}, mom[4] = {0, 0, 0, 0}, var[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (q < nk) {
+            p[q] = P[first + q * kW];
+            mom[q] = M[first + q * kW];
+            var[q] = V[first + q * kW];
+        }
+    const int t0 = *t;
+    const int share = (n + kCtas - 1) / kCtas, s_end = min(n, (c + 1) * share);
+    cluster_sync();   // every CTA of the cluster runs; parameters are loaded
+
+    for (int ep = 0; ep < epochs; ++ep) {
+        // ------------------------------------------------ phase 1: the samples
+        for (int s0 = c * share; s0 < s_end; s0 += kTile) {
+            const int ns = min(kTile, s_end - s0);
+            if (tid < kTile * kIn) sm.X[tid] = tid < ns * kIn ? X[(size_t)s0 * kIn + tid] : 0.0f;
+            __syncthreads();
+            // hidden layers: Z to H, then A = gelu(Z) and gelu'(Z)
+#pragma unroll
+            for (int l = 0; l < 3; ++l) {
+                float *H = sm.H[l];
+                if (l == 0) {
+                    for (int k = tid; k < kTile * kW; k += kTrainThreads) {
+                        const int s = k / kW, o = k % kW;
+                        float z = sm.b1[o];
+#pragma unroll
+                        for (int i = 0; i < kIn; ++i)
+                            z = fmaf(sm.X[s * kIn + i], sm.W1[i * kW + o], z);
+                        H[s * kHs + o] = z;
+                    }
+                } else if (tid < 256) {
+                    const float *W = (l == 1 ? sm.W2 : sm.W3) + j;
+                    const float bias = l == 1 ? sm.b2[j] : sm.b3[j];
+                    const int s = 4 * (tid >> 6);
+                    float z[4] = {bias, bias, bias, bias};
+                    dot4(sm.H[l - 1] + s * kHs, [&](int i) { return W[i * kWs]; }, z);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) H[(s + q) * kHs + j] = z[q];
+                }
+                __syncthreads();
+                for (int k = tid; k < kTile * kW; k += kTrainThreads) {
+                    const int s = k / kW, o = k % kW;
+                    const float z = H[s * kHs + o], a = gelu(z);
+                    H[s * kHs + o] = a;
+                    sm.D[l][s * kHs + o] = gelu_grad(z);
+                    if (s < ns) A[l * layer + (size_t)(s0 + s) * kW + o] = a;
+                }
+                __syncthreads();
+            }
+            // output and its gradient 2 (y - t) / n
+            if (tid < ns) {
+                float y = sm.b4;
+#pragma unroll
+                for (int i = 0; i < kW; ++i) y = fmaf(sm.H[2][tid * kHs + i], sm.W4[i], y);
+                const double r = (double)y - T[s0 + tid];
+                const float g = (float)(2.0 * r / n);
+                sm.dY[tid] = g;
+                dY[s0 + tid] = g;
+            } else if (tid < kTile) {
+                sm.dY[tid] = 0.0f;
+            }
+            __syncthreads();
+            for (int k = tid; k < kTile * kW; k += kTrainThreads) {
+                const int s = k / kW, i = k % kW;
+                const float g = fmaf(sm.dY[s], sm.W4[i], 0.0f) * sm.D[2][s * kHs + i];
+                sm.D[2][s * kHs + i] = g;
+                if (s < ns) dZ[2 * layer + (size_t)(s0 + s) * kW + i] = g;
+            }
+            __syncthreads();
+#pragma unroll
+            for (int l = 1; l >= 0; --l) {
+                if (tid < 256) {
+                    const float *W = (l == 1 ? sm.W3 : sm.W2) + j * kWs;
+                    const int s = 4 * (tid >> 6);
+                    float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+                    dot4(sm.D[l + 1] + s * kHs, [&](int o) { return W[o]; }, g);
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) {
+                        const float d = g[q] * sm.D[l][(s + q) * kHs + j];
+                        sm.D[l][(s + q) * kHs + j] = d;
+                        if (s + q < ns) dZ[l * layer + (size_t)(s0 + s + q) * kW + j] = d;
+                    }
+                }
+                __syncthreads();
+            }
+        }
+        cluster_sync();
+        // ------------------------------------- phase 2: gradients and parameters
+        float g[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        for (int c0 = 0; c0 < n; c0 += kChunk) {
+            const int nc = min(kChunk, n - c0);
+            for (int k = tid; k < nc * (kW / 4); k += kTrainThreads) {
+                copy16(sm.dZ[0] + 4 * k, dZ + layer + (size_t)c0 * kW + 4 * k);
+                copy16(sm.dZ[1] + 4 * k, dZ + 2 * layer + (size_t)c0 * kW + 4 * k);
+                if (c == 1) copy16(sm.E + 4 * k, dZ + (size_t)c0 * kW + 4 * k);
+                if (c == 2) copy16(sm.E + 4 * k, A + 2 * layer + (size_t)c0 * kW + 4 * k);
+            }
+            for (int k = tid; k < nc * (kRow / 4); k += kTrainThreads) {
+                const int s = k / (kRow / 4), q = 4 * (k % (kRow / 4));
+                const size_t src = (size_t)(c0 + s) * kW + kRow * c + q;
+                copy16(sm.A[0] + s * kRow + q, A + src);
+                copy16(sm.A[1] + s * kRow + q, A + layer + src);
+            }
+            if (c == 1)
+                for (int k = tid; k < nc * kIn; k += kTrainThreads)
+                    sm.e[k] = X[(size_t)c0 * kIn + k];
+            if (c == 2)
+                for (int k = tid; k < nc; k += kTrainThreads) sm.e[k] = __ldcg(dY + c0 + k);
+            asm volatile("cp.async.commit_group;\ncp.async.wait_group 0;" ::: "memory");
+            __syncthreads();
+            if (tid < 256) {
+                const float *dz = sm.dZ[m] + j, *a = sm.A[m] + r4;
+#pragma unroll 8
+                for (int s = 0; s < nc; ++s) {
+                    const float d = dz[s * kW];
+                    const float4 h = *(const float4 *)(a + s * kRow);
+                    g[0] = fmaf(h.x, d, g[0]);
+                    g[1] = fmaf(h.y, d, g[1]);
+                    g[2] = fmaf(h.z, d, g[2]);
+                    g[3] = fmaf(h.w, d, g[3]);
+                }
+            } else if (nk) {
+                if (c == 0) {
+                    const float *dz = sm.dZ[e >> 6] + (e & 63);
+#pragma unroll 8
+                    for (int s = 0; s < nc; ++s) g[0] += dz[s * kW];
+                } else if (c == 1) {
+                    const float *dz = sm.E + (e & 63);
+                    const int i = e >> 6;   // input of W1, kIn: the bias
+                    if (i < kIn) {
+#pragma unroll 8
+                        for (int s = 0; s < nc; ++s)
+                            g[0] = fmaf(sm.e[s * kIn + i], dz[s * kW], g[0]);
+                    } else {
+#pragma unroll 8
+                        for (int s = 0; s < nc; ++s) g[0] += dz[s * kW];
+                    }
+                } else if (e < kW) {
+#pragma unroll 8
+                    for (int s = 0; s < nc; ++s) g[0] = fmaf(sm.E[s * kW + e], sm.e[s], g[0]);
+                } else {
+#pragma unroll 8
+                    for (int s = 0; s < nc; ++s) g[0] += sm.e[s];
+                }
+            }
+            __syncthreads();
+        }
+        const AdamStep adam(lr, b1, b2, eps, t0 + ep + 1);
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            if (q < nk) {
+                adam(p[q], mom[q], var[q], g[q]);
+                store_all(at + q * kWs, p[q]);
+            }
+        cluster_sync();
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+        if (q < nk) {
+            P[first + q * kW] = p[q];
+            M[first + q * kW] = mom[q];
+            V[first + q * kW] = var[q];
+        }
+    if (c == 0 && tid == 0) *t = t0 + epochs;
 }
 
 __global__ void to_double_kernel(int n, const float *a, double *b)
@@ -223,9 +514,6 @@ struct llr_mlp {
     int *t = nullptr;
     double *norm = nullptr;   // mean[3], std[3]
     Buffers buf;
-    cudaGraphExec_t graph = nullptr;
-    int graph_n = -1;
-    float graph_lr = 0.0f;
 };
 
 namespace {
@@ -264,11 +552,6 @@ int ensure_buffers(llr_mlp *h, int n)
     MLP_CUDA(cudaMalloc(&b.raw, sizeof(double) * 4 * (size_t)n));
     MLP_CUDA(cudaMalloc(&b.loss, sizeof(double)));
     b.n = n;
-    if (h->graph) {
-        cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-        h->graph_n = -1;
-    }
     return LLR_OK;
 }
 
@@ -324,15 +607,6 @@ void enqueue_backward(llr_mlp *h, int n)
         n, kW, kW, b.dZ + L2, h->P + kOffW2, b.Z + L1, b.dZ + L1);
     linear_bwd_weight_kernel<<<blocks(kIn * kW + kW), 256, 0, h->stream>>>(
         n, kIn, kW, b.X, b.dZ + L1, h->G + kOffW1, h->G + kOffB1);
-}
-
-void enqueue_epoch(llr_mlp *h, int n, float lr)
-{
-    enqueue_forward(h, n);
-    enqueue_backward(h, n);
-    step_count_kernel<<<1, 1, 0, h->stream>>>(h->t);
-    adam_kernel<<<blocks(kNParams), 256, 0, h->stream>>>(kNParams, h->P, h->G, h->M, h->V, h->t,
-                                                         lr, 0.9f, 0.999f, 1e-8f);
 }
 
 }  // namespace
@@ -482,33 +756,15 @@ int llr_mlp_fit(llr_mlp_handle h, int n, const double *L, const double *e6v, con
                                                        h->norm + 3);
     enqueue_features(h, n);
     MLP_CUDA(cudaGetLastError());
-    // one epoch captured once as a CUDA graph, replayed `epochs` times
-    if (!h->graph || h->graph_n != n || h->graph_lr != (float)lr) {
-        if (h->graph) cudaGraphExecDestroy(h->graph);
-        h->graph = nullptr;
-        cudaStream_t cap = h->stream;
-        bool own = false;
-        if (!cap) {
-            MLP_CUDA(cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking));
-            own = true;
-            MLP_CUDA(cudaDeviceSynchronize());
-        }
-        cudaStream_t keep = h->stream;
-        h->stream = cap;
-        cudaGraph_t g;
-        MLP_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
-        enqueue_epoch(h, n, (float)lr);
-        cudaError_t ce = cudaStreamEndCapture(cap, &g);
-        h->stream = keep;
-        if (own) cudaStreamDestroy(cap);
-        MLP_CUDA(ce);
-        ce = cudaGraphInstantiate(&h->graph, g, 0);
-        cudaGraphDestroy(g);
-        MLP_CUDA(ce);
-        h->graph_n = n;
-        h->graph_lr = (float)lr;
+    if (epochs > 0) {
+        Buffers &b = h->buf;
+        MLP_CUDA(cudaFuncSetAttribute(train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                      (int)sizeof(TrainSmem)));
+        train_kernel<<<kCtas, kTrainThreads, sizeof(TrainSmem), h->stream>>>(
+            n, epochs, b.X, b.T, b.A, b.dZ, b.dY, h->P, h->M, h->V, h->t, (float)lr,
+            0.9f, 0.999f, 1e-8f);
+        MLP_CUDA(cudaGetLastError());
     }
-    for (int ep = 0; ep < epochs; ++ep) MLP_CUDA(cudaGraphLaunch(h->graph, h->stream));
     // loss of the final parameters
     enqueue_forward(h, n);
     loss_grad_kernel<<<1, 256, 0, h->stream>>>(n, h->buf.Y, h->buf.T, h->buf.dY, h->buf.loss);
@@ -526,7 +782,6 @@ int llr_mlp_destroy(llr_mlp_handle h)
     if (!h) return LLR_OK;
     if (h->stream) cudaStreamSynchronize(h->stream);
     else cudaDeviceSynchronize();
-    if (h->graph) cudaGraphExecDestroy(h->graph);
     Buffers &b = h->buf;
     cudaFree(b.X); cudaFree(b.Z); cudaFree(b.A); cudaFree(b.dZ); cudaFree(b.Y); cudaFree(b.dY);
     cudaFree(b.T); cudaFree(b.raw); cudaFree(b.loss);
