@@ -44,7 +44,7 @@ struct llr_ctx {
     // multicanonical weight: ln rho~ at the n + 1 edges, then the n slopes
     double *d_muca = nullptr;
     int muca_n = 0;
-    double muca_e0 = 0.0, muca_de = 0.0, muca_a0 = 0.0;
+    double muca_e0 = 0.0, muca_de = 0.0, muca_a0 = 0.0, muca_jump = 0.0;
     double *d_ehist = nullptr;       // energy history of llr_muca_sweep
     size_t ehist_cap = 0;
     // one captured Robbins-Monro step (memset, persistent kernel, step + 1)
@@ -94,6 +94,24 @@ llr::KernelArgs base_args(llr_handle h)
     a.max_L = h->max_L;
     a.slab_L = h->slab_L;
     return a;
+}
+
+// The multicanonical weight of a launch.
+void muca_args(llr_handle h, llr::KernelArgs &a)
+{
+    a.muca_lnr = h->d_muca;
+    a.muca_a = h->d_muca + h->muca_n + 1;
+    a.muca_n = h->muca_n;
+    a.muca_e0 = h->muca_e0;
+    a.muca_de = h->muca_de;
+    a.muca_a0 = h->muca_a0;
+    // beyond the energies a lattice can have, a clamped e0 makes the float32 form
+    // of the accept test unsure of everything (a NaN jump), and the exact one decides
+    const bool range = std::fabs(h->muca_e0) < 2.0e9;
+    a.muca_e0_fx = range ? std::llrint(h->muca_e0 * llr::kFx) : 0;
+    a.muca_de_f = (float)h->muca_de;
+    a.muca_inv_de = (float)(llr::kInvFx / h->muca_de);
+    a.muca_jump = range ? (float)h->muca_jump : std::nanf("");
 }
 
 // Launch the persistent kernel with the handle's shape; remember the shape.
@@ -330,12 +348,7 @@ int llr_pass(llr_handle h, int kind, const double *a_host, int class_mask)
     a.pass_kind = kind;
     a.class_mask = class_mask;
     if (kind == 2) {
-        a.muca_lnr = h->d_muca;
-        a.muca_a = h->d_muca + h->muca_n + 1;
-        a.muca_n = h->muca_n;
-        a.muca_e0 = h->muca_e0;
-        a.muca_de = h->muca_de;
-        a.muca_a0 = h->muca_a0;
+        muca_args(h, a);
     }
     if (a_host) {
         LLR_CUDA(cudaMemcpyAsync(h->d_a, a_host, sizeof(double) * (size_t)h->n,
@@ -538,6 +551,9 @@ int llr_set_muca_weight(llr_handle h, int n, double e0, double de, const double 
     h->muca_e0 = e0;
     h->muca_de = de;
     h->muca_a0 = a0;
+    h->muca_jump = 0.0;
+    for (int k = 0; k + 1 < n; ++k)
+        h->muca_jump = std::max(h->muca_jump, std::fabs(a_host[k + 1] - a_host[k]) * de);
     return LLR_OK;
 }
 
@@ -560,12 +576,7 @@ int llr_muca_sweep(llr_handle h, int n_sweeps, double *E_out)
     a.program = llr::kProgMuca;
     a.n_therm = 0;
     a.n_meas = n_sweeps;
-    a.muca_lnr = h->d_muca;
-    a.muca_a = h->d_muca + h->muca_n + 1;
-    a.muca_n = h->muca_n;
-    a.muca_e0 = h->muca_e0;
-    a.muca_de = h->muca_de;
-    a.muca_a0 = h->muca_a0;
+    muca_args(h, a);
     a.e_hist = E_out ? h->d_ehist : nullptr;
     LLR_CUDA(launch(h, a, h->stream));
     if (E_out)

@@ -428,11 +428,12 @@ struct Stage {
     long long *P;      // prefix sums of dE over the group, to each of its links
     long long *d;      // dE of each link
     float2 *thn;       // the proposals
+    float2 *u;         // multicanonical pass: the uniforms of the accept test
     uint2 *acc;        // written by the consumer: links 0-31 / 32-63 accepted
 };
 
 // Bytes of a stage per group: a multiple of 16, so every stage's P is aligned.
-constexpr int kStageGroupBytes = 64 * 20 + 16;
+constexpr int kStageGroupBytes = 64 * 24 + 16;
 
 __device__ __forceinline__ Stage stage_at(char *base, int groups, int s)
 {
@@ -441,7 +442,8 @@ __device__ __forceinline__ Stage stage_at(char *base, int groups, int s)
     g.P = (long long *)p;
     g.d = (long long *)(p + groups * 512);
     g.thn = (float2 *)(p + groups * 1024);
-    g.acc = (uint2 *)(p + groups * 1280);
+    g.u = (float2 *)(p + groups * 1280);
+    g.acc = (uint2 *)(p + groups * 1536);
     return g;
 }
 
@@ -472,7 +474,7 @@ struct Smem {
 //
 // The team's and the lattice's constants are read from shared memory where they
 // are used: kept in registers across the loop they would be spilled.
-template <int MU, bool ROW, bool RES, bool FAST>
+template <int MU, bool ROW, bool RES, bool MUCA, bool FAST>
 __device__ __noinline__ void produce_class(Smem &sm, int slot, int pw, float *th_, int lat_off,
                                            int p, uint32_t tag)
 {
@@ -608,6 +610,16 @@ __device__ __noinline__ void produce_class(Smem &sm, int slot, int pw, float *th
             flush(stg, ch - D);
         }
         stg.thn[pt] = thn;
+        if (MUCA && valid) {   // the uniforms of the links' accept tests
+            int x[4];
+            const uint32_t base = (uint32_t)MU * 2u * (uint32_t)st.half;
+            const uint32_t l0 = base + (uint32_t)decode_half(h, p, st.L, st.magic, x);
+            const uint32_t l1 =
+                ROW ? l0 + 2u : base + (uint32_t)decode_half(h + 1, p, st.L, st.magic, x);
+            stg.u[pt] = make_float2(
+                u01(philox4x32_10(l0, st.sweep, kTagMuca, 0u, st.key0, st.key1).x),
+                u01(philox4x32_10(l1, st.sweep, kTagMuca, 0u, st.key0, st.key1).x));
+        }
         ((longlong2 *)stg.P)[pt] = make_longlong2(P - d1, P);
         ((longlong2 *)stg.d)[pt] = make_longlong2(d0, d1);
         bar_arrive(bar, NT);
@@ -975,6 +987,41 @@ __device__ __forceinline__ double muca_lnrho(const KernelArgs &a, long long E_fx
     return a.muca_lnr[k] + a.muca_a[k] * (E - (a.muca_e0 + (double)k * a.muca_de));
 }
 
+// The multicanonical accept test of one link: whether a move of dE d (fixed point)
+// from the energy E is refused, i.e. not u < exp(x),
+// x = a0 d - (ln rho~(E + d) - ln rho~(E)).
+__device__ __forceinline__ bool muca_refuses(const KernelArgs &a, long long E, long long d, float u)
+{
+    const double x = a.muca_a0 * ((double)d * kInvFx) - (muca_lnrho(a, E + d) - muca_lnrho(a, E));
+    return !((double)u < exp(x));
+}
+
+// The same in float32 where that is sure of the outcome: sure = false where u is
+// within the error of exp(x).  E and E + d lie in interval k0 and k1 of the table
+// (q0, q1 in units of its intervals); with at most one edge between them
+//   x = (a0 - a[k0]) d - (a[k1] - a[k0]) (E + d - that edge).
+// ln rho~ is continuous, so an energy rounded across an edge costs no more than
+// the rounding of q (at most 3e-7 |q|) times de times the jump of the slope,
+// which muca_jump bounds.  FP64 runs at 1/73 of the float32 rate: the exact test
+// of every link made the deciding warp the pass's bound.
+__device__ __forceinline__ bool muca_refuses_fast(const KernelArgs &a, long long E, long long d,
+                                                  float u, bool &sure)
+{
+    const float inv = a.muca_inv_de;
+    const float q0 = (float)(E - a.muca_e0_fx) * inv, q1 = (float)(E + d - a.muca_e0_fx) * inv;
+    const int top = a.muca_n - 1;
+    const int k0 = min(max((int)floorf(q0), 0), top), k1 = min(max((int)floorf(q1), 0), top);
+    const double s0 = a.muca_a[k0];
+    const float df = (float)d * (float)kInvFx;
+    float x = (float)(a.muca_a0 - s0) * df;
+    if (k1 != k0) x -= (float)(a.muca_a[k1] - s0) * ((q1 - (float)max(k0, k1)) * a.muca_de_f);
+    const float err = 1e-6f * (a.muca_jump * (1.0f + fabsf(q0) + fabsf(q1)) + fabsf(x)) + 1e-7f;
+    const float e = __expf(x);
+    sure = abs(k1 - k0) <= 1 &&
+           fabsf(u - e) > e * (2.0f * err + 4e-6f * (1.0f + fabsf(x))) + 1e-7f;
+    return !(u < e);
+}
+
 // Consumer side of a multicanonical heat-bath class (Sec. 2.6): the links
 // are taken in link order by Metropolis-Hastings for the weight 1/rho~ with
 // the proposal at slope a0, i.e. with probability
@@ -984,47 +1031,34 @@ __device__ __forceinline__ double muca_lnrho(const KernelArgs &a, long long E_fx
 // link is decided as if all earlier ones were taken; the first refusal (one
 // ballot) fixes the links before it, its dE is dropped and the rest is decided
 // again.  Blocks of one link.
-__device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb, int mu, int p,
+__device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb,
                                                 const KernelArgs &args)
 {
     const int lane = threadIdx.x & 31, nwp = hb.nw - 1, CH = nwp * 64, D = hb.D, NT = hb.nw * 32;
-    const int L = st.L, half = st.half, nchunk = (half + CH - 1) / CH;
-    const uint32_t magic = st.magic, V = 2u * (uint32_t)half;
-    const uint32_t k0 = st.key0, k1 = st.key1, sweep = st.sweep;
-    const double a0 = args.muca_a0;
+    const int half = st.half, nchunk = (half + CH - 1) / CH;
     long long E = st.E_fx;
     for (int ch = 0; ch < nchunk; ++ch) {
         const int s = ch & (D - 1);
         bar_sync(hb.full + s, NT);
         const Stage stg = stage_at((char *)(g_dyn + hb.ring), nwp, s);
         for (int g = 0; g < 2 * nwp; ++g) {
-            const int h = ch * CH + g * 32 + lane, nval = min(32, half - (ch * CH + g * 32));
+            const int nval = min(32, half - (ch * CH + g * 32));
             if (nval <= 0) break;
             const long long *Pg = stg.P + g * 32;
             // the prefix sums run over 64 links: take the first half's out of the second's
             const long long off = (g & 1) ? Pg[-1] : 0ll;
             const long long Pk = Pg[lane] - off, dk = stg.d[g * 32 + lane];
-            const unsigned em = nval >= 32 ? kFull : (1u << nval) - 1u;
+            const float u = ((const float *)stg.u)[g * 32 + lane];
+            const unsigned em = kFull >> (32 - nval);
             unsigned rem = em, acc = 0u;
-            double u = 1.0;
-            if ((em >> lane) & 1u) {
-                int x[4];
-                const int site = decode_half(h, p, L, magic, x);
-                const U4 w = philox4x32_10((uint32_t)mu * V + (uint32_t)site, sweep, kTagMuca, 0u,
-                                           k0, k1);
-                u = (double)u01(w.x);
-            }
             long long R = 0;
             while (rem) {
-                const bool mine = (rem >> lane) & 1u;
-                bool refuse = false;
-                if (mine) {
-                    const long long Eb = E + (Pk - dk) - R;
-                    const double xk =
-                        a0 * ((double)dk * kInvFx) - (muca_lnrho(args, Eb + dk) - muca_lnrho(args, Eb));
-                    refuse = !(u < exp(xk));
-                }
-                const unsigned vm = __ballot_sync(kFull, refuse);
+                const long long Eb = E + (Pk - dk) - R;
+                bool sure;
+                bool refuse = muca_refuses_fast(args, Eb, dk, u, sure);
+                if (!sure && ((rem >> lane) & 1u)) refuse = muca_refuses(args, Eb, dk, u);
+                __syncwarp();
+                const unsigned vm = __ballot_sync(kFull, refuse) & rem;
                 if (vm == 0u) {
                     acc |= rem;
                     break;
@@ -1470,22 +1504,35 @@ struct Phase {
 };
 
 // One class of a heat-bath pass by the team's producers.
-template <int MU, bool FAST>
+template <int MU, bool MUCA, bool FAST>
 __device__ __forceinline__ void produce(Smem &sm, const Phase &ph, int slot, int pw, float *th,
                                         int p, uint32_t tag)
 {
-    const bool row = (sm.st[slot].L & 3) == 0;
+    // the accurate sine / cosine dominates without fast math: one form for any L
+    const bool row = FAST && (sm.st[slot].L & 3) == 0;
     const int off = slot * ph.slab;
     if (ph.res) {
         if (row)
-            produce_class<MU, true, true, FAST>(sm, slot, pw, th, off, p, tag);
+            produce_class<MU, FAST, true, MUCA, FAST>(sm, slot, pw, th, off, p, tag);
         else
-            produce_class<MU, false, true, FAST>(sm, slot, pw, th, off, p, tag);
+            produce_class<MU, false, true, MUCA, FAST>(sm, slot, pw, th, off, p, tag);
     } else {
         if (row)
-            produce_class<MU, true, false, FAST>(sm, slot, pw, th, off, p, tag);
+            produce_class<MU, FAST, false, MUCA, FAST>(sm, slot, pw, th, off, p, tag);
         else
-            produce_class<MU, false, false, FAST>(sm, slot, pw, th, off, p, tag);
+            produce_class<MU, false, false, MUCA, FAST>(sm, slot, pw, th, off, p, tag);
+    }
+}
+
+template <bool MUCA, bool FAST>
+__device__ __forceinline__ void produce(Smem &sm, const Phase &ph, int slot, int pw, float *th,
+                                        int mu, int p, uint32_t tag)
+{
+    switch (mu) {
+        case 0: produce<0, MUCA, FAST>(sm, ph, slot, pw, th, p, tag); break;
+        case 1: produce<1, MUCA, FAST>(sm, ph, slot, pw, th, p, tag); break;
+        case 2: produce<2, MUCA, FAST>(sm, ph, slot, pw, th, p, tag); break;
+        default: produce<3, MUCA, FAST>(sm, ph, slot, pw, th, p, tag); break;
     }
 }
 
@@ -1524,16 +1571,14 @@ __device__ __noinline__ void heatbath_phase(Smem &sm, const Phase &ph, const Ker
                 const int mu = cls >> 1, p = cls & 1;
                 if (consumer) {
                     if (kind == 2)
-                        consume_class_muca(st, sm.hb[slot], mu, p, args);
+                        consume_class_muca(st, sm.hb[slot], args);
                     else
                         consume_class(st, sm.hb[slot], B);
                 } else {
-                    switch (mu) {
-                        case 0: produce<0, FAST>(sm, ph, slot, pw, th, p, tag); break;
-                        case 1: produce<1, FAST>(sm, ph, slot, pw, th, p, tag); break;
-                        case 2: produce<2, FAST>(sm, ph, slot, pw, th, p, tag); break;
-                        default: produce<3, FAST>(sm, ph, slot, pw, th, p, tag); break;
-                    }
+                    if (kind == 2)
+                        produce<true, FAST>(sm, ph, slot, pw, th, mu, p, tag);
+                    else
+                        produce<false, FAST>(sm, ph, slot, pw, th, mu, p, tag);
                 }
                 // the next class reads the angles written here
                 bar_sync(sm.hb[slot].full, nw * 32);

@@ -56,6 +56,10 @@ struct KernelArgs {
     const double *muca_a;
     int muca_n;
     double muca_e0, muca_de, muca_a0;
+    // the same for the float32 form of the accept test: e0 in fixed point, de, 1 / de
+    // per unit of the fixed point, and de times the largest jump of the slopes
+    long long muca_e0_fx;
+    float muca_de_f, muca_inv_de, muca_jump;
     double *e_hist;       // kProgMuca, nullable: e_hist[sweep * n_lat + lattice] = E
     int max_L;            // largest L of the handle's lattices
     int slab_L;           // largest L <= 24 of them (0: none): shared-memory slabs
