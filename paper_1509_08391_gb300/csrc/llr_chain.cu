@@ -1089,17 +1089,39 @@ __device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb,
 // A thread reflects two links at a time, so the index arithmetic and (with
 // rows of even length, ROW) the loads serve two: links k, k + 1 of one x0 row
 // (one 8-byte load each), or, where the half row L / 2 is odd, the links at x2
-// and x2 + L / 2.  Threads map to (x2 plane, x1, k) and step over planes, so
-// only x2 changes from one unit of a thread to the next.
+// and x2 + L / 2.  With ROW threads map to (x2 plane, x1, k) and step over planes,
+// so only x2 changes from one unit of a thread to the next; planes of odd half
+// rows fill a team's threads badly (196 of 256 at L = 14, four iterations where
+// the units need three: 0.55 against 0.47 ms a pass of 456 lattices), so there a
+// thread takes every nt-th unit.
 // ---------------------------------------------------------------------------
 constexpr int kSlabMaxL = 24;       // 16 * 24^3 bytes = 216 KB
 constexpr int kResidentMaxL = 10;   // 16 * 10^4 bytes = 156 KB
 
 struct SlabGeo {
     int L, Lh, S1, S, half, SH;   // side, half row, plane, slab, class array, half slab (floats)
-    int F, nit, planes;           // planes per iteration, iterations, planes in all
-    int x2, h;                    // the thread's first plane (beyond all: idle) and link
+    int step, nit, planes;        // planes (ROW) or units per iteration, iterations, planes in all
+    uint32_t mL, mLh;             // magic divisors of the units (mLh = 0: by one)
+    int x2, h;                    // the unit's plane (beyond all: idle) and link
     int d1p, d1m, rdn, rup, par;  // x1 neighbours, x0 wraps, parity of x1
+
+    // the x1, k part of a unit's place
+    __device__ __forceinline__ void place(bool row, int x1, int k)
+    {
+        h = x2 * S1 + x1 * Lh + k;
+        d1p = x1 == L - 1 ? Lh - S1 : Lh;
+        d1m = x1 == 0 ? S1 - Lh : -Lh;
+        rdn = k == 0 ? Lh - 1 : -1;
+        rup = row ? (k + 2 == Lh ? 2 - Lh : 2) : (k == Lh - 1 ? 1 - Lh : 1);
+        par = x1 & 1;
+    }
+    // unit u of a slab's S / 2 (not ROW)
+    __device__ __forceinline__ void unit(int u)
+    {
+        const int r = mLh ? (int)__umulhi((uint32_t)u, mLh) : u;
+        x2 = (int)__umulhi((uint32_t)r, mL);
+        place(false, r - x2 * L, u - r * Lh);
+    }
 };
 
 template <bool ROW>
@@ -1113,19 +1135,22 @@ __device__ __forceinline__ SlabGeo slab_geo(int L, int nt, int tid)
     g.half = g.S * L;
     g.SH = g.S >> 1;
     g.planes = ROW ? L : g.Lh;
-    const int pr = ROW ? L >> 2 : g.Lh, pp = pr * L;   // pairs per row, per plane
-    int f = nt / pp;
-    f = f > g.planes ? g.planes : (f < 1 ? 1 : f);
-    g.nit = (g.planes + f - 1) / f;
-    g.F = (g.planes + g.nit - 1) / g.nit;              // the same number of iterations, evenly
-    const int pl = tid / pp, r = tid - pl * pp, x1 = r / pr, k = (r - x1 * pr) * (ROW ? 2 : 1);
-    g.x2 = pl < g.F ? pl : 1 << 20;
-    g.h = pl * g.S1 + x1 * g.Lh + k;
-    g.d1p = x1 == L - 1 ? -(L - 1) * g.Lh : g.Lh;
-    g.d1m = x1 == 0 ? (L - 1) * g.Lh : -g.Lh;
-    g.rdn = k == 0 ? g.Lh - 1 : -1;
-    g.rup = ROW ? (k + 2 == g.Lh ? 2 - g.Lh : 2) : (k == g.Lh - 1 ? 1 - g.Lh : 1);
-    g.par = x1 & 1;
+    g.mL = 0xffffffffu / (uint32_t)L + 1u;
+    g.mLh = g.Lh > 1 ? 0xffffffffu / (uint32_t)g.Lh + 1u : 0u;
+    if (ROW) {
+        const int pr = L >> 2, pp = pr * L;   // pairs per row, per plane
+        int f = nt / pp;
+        f = f > L ? L : (f < 1 ? 1 : f);
+        g.nit = (L + f - 1) / f;
+        g.step = (L + g.nit - 1) / g.nit;     // the same number of iterations, evenly
+        const int pl = tid / pp, r = tid - pl * pp, x1 = r / pr;
+        g.x2 = pl;
+        g.place(true, x1, 2 * (r - x1 * pr));
+        if (pl >= g.step) g.x2 = 1 << 20;
+    } else {
+        g.step = nt;
+        g.nit = (g.SH + nt - 1) / nt;
+    }
     return g;
 }
 
@@ -1289,18 +1314,26 @@ __device__ __forceinline__ void reflect_pair(const SlabGeo &g, int x2, int h, in
 
 // The two classes of direction MU in one slab.
 template <int MU, bool ROW, bool FAST>
-__device__ __forceinline__ void reflect_dir(const SlabGeo &g, const Team &tm_, int t, int mask,
+__device__ __forceinline__ void reflect_dir(SlabGeo &g, const Team &tm_, int t, int mask,
                                             float *sl, float *th, int tc, int tp, int tm)
 {
 #pragma unroll 1
     for (int p = 0; p < 2; ++p) {
         if (!((mask >> (2 * MU + p)) & 1)) continue;
-        int x2 = g.x2, h = g.h;
+        if (ROW) {
+            int x2 = g.x2, h = g.h;
 #pragma unroll 1
-        for (int i = 0; i < g.nit; ++i) {
-            if (x2 < g.planes) reflect_pair<MU, ROW, FAST>(g, x2, h, p, t, sl, th, tc, tp, tm);
-            x2 += g.F;
-            h += g.F * g.S1;
+            for (int i = 0; i < g.nit; ++i) {
+                if (x2 < g.planes) reflect_pair<MU, ROW, FAST>(g, x2, h, p, t, sl, th, tc, tp, tm);
+                x2 += g.step;
+                h += g.step * g.S1;
+            }
+        } else {
+#pragma unroll 1
+            for (int u = tm_.tid; u < g.SH; u += g.step) {
+                g.unit(u);
+                reflect_pair<MU, ROW, FAST>(g, g.x2, g.h, p, t, sl, th, tc, tp, tm);
+            }
         }
         tm_.sync();   // the next class reads the angles written here
     }
@@ -1315,8 +1348,8 @@ __device__ __noinline__ void reflect_slabs(Team team, int L_, float *th_, int sl
     const int L = uniform(L_);
     float *th = (float *)__shfl_sync(kFull, (unsigned long long)th_, 0);
     float *sl = g_dyn + uniform(slab_off);
-    const SlabGeo g = slab_geo<ROW>(L, team.nt, team.tid);
-    const int need = (g.F * (ROW ? L >> 2 : g.Lh) * L + 31) >> 5;
+    SlabGeo g = slab_geo<ROW>(L, team.nt, team.tid);
+    const int need = ((ROW ? g.step * (L >> 2) * L : min(g.SH, g.step)) + 31) >> 5;
     if (team.w >= need) return;
     team.nw = need < team.nw ? need : team.nw;
     team.nt = team.nw * 32;
@@ -1433,9 +1466,9 @@ __device__ __noinline__ void overrelax_pass(Smem &sm, int slot, const Team &team
     const long long bound = (long long)B * kOrDeltaMaxFx;
     const long long E = st.E_fx;   // the running energy; overrelaxation leaves it
     const bool free_all = E < lo || E > hi || (E - bound >= lo && E + bound <= hi);
-    // the pairs of one unit plane (L^2 / 4, or L^2 / 2 for odd half rows) need a thread each
+    // the L^2 / 4 pairs of a plane need a thread each
     const bool in_slabs =
-        free_all && (res || (L <= kSlabMaxL && L * L <= ((L & 3) == 0 ? 4 : 2) * team.nt));
+        free_all && (res || (L <= kSlabMaxL && ((L & 3) != 0 || L * L <= 4 * team.nt)));
     if (in_slabs && res) {
         switch (L) {
             case 2: reflect_lattice<2, FAST>(team, slab_off, class_mask); break;
@@ -1641,108 +1674,121 @@ __device__ __noinline__ void overrelax_phase(Smem &sm, const Phase &ph, const Ke
 //   result by up to 5e-9); then cos(rh + rl) = cos rh - rl sin rh and
 //   sin(rh + rl) = sin rh + rl cos rh (plus the rl^2 terms), and
 //   cos x = cos r, -sin r, -cos r, sin r for k = 0, 1, 2, 3 (mod 4).
-__device__ __forceinline__ float cos_unbiased(float hi, float lo)
+// Two angles at a time in packed arithmetic.
+__device__ __forceinline__ float2 cos_unbiased2(float2 hi, float2 lo)
 {
-    const float k = rintf(hi * 0.636619747f);
-    const float rh = fmaf(-k, 1.5707950592041016f, hi);
-    float rl = fmaf(-k, 1.2675900507019833e-06f, lo);
-    rl = fmaf(-k, 7.4435477313145038e-13f, rl);
-    const float z = rh * rh;
+    const float2 k = make_float2(rintf(hi.x * 0.636619747f), rintf(hi.y * 0.636619747f));
+    const float2 nk = make_float2(-k.x, -k.y);
+    const float2 rh = fma2(nk, both(1.5707950592041016f), hi);
+    float2 rl = fma2(nk, both(1.2675900507019833e-06f), lo);
+    rl = fma2(nk, both(7.4435477313145038e-13f), rl);
+    const float2 z = mul2(rh, rh);
     // cos rh = 1 - z/2 + z^2/4! - ... - z^7/14!
-    float c = -1.147074536e-11f;
-    c = fmaf(c, z, 2.087675588e-09f);
-    c = fmaf(c, z, -2.755731998e-07f);
-    c = fmaf(c, z, 2.480158764e-05f);
-    c = fmaf(c, z, -1.388888923e-03f);
-    c = fmaf(c, z, -1.241763470e-09f);   // 1/4! = 4.166666791e-02 - 1.241763470e-09
-    c += 4.166666791e-02f;
-    c = fmaf(c, z, -0.5f);
-    c = fmaf(c, z, 1.0f);
+    float2 c = both(-1.147074536e-11f);
+    c = fma2(c, z, both(2.087675588e-09f));
+    c = fma2(c, z, both(-2.755731998e-07f));
+    c = fma2(c, z, both(2.480158764e-05f));
+    c = fma2(c, z, both(-1.388888923e-03f));
+    c = fma2(c, z, both(-1.241763470e-09f));   // 1/4! = 4.166666791e-02 - 1.241763470e-09
+    c = add2(c, both(4.166666791e-02f));
+    c = fma2(c, z, both(-0.5f));
+    c = fma2(c, z, both(1.0f));
     // sin rh = rh (1 - z/3! + z^2/5! - ... - z^7/15!)
-    float t = -7.647163610e-13f;
-    t = fmaf(t, z, 1.605904437e-10f);
-    t = fmaf(t, z, -2.505210794e-08f);
-    t = fmaf(t, z, 2.755731884e-06f);
-    t = fmaf(t, z, -1.984127011e-04f);
-    t = fmaf(t, z, -4.346172033e-10f);   // 1/5! = 8.333333768e-03 - 4.346172033e-10
-    t += 8.333333768e-03f;
-    t = fmaf(t, z, 4.967053879e-09f);    // 1/3! = 1.666666716e-01 - 4.967053879e-09
-    t -= 1.666666716e-01f;
-    t = rh * fmaf(t, z, 1.0f);
+    float2 t = both(-7.647163610e-13f);
+    t = fma2(t, z, both(1.605904437e-10f));
+    t = fma2(t, z, both(-2.505210794e-08f));
+    t = fma2(t, z, both(2.755731884e-06f));
+    t = fma2(t, z, both(-1.984127011e-04f));
+    t = fma2(t, z, both(-4.346172033e-10f));   // 1/5! = 8.333333768e-03 - 4.346172033e-10
+    t = add2(t, both(8.333333768e-03f));
+    t = fma2(t, z, both(4.967053879e-09f));    // 1/3! = 1.666666716e-01 - 4.967053879e-09
+    t = sub2(t, both(1.666666716e-01f));
+    t = mul2(rh, fma2(t, z, both(1.0f)));
     // cos(rh + rl), sin(rh + rl) to second order in rl (|rl| <= 1e-5: the
     // dropped -rl^2/2 alone would bias cos by up to -5e-11); the small terms
     // are summed first, so the correction is not rounded away
-    const float h = 0.5f * rl * rl;
-    const float cr = c - fmaf(t, rl, c * h);
-    const float sr = t + fmaf(c, rl, -t * h);
-    const int q = (int)k & 3;
-    const float v = (q & 1) ? sr : cr;
-    return (q == 1 || q == 2) ? -v : v;
+    const float2 h = mul2(mul2(both(0.5f), rl), rl);
+    const float2 cr = sub2(c, fma2(t, rl, mul2(c, h)));
+    const float2 sr = add2(t, fma2(c, rl, mul2(make_float2(-t.x, -t.y), h)));
+    auto pick = [](float kf, float cv, float sv) {
+        const int q = (int)kf & 3;
+        const float v = (q & 1) ? sv : cv;
+        return (q == 1 || q == 2) ? -v : v;
+    };
+    return make_float2(pick(k.x, cr.x, sr.x), pick(k.y, cr.y, sr.y));
 }
 
-__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2 &s, float2 &e)
 {
-    s = __fadd_rn(a, b);
-    const float bb = __fsub_rn(s, a);
-    e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, bb)), __fsub_rn(b, bb));
+    s = add2(a, b);
+    const float2 bb = sub2(s, a);
+    e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
 }
 
-// cos of the plaquette angle a + b - c - d of four float angles: the angle is
-// formed exactly as hi + lo and its cosine taken by cos_unbiased.
-__device__ __forceinline__ float plaquette_cos(float a, float b, float c, float d)
+// cos of the plaquette angles a + b - c - d of two plaquettes, in packed
+// arithmetic: each angle is formed exactly as hi + lo and its cosine taken by
+// cos_unbiased2.
+__device__ __forceinline__ float2 plaquette_cos2(float2 a, float2 b, float2 c, float2 d)
 {
-    float s1, e1, s2, e2, hi, e3;
-    two_sum(a, b, s1, e1);
-    two_sum(c, d, s2, e2);
-    two_sum(s1, -s2, hi, e3);
-    const float lo = (e1 - e2) + e3;
-    return cos_unbiased(hi, lo);
+    float2 s1, e1, s2, e2, hi, e3;
+    two_sum2(a, b, s1, e1);
+    two_sum2(c, d, s2, e2);
+    two_sum2(s1, make_float2(-s2.x, -s2.y), hi, e3);
+    return cos_unbiased2(hi, add2(sub2(e1, e2), e3));
 }
 
 // Fresh energy of the team's lattice in fixed point: sum over the 6 V
-// plaquettes, exact int64 accumulation and reduction.  Valid in the team's thread 0.
+// plaquettes, exact int64 accumulation and reduction.  Two sites per thread (half
+// sites h, h + 1 of a parity), their plaquettes in packed arithmetic.  Valid in
+// the team's thread 0.
+template <bool ROW>
 __device__ __noinline__ long long fresh_energy_fx(const LatState &st_, const Team &team,
                                                   long long *red, const float *th)
 {
-    const int tid = team.tid, lane = tid & 31;
+    const int lane = team.tid & 31;
     const int L = uniform(st_.L), half = uniform(st_.half);
     const uint32_t magic = uniform(st_.magic);
-    const int V = 2 * half;
-    const int st[4] = {1, L, L * L, L * L * L};
     long long acc = 0;
-    for (int s = tid; s < V; s += team.nt) {
-        int x[4];
-        const int q = (int)__umulhi((uint32_t)s, magic);
-        x[0] = s - q * L;
-        const int q2 = (int)__umulhi((uint32_t)q, magic);
-        x[1] = q - q2 * L;
-        const int q3 = (int)__umulhi((uint32_t)q2, magic);
-        x[2] = q2 - q3 * L;
-        x[3] = q3;
-        const int p = (x[0] + x[1] + x[2] + x[3]) & 1;
-        const int hs = s >> 1;
-        float t[4];
-        int sp[4];
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p)
+#pragma unroll 1
+        for (int h = 2 * team.tid; h < half; h += 2 * team.nt) {
+            const LinkPair<ROW> n(h, p, L, magic);
+            const float *tp = th + p * half + h, *tq = th + (p ^ 1) * half + h;
+            auto up = [&](int nu, int mu) {   // theta_nu(x + mu)
+                const float *a = tq + 2 * nu * half;
+                if (ROW && mu > 0) return *(const float2 *)(a + n.up0[mu]);
+                return make_float2(a[n.up0[mu]], a[1 + n.up1[mu]]);
+            };
+            float2 t[4];
+            int hi = 0, lo = 0;
+            bool bad = false;
 #pragma unroll
-        for (int mu = 0; mu < 4; ++mu) {
-            t[mu] = th[(2 * mu + p) * half + hs];
-            sp[mu] = s + ((x[mu] == L - 1) ? -(L - 1) * st[mu] : st[mu]);
+            for (int mu = 0; mu < 4; ++mu) t[mu] = *(const float2 *)(tp + 2 * mu * half);
+#pragma unroll
+            for (int mu = 0; mu < 4; ++mu)
+#pragma unroll
+                for (int nu = mu + 1; nu < 4; ++nu) {
+                    const float2 v = plaquette_cos2(t[mu], up(nu, mu), up(mu, nu), t[nu]);
+                    int a, b;
+                    fx_parts(v.x, a, b);
+                    hi += a;
+                    lo += b;
+                    fx_parts(v.y, a, b);
+                    hi += a;
+                    lo += b;
+                    bad |= !(fabsf(v.x) < 512.0f) || !(fabsf(v.y) < 512.0f);
+                }
+            // 12 cosines: sums of parts within 32 bits.  Angles that are no numbers
+            // leave an energy that is none (the integer conversion's overflow value).
+            acc += bad ? -(1ll << 62) : (long long)hi * (1 << 20) + lo;
         }
-#pragma unroll
-        for (int mu = 0; mu < 4; ++mu)
-#pragma unroll
-            for (int nu = mu + 1; nu < 4; ++nu) {
-                const float tnu_xmu = th[(2 * nu + (p ^ 1)) * half + (sp[mu] >> 1)];
-                const float tmu_xnu = th[(2 * mu + (p ^ 1)) * half + (sp[nu] >> 1)];
-                acc += to_fx(plaquette_cos(t[mu], tnu_xmu, tmu_xnu, t[nu]));
-            }
-    }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
     if (lane == 0) red[team.w] = acc;
     team.sync();
     long long tot = 0;
-    if (tid == 0)
+    if (team.tid == 0)
         for (int w = 0; w < team.nw; ++w) tot += red[w];
     return tot;
 }
@@ -1758,7 +1804,10 @@ __device__ __noinline__ void energy_phase(Smem &sm, const Phase &ph, const Kerne
         const Team t{warp - slot * ph.tw, ph.tw, (int)threadIdx.x - slot * ph.tw * 32, ph.tw * 32,
                      1 + slot};
         LatState &st = sm.st[slot];
-        const long long fresh = fresh_energy_fx(st, t, sm.red + slot * ph.tw, ph.links(sm, args, slot));
+        const float *th = ph.links(sm, args, slot);
+        long long *red = sm.red + slot * ph.tw;
+        const long long fresh = (st.L & 3) == 0 ? fresh_energy_fx<true>(st, t, red, th)
+                                                : fresh_energy_fx<false>(st, t, red, th);
         if (t.tid == 0) {
             if (resync) {
                 const double drift = fabs((double)(st.E_fx - fresh) * kInvFx);

@@ -173,6 +173,21 @@ __device__ __forceinline__ long long to_fx(float v)
     return __float2ll_rn(v * 4294967296.0f);
 }
 
+// The same as a 2^20 + b, for |v| < 512.  The hardware's conversion to 64 bits
+// runs on the FP64 pipe (about 2 per clock and SM), which bounds a sum of cosines
+// (one resync of 456 lattices of L = 20: 1.17 ms against 0.99 ms), so it is done in
+// two float32 steps: a = the integer nearest v 2^12 (the low bits of
+// v 2^12 + 1.5 2^23), then b = the integer nearest the exact remainder times 2^32,
+// at most 2^19; a 2^20 is even, so ties stay ties to even.
+__device__ __forceinline__ void fx_parts(float v, int &a, int &b)
+{
+    constexpr float magic = 12582912.0f;   // 1.5 2^23, bits 0x4B400000
+    const float t = fmaf(v, 4096.0f, magic);
+    a = __float_as_int(t) - 0x4B400000;
+    const float r = fmaf(t - magic, -1.0f / 4096.0f, v);
+    b = __float_as_int(fmaf(r, 4294967296.0f, magic)) - 0x4B400000;
+}
+
 __device__ __forceinline__ long long dist_fx(long long E, long long lo, long long hi)
 {
     return E < lo ? lo - E : (E > hi ? E - hi : 0ll);
