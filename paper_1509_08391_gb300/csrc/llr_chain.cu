@@ -108,16 +108,19 @@ struct VonMises {
         const float z = __cosf(kPi * u1);
         const float f = __fdividef(fmaf(r, z, 1.0f), r + z);
         const float c = __fmul_rn(k, rm1 + (1.0f - f));
-        // second test ln(c / u2) + 1 - c >= 0, in base 2
-        return fmaf(c, 2.0f - c, -u2) > 0.0f ||
-               __log2f(c) - __log2f(u2) >= __fmul_rn(c - 1.0f, 1.4426950408889634f);
+        const bool quick = fmaf(c, 2.0f - c, -u2) > 0.0f;
+        // second test ln(c / u2) + 1 - c >= 0, in base 2 (no branch around it: the
+        // lanes of a warp rarely agree)
+        const bool full =
+            __log2f(c) - __log2f(u2) >= __fmul_rn(c - 1.0f, 1.4426950408889634f);
+        return quick | full;
     }
     // the two attempts of one Philox call: the first that accepts, its word 0
     __device__ __forceinline__ bool attempts(const U4 &w, uint32_t &w_acc) const
     {
         const bool first = accepts(w.x, w.y), second = accepts(w.z, w.w);
         w_acc = first ? w.x : w.z;
-        return first || second;
+        return first | second;
     }
     // (cos X, sin X) of the accepted attempt, without cancellation
     __device__ __forceinline__ void evaluate(float kappa, uint32_t w_acc, float &cX,
@@ -1580,7 +1583,10 @@ __device__ __noinline__ void heatbath_phase(Smem &sm, const Phase &ph, const Ker
         const int k = threadIdx.x;
         sm.acc_cnt[k] = 0ull;
         HbTeam &hb = sm.hb[k];
-        hb.nw = min(ph.tw, 1 + (sm.st[k].half + 63) / 64);   // no more producers than groups
+        // No more producers than groups.  With one lattice the deciding warp is the
+        // bound, so it has a quarter of the SM (a scheduler) to itself.
+        const int most = ph.teams == 1 ? kWarps / 4 * 3 + 1 : ph.tw;
+        hb.nw = min(most, 1 + (sm.st[k].half + 63) / 64);
         // the consumers of different teams on different quarters of the SM
         hb.cw = hb.nw - 1;
         for (int c = hb.nw - 1; c >= max(0, hb.nw - 4); --c)
@@ -1593,11 +1599,20 @@ __device__ __noinline__ void heatbath_phase(Smem &sm, const Phase &ph, const Ker
     const int warp = threadIdx.x >> 5, slot = warp / ph.tw, w = warp - slot * ph.tw;
     if (slot < ph.nl && sm.active[slot]) {
         LatState &st = sm.st[slot];
-        const int nw = sm.hb[slot].nw, cw = sm.hb[slot].cw;
-        if (w < nw) {
+        const int nw = sm.hb[slot].nw;
+        // consumer or not, and the rank among the producers (nw - 1 of them)
+        bool consumer;
+        int pw;
+        if (ph.teams == 1) {
+            consumer = w == kWarps - 1;
+            pw = (w & 3) == 3 ? nw : w / 4 * 3 + (w & 3);
+        } else {
+            const int cw = sm.hb[slot].cw;
+            consumer = w == cw;
+            pw = w - (w > cw ? 1 : 0);
+        }
+        if (consumer || pw < nw - 1) {
             float *th = args.theta + st.off;
-            const bool consumer = w == cw;
-            const int pw = w - (w > cw ? 1 : 0);   // rank among the producers
 #pragma unroll 1
             for (int cls = 0; cls < 8; ++cls) {
                 if (!((class_mask >> cls) & 1)) continue;
