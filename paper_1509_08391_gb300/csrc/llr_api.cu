@@ -840,6 +840,8 @@ struct MucaSamples {
     long long ns = 0;
     int gx = 1;
     double shift = 0.0;
+    double reach = 0.0, lr_reach = 0.0;   // bounds of |E - shift| and |ln rho~| over the samples
+    double *tab = nullptr;
     double *E = nullptr, *lr = nullptr, *beta = nullptr, *part = nullptr, *E1 = nullptr,
            *E2 = nullptr, *var = nullptr;
 };
@@ -852,6 +854,15 @@ int muca_samples_init(MucaSamples &w, long long ns, const double *E, int n, doub
         return fail(LLR_ERR_ARG, "need n >= 1 finite slopes, finite e0 and de > 0");
     for (long long i = 0; i < ns; ++i)
         if (!std::isfinite(E[i])) return fail(LLR_ERR_ARG, "non-finite sample " + std::to_string(i));
+    // four running maxima, so that one comparison does not wait for another
+    double reach[4] = {0.0, 0.0, 0.0, 0.0};
+    for (long long i = 0; i + 3 < ns; i += 4)
+        for (int k = 0; k < 4; ++k) {
+            const double v = std::fabs(E[i + k] - e0);
+            reach[k] = v > reach[k] ? v : reach[k];
+        }
+    for (long long i = ns & ~3ll; i < ns; ++i) reach[0] = std::max(reach[0], std::fabs(E[i] - e0));
+    w.reach = std::max(std::max(reach[0], reach[1]), std::max(reach[2], reach[3]));
     std::vector<double> tab;
     if (int r = muca_table(n, de, a, tab)) return r;
     int dev = 0, sms = 1;
@@ -863,12 +874,16 @@ int muca_samples_init(MucaSamples &w, long long ns, const double *E, int n, doub
     w.ns = ns;
     w.shift = e0;
     const int nb = MucaSamples::kBetaBatch;
-    const size_t total = 2 * (size_t)ns + tab.size() + (size_t)nb * (4 * (size_t)w.gx + 4);
+    double slope = 0.0;
+    for (int k = 0; k < n; ++k) slope = std::max(slope, std::fabs(a[k]));
+    w.lr_reach = slope * w.reach;
+    const size_t total = 2 * (size_t)ns + tab.size() + llr::reweight_table_doubles() + (size_t)nb * (4 * (size_t)w.gx + 4);
     LLR_CUDA(cudaMalloc(&w.buf.p, sizeof(double) * total));
     w.E = (double *)w.buf.p;
     w.lr = w.E + ns;
     double *dtab = w.lr + ns;
-    w.beta = dtab + tab.size();
+    w.tab = dtab + tab.size();
+    w.beta = w.tab + llr::reweight_table_doubles();
     w.part = w.beta + nb;
     w.E1 = w.part + 4 * (size_t)w.gx * nb;
     w.E2 = w.E1 + nb;
@@ -877,6 +892,7 @@ int muca_samples_init(MucaSamples &w, long long ns, const double *E, int n, doub
     LLR_CUDA(cudaMemcpy(dtab, tab.data(), sizeof(double) * tab.size(), cudaMemcpyHostToDevice));
     LLR_CUDA(llr::launch_muca_lnrho(ns, w.E, dtab, dtab + n + 1, n, e0, de, w.lr,
                                     (int)std::min(tiles, 8LL * sms), nullptr));
+    LLR_CUDA(llr::launch_reweight_table(w.tab, nullptr));
     return LLR_OK;
 }
 
@@ -888,8 +904,11 @@ int muca_moments(MucaSamples &w, int nb, const double *beta, double *E1, double 
         const int m = std::min(MucaSamples::kBetaBatch, nb - b0);
         LLR_CUDA(cudaMemcpy(w.beta, beta + b0, sizeof(double) * (size_t)m,
                             cudaMemcpyHostToDevice));
-        LLR_CUDA(llr::launch_reweight(w.ns, w.E, w.lr, w.shift, m, w.beta, w.gx, w.part, w.E1,
-                                      w.E2, w.var, nullptr));
+        double most = 0.0;
+        for (int i = 0; i < m; ++i) most = std::max(most, std::fabs(beta[b0 + i]));
+        const bool small = most * w.reach + w.lr_reach < 549755813888.0;   // 2^39
+        LLR_CUDA(llr::launch_reweight(w.ns, w.E, w.lr, w.shift, m, w.beta, small ? w.tab : nullptr,
+                                      w.gx, w.part, w.E1, w.E2, w.var, nullptr));
         const size_t bytes = sizeof(double) * (size_t)m;
         if (E1) LLR_CUDA(cudaMemcpy(E1 + b0, w.E1, bytes, cudaMemcpyDeviceToHost));
         if (E2) LLR_CUDA(cudaMemcpy(E2 + b0, w.E2, bytes, cudaMemcpyDeviceToHost));

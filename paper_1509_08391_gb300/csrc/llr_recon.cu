@@ -14,6 +14,7 @@
 // CTA per coupling forms the log-sum-exp observables, and the C_V peak is a grid
 // scan and a golden-section search on the device, many couplings at once.
 #include <algorithm>
+#include <climits>
 #include <cmath>
 #include <string>
 
@@ -324,6 +325,7 @@ __global__ void __launch_bounds__(kT) muca_lnrho_kernel(long long ns, const doub
         out[i] = lnrho_piecewise(lnr, a, n, e0, de, E[i]);
 }
 
+// Exponents of any size (the table form below takes those within 2^39).
 // Block (x, y): coupling beta[y] over the samples of kT-wide tiles x,
 // x + gridDim.x, ...  Each thread keeps a running maximum m of the exponent
 // and rescales its sums when it grows; the block then brings its threads to
@@ -366,10 +368,99 @@ __global__ void __launch_bounds__(kT) reweight_partial_kernel(long long ns, cons
     }
 }
 
-// One block per coupling: combine the gx partials of reweight_partial_kernel.
-// E1 = <E>, var = <E^2> - <E>^2, E2 = <E^2> (any of them may be null).
+// The same for NB couplings a block, with the exponentials by table (Tang, "Table-
+// driven implementation of the exponential function in IEEE floating-point
+// arithmetic", 1989): exp(y) = 2^(k / 2048) (1 + r + r^2 / 2 + r^3 / 6) with k the
+// integer nearest 2048 y / ln 2 and |r| <= ln 2 / 4096 the rest of y (r^4 / 24 <
+// 4e-17).  The kernel is bound by the FP64 pipe (1.6 operations per clock and
+// SM), so everything that need not be FP64 is not: k's power of two goes into the
+// exponent field, and the sums' scale is an exact power of two, found and kept as
+// an integer.  12 FP64 operations per sample and coupling (87 % of the pipe's time)
+// where the library's exp and the running maximum took about twice as many, and
+// fewer, longer blocks: a coupling of 512000 samples 47 us -> 18 us.  The exponent is formed over d = E - shift, whose rounding is smaller than
+// E's.  Writes (N, s0, s1, s2), s_j = sum d^j exp(b d + lr) / 2^N.
+constexpr int kExpBits = 11, kExpTable = 1 << kExpBits;
+
+__global__ void __launch_bounds__(kT) exp_table_kernel(double *tab)
+{
+    const int j = blockIdx.x * kT + threadIdx.x;
+    if (j < kExpTable) tab[j] = exp2((double)j / kExpTable);
+}
+
+template <int NB>
+__global__ void __launch_bounds__(kT) reweight_table_kernel(long long ns, const double *E,
+                                                            const double *lr, double shift,
+                                                            int n_beta, const double *beta,
+                                                            const double *tab, double *part)
+{
+    __shared__ double T[kExpTable];
+    __shared__ double red[kT / 32];
+    constexpr double kMagic = 6755399441055744.0;   // 1.5 2^52: rounds to an integer in the low bits
+    constexpr double kInv = 2954.639443740597;     // 2048 / ln 2
+    constexpr double kHi = 3.384507717577858e-4;   // ln 2 / 2048, and what its rounding leaves
+    constexpr double kLo = 1.1323470770733885e-20;
+    for (int j = threadIdx.x; j < kExpTable; j += kT) T[j] = tab[j];
+    const int b0 = blockIdx.y * NB;
+    double b[NB], s0[NB], s1[NB], s2[NB];
+    long long N[NB];
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        b[q] = beta[min(b0 + q, n_beta - 1)];
+        s0[q] = s1[q] = s2[q] = 0.0;
+        N[q] = LLONG_MIN;
+    }
+    __syncthreads();
+    const long long stride = (long long)gridDim.x * kT;
+    for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < ns; i += stride) {
+        const double d = E[i] - shift, l = lr[i], d2 = d * d;
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            const double y = fma(b[q], d, l);
+            const double kd = fma(y, kInv, kMagic);
+            const double kf = kd - kMagic;
+            const double r = fma(kf, -kLo, fma(kf, -kHi, y));
+            const long long k = __double_as_longlong(kd) - 0x4338000000000000ll;
+            const long long n = k >> kExpBits;   // power of two
+            if (n > N[q]) {   // a larger term than any before: rescale, rarely
+                const double f = N[q] == LLONG_MIN ? 0.0 : exp2((double)(N[q] - n));
+                s0[q] *= f;
+                s1[q] *= f;
+                s2[q] *= f;
+                N[q] = n;
+            }
+            const double t = T[(int)k & (kExpTable - 1)];
+            double w = fma(t, r * fma(r, fma(r, 1.0 / 6.0, 0.5), 1.0), t);   // in [1, 2)
+            const long long down = N[q] - n;
+            w = down < 1000 ? __hiloint2double(__double2hiint(w) - ((int)down << 20),
+                                               __double2loint(w))
+                            : 0.0;
+            s0[q] += w;
+            s1[q] = fma(d, w, s1[q]);
+            s2[q] = fma(d2, w, s2[q]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NB; ++q) {
+        const double nq = N[q] == LLONG_MIN ? -INFINITY : (double)N[q];
+        const double M = block_max(nq, red);
+        const double f = N[q] == LLONG_MIN ? 0.0 : exp2(nq - M);
+        const double t0 = block_sum(s0[q] * f, red), t1 = block_sum(s1[q] * f, red),
+                     t2 = block_sum(s2[q] * f, red);
+        if (threadIdx.x == 0 && b0 + q < n_beta) {
+            double *p = part + 4 * ((size_t)(b0 + q) * gridDim.x + blockIdx.x);
+            p[0] = M;
+            p[1] = t0;
+            p[2] = t1;
+            p[3] = t2;
+        }
+    }
+}
+
+// One block per coupling: combine the gx partials of reweight_partial_kernel or
+// (pow2) reweight_table_kernel.  E1 = <E>, var = <E^2> - <E>^2, E2 = <E^2> (any of
+// them may be null).
 __global__ void __launch_bounds__(kT) reweight_combine_kernel(int gx, const double *part,
-                                                              double shift, double *E1,
+                                                              bool pow2, double shift, double *E1,
                                                               double *E2, double *var)
 {
     __shared__ double red[kT / 32];
@@ -381,7 +472,7 @@ __global__ void __launch_bounds__(kT) reweight_combine_kernel(int gx, const doub
     for (int j = threadIdx.x; j < gx; j += kT) {
         const double mj = p[4 * j];
         if (mj == -INFINITY) continue;        // a block without samples
-        const double r = exp(mj - m);
+        const double r = pow2 ? exp2(mj - m) : exp(mj - m);
         s0 += r * p[4 * j + 1];
         s1 += r * p[4 * j + 2];
         s2 += r * p[4 * j + 3];
@@ -430,13 +521,37 @@ cudaError_t launch_muca_lnrho(long long ns, const double *E, const double *lnr, 
     return cudaGetLastError();
 }
 
+size_t reweight_table_doubles()
+{
+    return kExpTable;
+}
+
+cudaError_t launch_reweight_table(double *tab, cudaStream_t s)
+{
+    exp_table_kernel<<<kExpTable / kT, kT, 0, s>>>(tab);
+    return cudaGetLastError();
+}
+
 cudaError_t launch_reweight(long long ns, const double *E, const double *lr, double shift,
-                            int n_beta, const double *beta, int gx, double *part, double *E1,
-                            double *E2, double *var, cudaStream_t s)
+                            int n_beta, const double *beta, const double *tab, int gx,
+                            double *part, double *E1, double *E2, double *var, cudaStream_t s)
 {
     if (n_beta <= 0) return cudaSuccess;
-    reweight_partial_kernel<<<dim3(gx, n_beta), kT, 0, s>>>(ns, E, lr, shift, beta, part);
-    reweight_combine_kernel<<<n_beta, kT, 0, s>>>(gx, part, shift, E1, E2, var);
+    constexpr int NB = 4;   // couplings a block: samples and table are read once for all
+    if (tab && n_beta >= NB) {
+        // one wave over all couplings (three blocks an SM by registers; gx is two): a
+        // block's table and reductions cost as much as some thousand samples
+        const int groups = (n_beta + NB - 1) / NB;
+        gx = std::max(1, std::min(gx, 3 * gx / 2 / groups));
+        reweight_table_kernel<NB><<<dim3(gx, groups), kT, 0, s>>>(ns, E, lr, shift, n_beta, beta,
+                                                                 tab, part);
+    }
+    else if (tab)
+        reweight_table_kernel<1><<<dim3(gx, n_beta), kT, 0, s>>>(ns, E, lr, shift, n_beta, beta,
+                                                                 tab, part);
+    else
+        reweight_partial_kernel<<<dim3(gx, n_beta), kT, 0, s>>>(ns, E, lr, shift, beta, part);
+    reweight_combine_kernel<<<n_beta, kT, 0, s>>>(gx, part, tab != nullptr, shift, E1, E2, var);
     return cudaGetLastError();
 }
 
