@@ -42,7 +42,7 @@ def parse():
     p.add_argument("--n-therm", type=int, default=2)
     p.add_argument("--n-meas", type=int, default=8)
     p.add_argument("--threads", type=int, default=0,
-                   help="threads per CTA (128/256/512); 0 = autotuned")
+                   help="threads per lattice (128/256/512); 0 = autotuned")
     p.add_argument("--no-e2e", action="store_true")
     p.add_argument("--no-cpu", action="store_true")
     p.add_argument("--intervals", type=int, default=256)
@@ -1187,7 +1187,7 @@ def run_uneven(args):
 
 def run_phases(args):
     """One launch per pass kind on 456 lattices of the benchmark workload (one
-    full wave of 256-thread CTAs: 3 per SM on 152 SMs), so an ncu capture
+    full wave of 152 CTAs, three lattices each), so an ncu capture
     (-k regex:llr_kernel) sees: resync, approach, two composite sweeps (one
     launch), overrelaxation pass, heat-bath pass, composite sweep."""
     import torch

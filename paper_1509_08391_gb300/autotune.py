@@ -2,9 +2,10 @@
 
 Knobs (none changes the chains: every shape runs the same per-link
 arithmetic in the same order, so the choice changes speed only):
-  * threads per CTA: 128, 160, 192, 256, 512 (one warp takes the window
-    decisions, the others propose; the chunk of a heat-bath pass is the
-    proposing warps x 32 links, so this also sets the chunk size);
+  * threads per lattice: 128, 160 or 192, 256, 512 (the 24 warps of a CTA
+    advance 6, 4, 3 or 1 lattices together; of a lattice's warps one takes the
+    window decisions and the others propose, 64 links per warp and chunk, so
+    this also sets the chunk size of a heat-bath pass);
   * ring: stages of the producer/consumer ring in use (1, 2, 4), how many
     chunks the proposing warps may run ahead of the deciding warp;
   * carveout: the shared-memory share of the SM's unified L1/shared storage

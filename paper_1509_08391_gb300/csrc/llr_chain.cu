@@ -22,9 +22,10 @@
 //     across SMs.  The lattices of an item advance together, phase by phase
 //     (heat-bath pass, overrelaxation passes, energy).
 //   * Lattices per item (choose_teams): with fewer lattices than SMs, one with
-//     all 24 warps; with many, three with 8 warps each in the heat-bath pass,
-//     whose deciding warps are serial and need company, while the
-//     overrelaxation pass takes them together or one after another.
+//     all 24 warps; with many, three with 8 warps each or four with 6 in the
+//     heat-bath pass, whose deciding warps are serial and need company, while
+//     the overrelaxation pass takes up to three together, or one after another
+//     where a slab fills the shared memory.
 //   * A heat-bath pass runs class by class over the whole lattice (one
 //     pipeline drain per class); an overrelaxation pass is slab-major: for
 //     each x3 slab, all 8 checkerboard classes of that slab in order.
@@ -36,8 +37,8 @@
 //     64 links; a consumer warp walks the chunks in link order and decides
 //     each block of B links with the restricted Metropolis rule
 //     dist(E + dE_block) <= dist(E), using a ballot to find the first rejected
-//     block among 32 speculatively accepted ones, and publishes the accepted
-//     links; the producers write their angles.  Chunks pass through a ring of
+//     block among those of 32 speculatively accepted links, and publishes the
+//     accepted links; the producers write their angles.  Chunks pass through a ring of
 //     1 to 4 stages in shared memory guarded by named barriers, so proposals
 //     for later chunks overlap with the scan of earlier ones.
 //   * The multicanonical pass (Sec. 2.6) has the same producers at a fixed
@@ -52,13 +53,13 @@
 //     fused operations written out, so every program (batched sweeps, single
 //     passes, the plain form), launch shape and build gives bit-identical chains.
 //   * After 1 + n_or passes the 6V plaquettes are summed (float32 angles
-//     summed exactly as hi + lo, cosf, fixed-point accumulation) and the tracked
-//     energy is resynchronised.
+//     summed exactly as hi + lo, their unbiased cosine in packed arithmetic,
+//     fixed-point accumulation) and the tracked energy is resynchronised.
 //
 // Measured (GB300, 2070 MHz; one pass of 456 lattices of L = 20, ms, before ->
-// now): heat-bath 10.1 -> 7.8 (797 -> 640 instructions per link), overrelaxation
-// 2.7 -> 1.9 (184 -> 125), against one CTA of 256 threads per lattice and one
-// link per thread; L = 8, 128 lattices: 0.28 -> 0.22 and 0.08 -> 0.07.
+// now): heat-bath 10.1 -> 7.4 (797 -> 628 instructions per link), overrelaxation
+// 2.7 -> 1.9 (184 -> 120), energy 1.3 -> 0.97, against one CTA of 256 threads per
+// lattice and one link per thread.
 #include <algorithm>
 #include <cstdio>
 
@@ -732,8 +733,8 @@ __device__ __forceinline__ float overrelax_link(const float *th, const float *ow
 }
 
 // One overrelaxation group (the links of class (MU, p) with half-site index
-// in [h0, h0 + count)) of a lattice whose slab is too large for shared memory
-// (L > kSlabMaxL): every thread reflects its links, neighbours by plain loads.
+// in [h0, h0 + count)) of a lattice with planes of more pairs than the team has
+// threads: every thread reflects its links, neighbours by plain loads.
 template <int MU, bool FAST>
 __device__ __noinline__ void overrelax_class(const LatState &st, const Team &t, float *th, int p,
                                              int h0, int count)
@@ -1080,14 +1081,16 @@ __device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb,
 }
 
 // ---------------------------------------------------------------------------
-// Overrelaxation pass with the current slab in shared memory.
+// Overrelaxation pass slab by slab, the current slab in shared memory where it fits.
 //
 // The pass goes slab by slab of x3, in each slab class by class, so every class
 // reads the same 8 class arrays of the slab (4 L^3 angles) again: they are
 // copied to shared memory once per slab (16 L^3 bytes, 128 KB at L = 20) and
 // the classes read 13 to 14 of a link's 18 neighbours there; the others lie in
 // the slabs before and after and are plain loads (neither slab changes during
-// this one).  New angles go to shared memory and to global memory.
+// this one).  New angles go to shared memory and to global memory.  Slabs of
+// L > 24 do not fit and are read in place, one lattice at a time (304 of L = 28: two
+// sweeps 111 ms; link by link, two or three lattices at a time, 150 to 167 ms).
 //
 // A thread reflects two links at a time, so the index arithmetic and (with
 // rows of even length, ROW) the loads serve two: links k, k + 1 of one x0 row
@@ -1095,7 +1098,7 @@ __device__ __noinline__ void consume_class_muca(LatState &st, const HbTeam &hb,
 // and x2 + L / 2.  With ROW threads map to (x2 plane, x1, k) and step over planes,
 // so only x2 changes from one unit of a thread to the next; planes of odd half
 // rows fill a team's threads badly (196 of 256 at L = 14, four iterations where
-// the units need three: 0.55 against 0.47 ms a pass of 456 lattices), so there a
+// the units need three: 0.55 against 0.50 ms a pass of 456 lattices), so there a
 // thread takes every nt-th unit.
 // ---------------------------------------------------------------------------
 constexpr int kSlabMaxL = 24;       // 16 * 24^3 bytes = 216 KB
@@ -1204,13 +1207,14 @@ __device__ __forceinline__ float2 pair_dn0(const float *a, const X0Off<ROW> &x, 
 }
 
 // Reflect the pair of links theta_MU of parity p at plane x2, offset h of the
-// slab; sl: the slab's class arrays in shared memory (stride S); th: the
-// lattice, tc / tp / tm its offsets of this slab, the next and the one before.
-template <int MU, bool ROW, bool FAST>
+// slab; sl: the slab's class arrays, COPY: in shared memory (stride S), otherwise
+// where they are (stride half); th: the lattice, tc / tp / tm its offsets of this
+// slab, the next and the one before.
+template <int MU, bool ROW, bool COPY, bool FAST>
 __device__ __forceinline__ void reflect_pair(const SlabGeo &g, int x2, int h, int p, int t,
                                              float *sl, float *th, int tc, int tp, int tm)
 {
-    const int q = p ^ 1, S = g.S, SH = g.SH, half = g.half, wr = S - g.S1;
+    const int q = p ^ 1, SH = g.SH, half = g.half, S = COPY ? g.S : half, wr = g.S - g.S1;
     const int d1p = g.d1p, d1m = g.d1m;
     // x2 neighbours of the first link; of the second, relative to h
     const int d2p = (ROW && x2 == g.L - 1) ? -wr : g.S1, d2m = x2 == 0 ? wr : -g.S1;
@@ -1305,18 +1309,20 @@ __device__ __forceinline__ void reflect_pair(const SlabGeo &g, int x2, int h, in
     tn.y = wrap_angle(-t0.y - 2.0f * al.y);
     const int so = h + (2 * MU + p) * S, go = h + (2 * MU + p) * half + tc;
     if (ROW) {
-        *(float2 *)(sl + so) = tn;
+        if (COPY) *(float2 *)(sl + so) = tn;
         *(float2 *)(th + go) = tn;
     } else {
-        sl[so] = tn.x;
-        sl[so + SH] = tn.y;
+        if (COPY) {
+            sl[so] = tn.x;
+            sl[so + SH] = tn.y;
+        }
         th[go] = tn.x;
         th[go + SH] = tn.y;
     }
 }
 
 // The two classes of direction MU in one slab.
-template <int MU, bool ROW, bool FAST>
+template <int MU, bool ROW, bool COPY, bool FAST>
 __device__ __forceinline__ void reflect_dir(SlabGeo &g, const Team &tm_, int t, int mask,
                                             float *sl, float *th, int tc, int tp, int tm)
 {
@@ -1327,7 +1333,8 @@ __device__ __forceinline__ void reflect_dir(SlabGeo &g, const Team &tm_, int t, 
             int x2 = g.x2, h = g.h;
 #pragma unroll 1
             for (int i = 0; i < g.nit; ++i) {
-                if (x2 < g.planes) reflect_pair<MU, ROW, FAST>(g, x2, h, p, t, sl, th, tc, tp, tm);
+                if (x2 < g.planes)
+                    reflect_pair<MU, ROW, COPY, FAST>(g, x2, h, p, t, sl, th, tc, tp, tm);
                 x2 += g.step;
                 h += g.step * g.S1;
             }
@@ -1335,7 +1342,7 @@ __device__ __forceinline__ void reflect_dir(SlabGeo &g, const Team &tm_, int t, 
 #pragma unroll 1
             for (int u = tm_.tid; u < g.SH; u += g.step) {
                 g.unit(u);
-                reflect_pair<MU, ROW, FAST>(g, g.x2, g.h, p, t, sl, th, tc, tp, tm);
+                reflect_pair<MU, ROW, COPY, FAST>(g, g.x2, g.h, p, t, sl, th, tc, tp, tm);
             }
         }
         tm_.sync();   // the next class reads the angles written here
@@ -1343,9 +1350,9 @@ __device__ __forceinline__ void reflect_dir(SlabGeo &g, const Team &tm_, int t, 
 }
 
 // The whole pass of the team's lattice: every reflection is taken (see
-// overrelax_pass).  slab_off: the team's slab in g_dyn.  The team shrinks to
+// overrelax_pass).  slab_off: the team's slab in g_dyn (COPY).  The team shrinks to
 // the warps that hold a link; the others return.
-template <bool ROW, bool FAST>
+template <bool ROW, bool COPY, bool FAST>
 __device__ __noinline__ void reflect_slabs(Team team, int L_, float *th_, int slab_off, int mask)
 {
     const int L = uniform(L_);
@@ -1360,23 +1367,27 @@ __device__ __noinline__ void reflect_slabs(Team team, int L_, float *th_, int sl
 #pragma unroll 1
     for (int t = 0; t < L; ++t) {
         const int tc = t * S, tp = (t == L - 1 ? 0 : t + 1) * S, tm = (t == 0 ? L - 1 : t - 1) * S;
-        // S = L^3 / 2 is a multiple of 4 floats for even L, as are all offsets
+        if (COPY) {
+            // S = L^3 / 2 is a multiple of 4 floats for even L, as are all offsets
 #pragma unroll 1
-        for (int a = 0; a < 8; ++a)
-            for (int i = 4 * team.tid; i < S; i += 4 * team.nt)
-                cp_async16(sl + a * S + i, th + tc + a * half + i);
-        cp_async_commit();
-        // the next slab on its way from HBM to L2
+            for (int a = 0; a < 8; ++a)
+                for (int i = 4 * team.tid; i < S; i += 4 * team.nt)
+                    cp_async16(sl + a * S + i, th + tc + a * half + i);
+            cp_async_commit();
+            // the next slab on its way from HBM to L2
 #pragma unroll 1
-        for (int a = 0; a < 8; ++a)
-            for (int i = 32 * team.tid; i < S; i += 32 * team.nt)
-                asm volatile("prefetch.global.L2 [%0];" ::"l"(th + tp + a * half + i));
-        cp_async_wait<0>();
-        team.sync();
-        reflect_dir<0, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
-        reflect_dir<1, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
-        reflect_dir<2, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
-        reflect_dir<3, ROW, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+            for (int a = 0; a < 8; ++a)
+                for (int i = 32 * team.tid; i < S; i += 32 * team.nt)
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(th + tp + a * half + i));
+            cp_async_wait<0>();
+            team.sync();
+        } else {
+            sl = th + tc;
+        }
+        reflect_dir<0, ROW, COPY, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<1, ROW, COPY, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<2, ROW, COPY, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
+        reflect_dir<3, ROW, COPY, FAST>(g, team, t, mask, sl, th, tc, tp, tm);
     }
 }
 
@@ -1470,8 +1481,7 @@ __device__ __noinline__ void overrelax_pass(Smem &sm, int slot, const Team &team
     const long long E = st.E_fx;   // the running energy; overrelaxation leaves it
     const bool free_all = E < lo || E > hi || (E - bound >= lo && E + bound <= hi);
     // the L^2 / 4 pairs of a plane need a thread each
-    const bool in_slabs =
-        free_all && (res || (L <= kSlabMaxL && ((L & 3) != 0 || L * L <= 4 * team.nt)));
+    const bool in_slabs = free_all && (res || (L & 3) != 0 || L * L <= 4 * team.nt);
     if (in_slabs && res) {
         switch (L) {
             case 2: reflect_lattice<2, FAST>(team, slab_off, class_mask); break;
@@ -1480,11 +1490,16 @@ __device__ __noinline__ void overrelax_pass(Smem &sm, int slot, const Team &team
             case 8: reflect_lattice<8, FAST>(team, slab_off, class_mask); break;
             default: reflect_lattice<10, FAST>(team, slab_off, class_mask); break;
         }
+    } else if (in_slabs && L <= kSlabMaxL) {
+        if ((L & 3) == 0)
+            reflect_slabs<true, true, FAST>(team, L, th, slab_off, class_mask);
+        else
+            reflect_slabs<false, true, FAST>(team, L, th, slab_off, class_mask);
     } else if (in_slabs) {
         if ((L & 3) == 0)
-            reflect_slabs<true, FAST>(team, L, th, slab_off, class_mask);
+            reflect_slabs<true, false, FAST>(team, L, th, slab_off, class_mask);
         else
-            reflect_slabs<false, FAST>(team, L, th, slab_off, class_mask);
+            reflect_slabs<false, false, FAST>(team, L, th, slab_off, class_mask);
     }
     int taken = 0;              // moves taken by this thread in near-edge groups
     if (!in_slabs) {
@@ -2109,7 +2124,7 @@ __global__ void hot_start_kernel(LatState *lats, float *theta)
 // FP64 fresh energy: plaquette angle and cos in double, warp-shuffle FP64
 // reduction.  Bound by the FP64 cosines (about 1.6 DFMA per clock and SM), so a
 // lattice is spread over gridDim.x CTAs, one part of the sum each: one lattice of
-// L = 20 took 5.8 ms on one SM, 0.05 ms on all.
+// L = 20 takes 0.10 ms a call where one CTA took 6.7 ms.
 constexpr int kEnergyThreads = 256, kEnergyCtas = 4096;
 
 __global__ void __launch_bounds__(kEnergyThreads)
@@ -2270,7 +2285,9 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
         const size_t stage = (size_t)kStaged * kThreads * sizeof(float2);
         while (a.ring > 1 && stage + stage1 * a.ring > kDynMax) a.ring >>= 1;
         rings = stage1 * a.ring;
-        a.or_teams = or_most;
+        // lattices read in place go one by one, which leaves each the L1 (a sweep
+        // of 304 of L = 28: 56 ms against 82 ms two at a time)
+        a.or_teams = a.max_L > kSlabMaxL ? 1 : or_most;
         while (a.or_teams > 1 && slab * a.or_teams > kDynMax) --a.or_teams;
         a.slab = (int)(slab / sizeof(float));
         a.ring_off = (int)(stage / sizeof(float));

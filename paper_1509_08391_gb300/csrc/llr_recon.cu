@@ -150,8 +150,9 @@ __global__ void __launch_bounds__(kT) cv_grid_kernel(int n, const double *c, con
 // step needs the comparison before it, so the steps are taken several at a
 // time: a round evaluates the points of all outcomes of the next comparisons at
 // once, one block each, and the next round replays the comparisons on the
-// values found.  512 centres, 1601 grid points, tol 1e-10 (26 steps): 14.4 ms
-// with one block for everything, 0.1 ms with the grid in parallel and 5 rounds.
+// values found.  512 centres, 1601 grid points, tol 1e-10 (26 steps): a call takes
+// 15.6 ms with one block for everything, 0.47 ms with the grid in parallel and 5
+// rounds.
 constexpr int kFirstDepth = 6, kDepth = 7;            // comparisons ahead per round
 constexpr int kFirstNodes = 2 + 2 * ((1 << kFirstDepth) - 1);   // x1, x2, a tree per outcome
 constexpr int kNodes = (1 << kDepth) - 1;             // one tree: the first outcome is known
@@ -377,8 +378,9 @@ __global__ void __launch_bounds__(kT) reweight_partial_kernel(long long ns, cons
 // exponent field, and the sums' scale is an exact power of two, found and kept as
 // an integer.  12 FP64 operations per sample and coupling (87 % of the pipe's time)
 // where the library's exp and the running maximum took about twice as many, and
-// fewer, longer blocks: a coupling of 512000 samples 47 us -> 18 us.  The exponent is formed over d = E - shift, whose rounding is smaller than
-// E's.  Writes (N, s0, s1, s2), s_j = sum d^j exp(b d + lr) / 2^N.
+// fewer, longer blocks: a coupling of 512000 samples 47 us -> 18 us.  The exponent
+// is formed over d = E - shift, whose rounding is smaller than E's.  Writes
+// (N, s0, s1, s2), s_j = sum d^j exp(b d + lr) / 2^N.
 constexpr int kExpBits = 11, kExpTable = 1 << kExpBits;
 
 __global__ void __launch_bounds__(kT) exp_table_kernel(double *tab)

@@ -2,8 +2,8 @@
 
 Sides: L <= 10 stays in shared memory (one link per thread), L = 12 .. 24 has its
 x3 slabs there (pairs in a row where 4 divides L, pairs at x2 and x2 + L / 2
-where not), L = 26 has neither; L = 2 and 6 leave most of a warp idle.  Batches:
-one, two, three or more lattices per CTA.  Every route against the FP64 oracle
+where not), L = 26 and 28 read them in place; L = 2 and 6 leave most of a warp
+idle.  Batches: one, two, three or more lattices per CTA.  Every route against the FP64 oracle
 (tolerances of tests/gpu_helpers.py) or bit for bit against another route."""
 import numpy as np
 import pytest
@@ -58,7 +58,7 @@ def test_class_updates_match_oracle(L, block, threads):
 
 
 @pytest.mark.parametrize("L,n", [(2, 2), (6, 2), (10, 1), (12, 2), (14, 2), (16, 1), (18, 1),
-                                 (20, 1), (22, 1), (24, 1), (26, 1)])
+                                 (20, 1), (22, 1), (24, 1), (26, 1), (28, 1)])
 def test_overrelaxation_pass_matches_oracle(L, n):
     w = _workload(L, n)
     six_v = 6.0 * L ** 4
