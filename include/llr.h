@@ -306,13 +306,14 @@ int llr_muca_cv_peak(long long n_samples, const double *E, int n, double e0, dou
 int llr_muca_tunnellings(int n_steps, int n_chains, const double *E, double lo, double hi,
                          int *out);
 
-/* Launch shape of the batched sweep kernel: the most threads that work on one
+/* Launch shape of the batched sweep kernel: the threads that work on one
  * lattice (128, 160, 192, 256 or 512).  A CTA has 768 threads and advances 6, 4,
- * 4, 3 or 1 lattices at a time accordingly.  fast_math (1: hardware sine/cosine
+ * 4, 3 or 1 lattices at a time accordingly, fewer where the batch has fewer for
+ * every SM.  fast_math (1: hardware sine/cosine
  * approximations for the staples, 0: correctly rounded-class sincosf).
  * Chosen per lattice size by the autotuner; default 256 threads, fast math, and,
  * until a shape is set, more threads per lattice for batches of fewer lattices
- * than 3 per SM. */
+ * than 3 per SM, fewer for L <= 6 and for many large lattices. */
 int llr_set_kernel_config(llr_handle h, int threads, int fast_math);
 
 /* The full launch shape of the batched sweep kernel, as the autotuner sets

@@ -25,7 +25,7 @@
 //     all 24 warps; with many, three with 8 warps each or four with 6 in the
 //     heat-bath pass, whose deciding warps are serial and need company, while
 //     the overrelaxation pass takes up to three together, or one after another
-//     where a slab fills the shared memory.
+//     where a slab fills the shared memory; up to six of L <= 6.
 //   * A heat-bath pass runs class by class over the whole lattice (one
 //     pipeline drain per class); an overrelaxation pass is slab-major: for
 //     each x3 slab, all 8 checkerboard classes of that slab in order.
@@ -2239,19 +2239,31 @@ int prepare_kernel(int carveout)
     return sms[dev];
 }
 
-// Lattices a CTA works on at a time: one while there are not many more than SMs
-// (time is one lattice's then), two, three.  Where a lattice's slab leaves no room
-// for another's, so that overrelaxation takes them one by one anyway, and there
-// are enough to go round evenly, a fourth keeps the heat-bath's schedulers fuller:
-// a sweep of L = 20 per lattice and SM is 5.30 ms with three and 5.15 ms with four,
-// of L = 14 1.46 ms and 1.6 ms.
-int choose_teams(const LaunchCfg &cfg, int n_lat, int sms, bool one_slab)
+// Lattices a CTA works on at a time.
+//   * One while there are not many more than SMs (time is one lattice's then), two,
+//     three.
+//   * Where a lattice's slab leaves no room for another's, so that overrelaxation
+//     takes them one by one anyway, and there are enough to go round evenly, a
+//     fourth keeps the heat-bath's schedulers fuller: a sweep of 1824 lattices of
+//     L = 20 takes 62.3 ms with three and 61.4 ms with four, a Robbins-Monro step of
+//     2048 362 and 348 ms; of L = 14, where it costs, 16.0 and 17.6 ms.
+//   * Up to six of L <= 6, whose classes (L^3 / 2 links of a slab, L^4 / 2 of the
+//     lattice) leave most of a third of the CTA idle: six sweeps of 4096 lattices of
+//     L = 2 / 4 / 6 take 4.0 / 5.7 / 10.9 ms with three, 2.5 / 3.6 / 7.7 ms with six; of
+//     L = 8 21.5 ms with three, 26.0 ms with six.
+int choose_teams(const LaunchCfg &cfg, int n_lat, int sms, int max_L, bool one_slab)
 {
+    int most = one_slab && n_lat >= 8 * sms ? 4 : 3;
     if (!cfg.auto_threads)
-        return cfg.threads >= 512 ? 1 : cfg.threads >= 256 ? 3 : cfg.threads >= 160 ? 4 : 6;
-    if (n_lat <= sms + sms / 2) return 1;
-    if (n_lat <= 2 * sms) return 2;
-    return one_slab && n_lat >= 8 * sms ? 4 : 3;
+        most = cfg.threads >= 512 ? 1 : cfg.threads >= 256 ? 3 : cfg.threads >= 160 ? 4 : 6;
+    else if (n_lat <= sms + sms / 2)
+        most = 1;
+    else if (max_L <= 6)
+        most = 6;
+    // no more than the batch has for every SM (152 lattices of L = 8 asked to run
+    // six to a CTA: 1.90 ms on 26 SMs, 0.65 ms on all)
+    const int each = (n_lat + sms - 1) / sms;
+    return each >= most ? most : each == 5 ? 4 : each;
 }
 
 template <bool FAST>
@@ -2261,7 +2273,7 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     const int per_lat = multi ? (a.n_therm + a.n_meas) : 1;
     if ((long long)a.n_lat * per_lat <= 0) return cudaSuccess;
     const int sms = prepare_kernel<FAST>(cfg.carveout);
-    a.teams = choose_teams(cfg, a.n_lat, sms, a.slab_L > 0 && 2 * slab_bytes(a.slab_L) > kDynMax);
+    a.teams = choose_teams(cfg, a.n_lat, sms, a.max_L, a.slab_L > 0 && 2 * slab_bytes(a.slab_L) > kDynMax);
     // 15 named barriers, two per ring stage of each team
     const int most = a.teams == 1 ? 4 : a.teams <= 3 ? 2 : 1;
     a.ring = cfg.ring < most ? cfg.ring : most;
@@ -2269,9 +2281,10 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     const size_t lattices = (size_t)a.teams * lattice_bytes(a.max_L);
     // a lattice may be resident if a team of the overrelaxation pass has a
     // thread for each of the L^3 / 2 links of a slab's class
-    const int or_most = std::min(a.teams, 3);
+    const int links = a.max_L <= kResidentMaxL ? a.max_L * a.max_L * a.max_L / 2 : kThreads;
+    const int or_most = links <= kWarps / a.teams * 32 ? a.teams : std::min(a.teams, 3);
     a.resident = a.max_L <= kResidentMaxL && lattices + stage1 <= kDynMax &&
-                 a.max_L * a.max_L * a.max_L / 2 <= kWarps / or_most * 32;
+                 links <= kWarps / or_most * 32;
     while (a.resident && lattices + stage1 * a.ring > kDynMax) a.ring >>= 1;
     size_t rings = stage1 * a.ring;
     size_t dyn;
@@ -2287,7 +2300,7 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
         rings = stage1 * a.ring;
         // lattices read in place go one by one, which leaves each the L1 (a sweep
         // of 304 of L = 28: 56 ms against 82 ms two at a time)
-        a.or_teams = a.max_L > kSlabMaxL ? 1 : or_most;
+        a.or_teams = a.max_L > kSlabMaxL ? 1 : std::min(a.teams, 3);
         while (a.or_teams > 1 && slab * a.or_teams > kDynMax) --a.or_teams;
         a.slab = (int)(slab / sizeof(float));
         a.ring_off = (int)(stage / sizeof(float));

@@ -45,10 +45,12 @@ def test_class_updates_match_oracle(L, block, threads):
     """Every class of a heat-bath and an overrelaxation pass: groups of links
     that end a class in any place, every block size, every team."""
     n = 2 if L <= 10 else 1
-    w = _workload(L, n, block=block)
+    # a CTA takes more than one lattice where the batch has that many for every SM
+    total = n if threads == 512 else 919
+    w = _workload(L, total, block=block)
     if L == 2:   # 96 plaquettes: a window that any energy is in
         w.E_lo, w.dE = [-100.0] * n, [200.0] * n
-    a = np.linspace(-1.02, -0.98, n)
+    a = np.linspace(-1.02, -0.98, total)
     with llr.Batch.from_workload(w, max_approach=5000) as b:
         b.set_kernel_config(threads, True)
         b.sweep(a, 2)
@@ -74,7 +76,7 @@ def test_overrelaxation_pass_matches_oracle(L, n):
 @pytest.mark.parametrize("L", [4, 6, 10, 12, 14, 20])
 def test_chains_do_not_depend_on_lattices_per_cta(L):
     """1, 3, 4 and 6 lattices per CTA, with and without fast math, in windows."""
-    w = _workload(L, 7 if L < 20 else 3)
+    w = _workload(L, 919)
     a = np.linspace(-1.02, -0.99, w.n_lattices)
     for fast in (True, False):
         outs = []
