@@ -2277,7 +2277,14 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     // 15 named barriers, two per ring stage of each team
     const int most = a.teams == 1 ? 4 : a.teams <= 3 ? 2 : 1;
     a.ring = cfg.ring < most ? cfg.ring : most;
-    const size_t stage1 = (size_t)a.teams * (kWarps / a.teams - 1) * kStageGroupBytes;
+    const int groups = kWarps / a.teams - 1;
+    // two stages serve a class of two chunks (128 of L = 8: a sweep 0.272 ms with
+    // two, 0.285 ms with four); longer classes use all (152 of L = 20 6.50, 6.60 ms
+    // with one)
+    if (a.ring > 2 && a.max_L <= kResidentMaxL &&
+        a.max_L * a.max_L * a.max_L * a.max_L / 2 <= 2 * 64 * groups)
+        a.ring = 2;
+    const size_t stage1 = (size_t)a.teams * groups * kStageGroupBytes;
     const size_t lattices = (size_t)a.teams * lattice_bytes(a.max_L);
     // a lattice may be resident if a team of the overrelaxation pass has a
     // thread for each of the L^3 / 2 links of a slab's class
