@@ -190,7 +190,9 @@ int llr_replica_exchange(llr_handle h, int n_pairs, const int *pairs, const doub
 int llr_energy(llr_handle h, double *E_out);
 
 /* The tracked energies that the window test uses (after the last resync).
- * E_out: host double[n_lattices]. */
+ * E_out: host double[n_lattices]; NaN where that resync (or llr_set_links)
+ * found links that are no numbers, which also sets the lattice's status to
+ * LLR_ERR_NUMERIC at a resync. */
 int llr_tracked_energy(llr_handle h, double *E_out);
 
 /* Copy one lattice's links to / from a host float[4 L^4] in the canonical

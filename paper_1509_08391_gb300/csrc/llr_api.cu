@@ -604,7 +604,7 @@ int llr_tracked_energy(llr_handle h, double *E_out)
     if (!E_out) return fail(LLR_ERR_ARG, "null E_out");
     std::vector<LatState> st;
     if (int r = pull_states(h, st)) return r;
-    for (int i = 0; i < h->n; ++i) E_out[i] = (double)st[(size_t)i].E_fx * llr::kInvFx;
+    for (int i = 0; i < h->n; ++i) E_out[i] = llr::energy_of(st[(size_t)i].E_fx);
     return LLR_OK;
 }
 

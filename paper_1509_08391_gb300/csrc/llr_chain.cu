@@ -1770,7 +1770,8 @@ __device__ __forceinline__ float2 plaquette_cos2(float2 a, float2 b, float2 c, f
 // Fresh energy of the team's lattice in fixed point: sum over the 6 V
 // plaquettes, exact int64 accumulation and reduction.  Two sites per thread (half
 // sites h, h + 1 of a parity), their plaquettes in packed arithmetic.  Valid in
-// the team's thread 0.
+// the team's thread 0.  Angles that are no numbers leave no energy: kNoEnergy, found
+// apart from the sum, in which the parts of several such plaquettes could cancel.
 template <bool ROW>
 __device__ __noinline__ long long fresh_energy_fx(const LatState &st_, const Team &team,
                                                   long long *red, const float *th)
@@ -1779,6 +1780,7 @@ __device__ __noinline__ long long fresh_energy_fx(const LatState &st_, const Tea
     const int L = uniform(st_.L), half = uniform(st_.half);
     const uint32_t magic = uniform(st_.magic);
     long long acc = 0;
+    unsigned wild = 0;   // 2^21 or more: a plaquette was no number
 #pragma unroll 1
     for (int p = 0; p < 2; ++p)
 #pragma unroll 1
@@ -1809,18 +1811,25 @@ __device__ __noinline__ long long fresh_energy_fx(const LatState &st_, const Tea
                     lo += b;
                     bad |= !(fabsf(v.x) < 512.0f) || !(fabsf(v.y) < 512.0f);
                 }
-            // 12 cosines: sums of parts within 32 bits.  Angles that are no numbers
-            // leave an energy that is none (the integer conversion's overflow value).
-            acc += bad ? -(1ll << 62) : (long long)hi * (1 << 20) + lo;
+            // 12 cosines: sums of parts within 32 bits, and |hi| <= 12 2^12 but for NaNs:
+            // each has the part 0x7fffffff - 0x4b400000, and of 1 to 12 of these none
+            // sums to below 2^26 in size modulo 2^32.  (One flag would do for both
+            // lines; carried through the loop as `bad` it costs the compiler's
+            // schedule: 1824 of L = 20 4.37 ms, with the test of hi alone 4.03, so 3.75.)
+            wild |= (unsigned)(hi + (1 << 20));
+            acc += bad ? 0ll : (long long)hi * (1 << 20) + lo;
         }
+    bool none = __any_sync(kFull, wild >= (1u << 21));
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(kFull, acc, o);
-    if (lane == 0) red[team.w] = acc;
+    if (lane == 0) red[team.w] = none ? kNoEnergy : acc;
     team.sync();
-    long long tot = 0;
-    if (team.tid == 0)
-        for (int w = 0; w < team.nw; ++w) tot += red[w];
-    return tot;
+    if (team.w != 0) return 0;
+    long long tot = lane < team.nw ? red[lane] : 0;   // 24 warps at most
+    none = __any_sync(kFull, tot == kNoEnergy);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) tot += __shfl_down_sync(kFull, tot, o);
+    return none ? kNoEnergy : tot;
 }
 
 // Fresh energies of the active lattices of the item, each by its team, into
@@ -1839,13 +1848,14 @@ __device__ __noinline__ void energy_phase(Smem &sm, const Phase &ph, const Kerne
         const long long fresh = (st.L & 3) == 0 ? fresh_energy_fx<true>(st, t, red, th)
                                                 : fresh_energy_fx<false>(st, t, red, th);
         if (t.tid == 0) {
+            if (fresh == kNoEnergy) st.status = -5;   // LLR_ERR_NUMERIC
             if (resync) {
                 const double drift = fabs((double)(st.E_fx - fresh) * kInvFx);
                 if (drift > st.max_drift) st.max_drift = drift;
                 st.sweep += 1u;
                 st.sweeps_done += 1ull;
                 if (measure) {
-                    const double dEm = (double)fresh * kInvFx - (st.E_lo + 0.5 * st.dE);
+                    const double dEm = energy_of(fresh) - (st.E_lo + 0.5 * st.dE);
                     st.sum_dE += dEm;
                     st.sum_dE2 += dEm * dEm;
                     st.n_meas += 1;
@@ -2072,7 +2082,7 @@ __global__ void __launch_bounds__(kThreads, 1) llr_kernel(const __grid_constant_
                 energy_phase(sm, ph, args, true, false);
                 if (mine && args.e_hist)
                     args.e_hist[(size_t)j * (size_t)args.n_lat + (size_t)lat] =
-                        (double)sm.st[tid].E_fx * kInvFx;
+                        energy_of(sm.st[tid].E_fx);
                 break;
             }
             case kProgFinish:

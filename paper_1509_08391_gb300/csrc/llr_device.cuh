@@ -3,6 +3,7 @@
 // per-lattice state record.  Internal to the CUDA library.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -167,6 +168,16 @@ __device__ __forceinline__ float2 arg_fast2(float2 y, float2 x)
 // ---------------------------------------------------------------------------
 constexpr double kFx = 4294967296.0;   // 2^32
 constexpr double kInvFx = 1.0 / 4294967296.0;
+
+// The energy of a lattice whose links are no numbers (no lattice of L <= 64 has one
+// of this size), and what stands for it outside: a NaN.  FP64 energies that are NaN
+// convert to an even lower value.
+constexpr long long kNoEnergy = -(1ll << 62);
+
+__host__ __device__ inline double energy_of(long long fx)
+{
+    return fx <= kNoEnergy ? nan("") : (double)fx * kInvFx;
+}
 
 __device__ __forceinline__ long long to_fx(float v)
 {
