@@ -1021,7 +1021,9 @@ __device__ __forceinline__ bool muca_refuses_fast(const KernelArgs &a, long long
     if (k1 != k0) x -= (float)(a.muca_a[k1] - s0) * ((q1 - (float)max(k0, k1)) * a.muca_de_f);
     const float err = 1e-6f * (a.muca_jump * (1.0f + fabsf(q0) + fabsf(q1)) + fabsf(x)) + 1e-7f;
     const float e = __expf(x);
-    sure = abs(k1 - k0) <= 1 &&
+    // 2 err bounds exp(err) - 1 up to 1.25 (a table that starts 1e9 below the energies,
+    // where float32 places them to 32 only, has err in the thousands)
+    sure = abs(k1 - k0) <= 1 && err < 1.0f &&
            fabsf(u - e) > e * (2.0f * err + 4e-6f * (1.0f + fabsf(x))) + 1e-7f;
     return !(u < e);
 }

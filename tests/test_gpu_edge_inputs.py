@@ -2,7 +2,9 @@
 import numpy as np
 import pytest
 
+import oracle
 from paper_1509_08391_gb300 import llr, workloads
+from tests import gpu_helpers as gh
 
 pytestmark = pytest.mark.gpu
 
@@ -11,6 +13,7 @@ pytestmark = pytest.mark.gpu
 def _built():
     from paper_1509_08391_gb300 import build
     build.build()
+    oracle.build()
 
 
 @pytest.mark.parametrize("L", [4, 10, 12, 14])
@@ -47,3 +50,30 @@ def test_robbins_monro_step_reports_links_that_are_no_numbers():
             b.rm_step(np.array([-1.0, -1.0]), 0, 1, 0)
         assert e.value.code == llr.LLR_ERR_NUMERIC
         assert list(b.status()) == [0, llr.LLR_ERR_NUMERIC]
+
+
+@pytest.mark.parametrize("jump", [0.05, 2.0, 10.0])
+def test_multicanonical_decisions_far_from_the_table_origin(jump):
+    """A table that starts 1e9 below the energies, with a jump of the slope at
+    them: float32 places the energy to no better than 32, so only the exact form
+    of the accept test can decide."""
+    w = workloads.subset(workloads.small_l4(), range(4))
+    a0, de, n = -1.0, 1e8, 20
+    a = np.where(np.arange(n) < 10, -1.0, -1.0 + jump)
+    with llr.Batch.from_workload(w, max_approach=1000) as b:
+        b.sweep(np.full(w.n_lattices, -1.0), 1)
+        e0 = float(np.round(np.median(b.tracked_energy()))) - 10 * de   # edge 10: that energy
+        weight = oracle.MucaWeight(e0, de, a)
+        b.set_muca_weight(e0, de, a, a0)
+        for cls in (0, 3, 6):
+            mirrors = {i: gh.oracle_mirror(b, w, i) for i in range(w.n_lattices)}
+            S = {i: mirrors[i].staple_moduli() for i in mirrors}
+            b.single_pass(2, None, class_mask=1 << cls)
+            for i, o in mirrors.items():
+                tr = oracle.muca_class_trace(o, weight, cls, a0)
+                order = gh.class_links(w.L[i], cls)
+                d = np.abs(gh.wrapped_diff(b.get_links(i).astype(np.float64), o.links()))[order]
+                bad = np.nonzero(d > gh.link_tolerance(S[i])[order])[0]
+                if bad.size:   # the first difference must be a decision at a near tie
+                    k = int(bad[0])
+                    assert abs(np.log(tr["u"][k]) - tr["x"][k]) < 1e-4 * (1 + jump), (cls, i, k)
