@@ -309,13 +309,13 @@ int llr_muca_tunnellings(int n_steps, int n_chains, const double *E, double lo, 
                          int *out);
 
 /* Launch shape of the batched sweep kernel: the threads that work on one
- * lattice (128, 160, 192, 256 or 512).  A CTA has 768 threads and advances 6, 4,
- * 4, 3 or 1 lattices at a time accordingly, fewer where the batch has fewer for
- * every SM.  fast_math (1: hardware sine/cosine
- * approximations for the staples, 0: correctly rounded-class sincosf).
- * Chosen per lattice size by the autotuner; default 256 threads, fast math, and,
- * until a shape is set, more threads per lattice for batches of fewer lattices
- * than 3 per SM, fewer for L <= 6 and for many large lattices. */
+ * lattice.  A CTA has 768 threads and advances 6, 4, 4 or 1 lattices at a time
+ * for 128, 160, 192 or 512 of them, fewer where the batch has fewer for every
+ * SM.  256, the default, leaves the number to the batch's lattices: more threads
+ * each for batches of fewer lattices than 3 per SM, fewer for L <= 6 and for many
+ * large lattices.  fast_math (1: hardware sine/cosine approximations for the
+ * staples, 0: correctly rounded-class sincosf; default 1).
+ * Chosen per lattice size by the autotuner. */
 int llr_set_kernel_config(llr_handle h, int threads, int fast_math);
 
 /* The full launch shape of the batched sweep kernel, as the autotuner sets

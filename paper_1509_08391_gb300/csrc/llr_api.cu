@@ -714,7 +714,6 @@ int llr_set_kernel_shape(llr_handle h, int threads, int fast_math, int ring, int
     if (ring != 1 && ring != 2 && ring != 4) return fail(LLR_ERR_ARG, "ring must be 1, 2 or 4");
     if (carveout != -1 && carveout != 50 && carveout != 75 && carveout != 100)
         return fail(LLR_ERR_ARG, "carveout must be -1 (default), 50, 75 or 100");
-    h->cfg.auto_threads = false;
     h->cfg.threads = threads;
     h->cfg.fast_math = fast_math != 0;
     h->cfg.ring = ring;

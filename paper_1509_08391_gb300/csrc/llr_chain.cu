@@ -2266,8 +2266,8 @@ int prepare_kernel(int carveout)
 int choose_teams(const LaunchCfg &cfg, int n_lat, int sms, int max_L, bool one_slab)
 {
     int most = one_slab && n_lat >= 8 * sms ? 4 : 3;
-    if (!cfg.auto_threads)
-        most = cfg.threads >= 512 ? 1 : cfg.threads >= 256 ? 3 : cfg.threads >= 160 ? 4 : 6;
+    if (cfg.threads != 256)   // asked for
+        most = cfg.threads >= 512 ? 1 : cfg.threads >= 160 ? 4 : 6;
     else if (n_lat <= sms + sms / 2)
         most = 1;
     else if (max_L <= 6)

@@ -73,8 +73,7 @@ struct KernelArgs {
 cudaError_t launch_step_increment(int *step, cudaStream_t s);
 
 struct LaunchCfg {
-    bool auto_threads = true;   // until a shape is set: lattices per CTA by the batch's size
-    int threads = 256;    // most threads per lattice (128, 160, 192, 256 or 512)
+    int threads = 256;    // threads per lattice: 128, 160, 192 or 512, or 256: by the batch
     bool fast_math = true;
     int ring = 4;         // stages of the heat-bath producer/consumer ring in use: 1, 2 or 4
     int carveout = -1;    // shared-memory carve-out preference in percent, -1 = default

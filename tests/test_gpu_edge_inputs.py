@@ -77,3 +77,24 @@ def test_multicanonical_decisions_far_from_the_table_origin(jump):
                 if bad.size:   # the first difference must be a decision at a near tie
                     k = int(bad[0])
                     assert abs(np.log(tr["u"][k]) - tr["x"][k]) < 1e-4 * (1 + jump), (cls, i, k)
+
+
+def test_accurate_functions_keep_the_automatic_shape():
+    """Asking for the default shape, to change the functions only, leaves the
+    lattices per CTA to the batch, in a launch and in a captured step alike."""
+    import torch
+    w = workloads._grid("auto", [4], 200, 0.60, 0.66, [8.0], 1, 3)
+    a = np.full(w.n_lattices, -1.0)
+    ad = torch.full((w.n_lattices,), -1.0, dtype=torch.float64, device="cuda")
+    grids = []
+    with llr.Batch.from_workload(w, max_approach=0) as b:
+        for setting in (None, lambda: b.set_kernel_shape(256, True, 4, -1),
+                        lambda: b.set_kernel_config(256, False)):
+            if setting:
+                setting()
+            b.sweep(a, 1)
+            grids.append(b.last_launch()["grid"])
+            b.rm_run(ad, 0, 1, 0, 1)
+            torch.cuda.synchronize()
+            grids.append(b.last_launch()["grid"])
+    assert len(set(grids)) == 1, grids
