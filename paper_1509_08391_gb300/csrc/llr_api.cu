@@ -39,6 +39,7 @@ struct llr_ctx {
     unsigned long long wait_limit_ns = 20000000000ull;
     unsigned *d_sync = nullptr;      // work queue of the persistent kernel: 2 + n words
     int *d_order = nullptr;          // 0 .. n-1 (single-lattice launches point into it)
+    int *d_by_size = nullptr;        // lattices by falling side; null where all are alike
     int *d_step = nullptr;           // Robbins-Monro step counter of graph replays
     int *d_pairs = nullptr;          // replica-exchange pairs (n ints: at most n/2 pairs)
     // multicanonical weight: ln rho~ at the n + 1 edges, then the n slopes
@@ -84,6 +85,7 @@ llr::KernelArgs base_args(llr_handle h)
     a.lats = h->d_lat;
     a.theta = h->d_theta;
     a.n_lat = h->n;
+    a.order = h->d_by_size;
     a.n_or = h->n_or;
     a.block = h->block;
     a.beta_up = h->beta_up;
@@ -277,6 +279,18 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
         for (int i = 0; i < n; ++i) ord[(size_t)i] = i;
         LLR_CUDA(cudaMemcpy(h->d_order, ord.data(), sizeof(int) * (size_t)n,
                             cudaMemcpyHostToDevice));
+        // The lattices of a CTA advance phase by phase, so the smaller ones of a group
+        // wait for its largest: groups of like sides, the largest first, so that the
+        // small ones fill what is left.  300 each of L = 8 and 20 in random order: one
+        // sweep 23.8 -> 15.5 ms (20.9 one lattice to a CTA).
+        if (std::any_of(st.begin(), st.end(), [&](const LatState &s) { return s.L != max_L; })) {
+            std::stable_sort(ord.begin(), ord.end(), [&](int i, int j) {
+                return st[(size_t)i].L > st[(size_t)j].L;
+            });
+            LLR_CUDA(cudaMalloc(&h->d_by_size, sizeof(int) * (size_t)n));
+            LLR_CUDA(cudaMemcpy(h->d_by_size, ord.data(), sizeof(int) * (size_t)n,
+                                cudaMemcpyHostToDevice));
+        }
     }
     LLR_CUDA(cudaMemsetAsync(h->d_theta, 0, off * sizeof(float), h->stream));
     LLR_CUDA(cudaMemcpyAsync(h->d_lat, st.data(), sizeof(LatState) * (size_t)n,
@@ -797,6 +811,7 @@ int llr_destroy(llr_handle h)
     cudaFree(h->d_links);
     cudaFree(h->d_sync);
     cudaFree(h->d_order);
+    cudaFree(h->d_by_size);
     cudaFree(h->d_step);
     cudaFree(h->d_pairs);
     cudaFree(h->d_muca);

@@ -98,3 +98,28 @@ def test_accurate_functions_keep_the_automatic_shape():
             torch.cuda.synchronize()
             grids.append(b.last_launch()["grid"])
     assert len(set(grids)) == 1, grids
+
+
+def test_sides_that_alternate_give_the_chains_of_separate_batches():
+    """Several lattices of different sides to a CTA, in and out of shared memory:
+    every chain, history and energy is that of a batch of its side alone."""
+    import torch
+    for Ls in ([4, 8, 2], [4, 12, 6]):
+        n = 170
+        w = workloads._grid("mix", Ls, n, 0.60, 0.66, [16.0] * 3, 1, 9)
+        idx = [(i % 3) * n + i // 3 for i in range(3 * n)]
+        runs = {}
+        for part in (idx, list(range(n)), list(range(n, 2 * n)), list(range(2 * n, 3 * n))):
+            with llr.Batch.from_workload(workloads.subset(w, part), max_approach=0) as b:
+                app = b.approach(1000) if 2 not in Ls else np.zeros(len(part), dtype=np.int32)
+                a, mean = b.rm_step(np.full(len(part), -1.0), 1, 2, 3)
+                ad = torch.tensor(a, device="cuda")
+                hist = torch.zeros((2, len(part)), dtype=torch.float64, device="cuda")
+                b.rm_run(ad, 0, 2, 4, 2, hist)
+                E = b.tracked_energy()
+                h = hist.cpu().numpy()
+                for k, i in enumerate(part):
+                    got = (app[k], a[k], mean[k], E[k], h[0, k], h[1, k],
+                           hash(b.get_links(k).tobytes()))
+                    assert runs.setdefault(i, got) == got, (Ls, i)
+        assert len(runs) == 3 * n
