@@ -31,6 +31,7 @@ struct llr_ctx {
     size_t links_cap = 0;
     int max_half = 0;
     int max_L = 0;
+    int work = 1;                    // links in lattices of side max_L, rounded up
     int slab_L = 0;                  // largest L <= 24 (the sweep kernel's shared-memory slabs)
     int n_or = 4, block = 1;
     double beta_up = 1.5, beta_dn = 0.5;
@@ -94,6 +95,7 @@ llr::KernelArgs base_args(llr_handle h)
     a.sync = h->d_sync;
     a.wait_limit_ns = h->wait_limit_ns;
     a.max_L = h->max_L;
+    a.work = h->work;
     a.slab_L = h->slab_L;
     return a;
 }
@@ -259,6 +261,9 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
     h->h_lat = st;
     h->max_half = max_half;
     h->max_L = max_L;
+    long long halves = 0;
+    for (const LatState &s : st) halves += s.half;
+    h->work = (int)((halves + max_half - 1) / max_half);
     h->slab_L = slab_L;
     h->n_floats = off;
     cudaGetDevice(&h->device);

@@ -61,6 +61,7 @@
 // 2.7 -> 1.9 (184 -> 120), energy 1.3 -> 0.97, against one CTA of 256 threads per
 // lattice and one link per thread.
 #include <algorithm>
+#include <climits>
 #include <cstdio>
 
 #include "llr_internal.h"
@@ -2251,31 +2252,56 @@ int prepare_kernel(int carveout)
     return sms[dev];
 }
 
-// Lattices a CTA works on at a time.
-//   * One while there are not many more than SMs (time is one lattice's then), two,
-//     three.
-//   * Where a lattice's slab leaves no room for another's, so that overrelaxation
-//     takes them one by one anyway, and there are enough to go round evenly, a
-//     fourth keeps the heat-bath's schedulers fuller: a sweep of 1824 lattices of
-//     L = 20 takes 62.3 ms with three and 61.4 ms with four, a Robbins-Monro step of
-//     2048 362 and 348 ms; of L = 14, where it costs, 16.0 and 17.6 ms.
-//   * Up to six of L <= 6, whose classes (L^3 / 2 links of a slab, L^4 / 2 of the
-//     lattice) leave most of a third of the CTA idle: six sweeps of 4096 lattices of
-//     L = 2 / 4 / 6 take 4.0 / 5.7 / 10.9 ms with three, 2.5 / 3.6 / 7.7 ms with six; of
-//     L = 8 21.5 ms with three, 26.0 ms with six.
-int choose_teams(const LaunchCfg &cfg, int n_lat, int sms, int max_L, bool one_slab)
+// Lattices a CTA works on at a time: those that let the launch end soonest.
+//
+// A CTA takes longer over G lattices than over one, but less than G times as long.
+// kGroupTime is that ratio for a composite sweep, in percent (measured with 152 G
+// lattices, one group for every SM).  A launch of `groups` groups and per_lat sweeps
+// takes max(per_lat, groups per_lat / SMs) rounds of it.
+//   * L <= 6 leaves most of a CTA idle, so six go in little more than the time of one.
+//   * L = 8: up to three are held in shared memory.
+//   * L >= 18: the slabs go one or two at a time, and a fourth lattice keeps the
+//     heat-bath's schedulers fuller.
+//   * L > 24, read in place, was measured up to three.
+// One sweep of 200 lattices of L = 4 / 8 / 12: 0.247 / 0.613 / 1.97 ms one to a CTA,
+// 0.149 / 0.383 / 1.60 ms two to a CTA; six sweeps of 200 of L = 12 7.74 and 9.33 ms.
+constexpr int kGroupTime[6][7] = {
+    {0, 100, 108, 118, 130, 0, 155},   // L <= 6
+    {0, 100, 124, 145, 270, 0, 340},   // L = 8
+    {0, 100, 165, 214, 330, 0, 445},   // L = 10, 12
+    {0, 100, 156, 219, 322, 0, 440},   // L = 14, 16
+    {0, 100, 161, 252, 314, 0, 483},   // L = 18
+    {0, 100, 172, 254, 330, 0, 510},   // L >= 20
+};
+
+// work: the batch's lattices, counted in lattices of its largest side.
+int choose_teams(const LaunchCfg &cfg, int n_lat, int work, int per_lat, int sms, int max_L)
 {
-    int most = one_slab && n_lat >= 8 * sms ? 4 : 3;
-    if (cfg.threads != 256)   // asked for
-        most = cfg.threads >= 512 ? 1 : cfg.threads >= 160 ? 4 : 6;
-    else if (n_lat <= sms + sms / 2)
-        most = 1;
-    else if (max_L <= 6)
-        most = 6;
-    // no more than the batch has for every SM (152 lattices of L = 8 asked to run
-    // six to a CTA: 1.90 ms on 26 SMs, 0.65 ms on all)
-    const int each = (n_lat + sms - 1) / sms;
-    return each >= most ? most : each == 5 ? 4 : each;
+    if (cfg.threads != 256) {
+        // asked for, but no more than the batch has for every SM (152 lattices of
+        // L = 8 asked to run six to a CTA: 1.90 ms on 26 SMs, 0.65 ms on all)
+        const int most = cfg.threads >= 512 ? 1 : cfg.threads >= 160 ? 4 : 6;
+        const int each = (n_lat + sms - 1) / sms;
+        return each >= most ? most : each == 5 ? 4 : each;
+    }
+    const int *t = kGroupTime[max_L <= 6    ? 0
+                              : max_L <= 8  ? 1
+                              : max_L <= 12 ? 2
+                              : max_L <= 16 ? 3
+                              : max_L <= 18 ? 4
+                                            : 5];
+    int best = 1;
+    long long least = LLONG_MAX;
+    for (int g = 1; g <= (max_L > kSlabMaxL ? 3 : kMaxTeams); ++g) {
+        if (t[g] == 0) continue;
+        const long long items = (long long)((work + g - 1) / g) * per_lat;
+        const long long time = std::max<long long>(per_lat, (items + sms - 1) / sms) * t[g];
+        if (time < least) {
+            least = time;
+            best = g;
+        }
+    }
+    return best;
 }
 
 template <bool FAST>
@@ -2285,7 +2311,7 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     const int per_lat = multi ? (a.n_therm + a.n_meas) : 1;
     if ((long long)a.n_lat * per_lat <= 0) return cudaSuccess;
     const int sms = prepare_kernel<FAST>(cfg.carveout);
-    a.teams = choose_teams(cfg, a.n_lat, sms, a.max_L, a.slab_L > 0 && 2 * slab_bytes(a.slab_L) > kDynMax);
+    a.teams = choose_teams(cfg, a.n_lat, std::min(a.n_lat, a.work), per_lat, sms, a.max_L);
     // 15 named barriers, two per ring stage of each team
     const int most = a.teams == 1 ? 4 : a.teams <= 3 ? 2 : 1;
     a.ring = cfg.ring < most ? cfg.ring : most;

@@ -123,3 +123,17 @@ def test_sides_that_alternate_give_the_chains_of_separate_batches():
                            hash(b.get_links(k).tobytes()))
                     assert runs.setdefault(i, got) == got, (Ls, i)
         assert len(runs) == 3 * n
+
+
+@pytest.mark.parametrize("L,n,sweeps,grid", [(4, 160, 1, 80), (8, 200, 1, 100), (12, 200, 1, 100),
+                                             (12, 200, 12, 152), (8, 152, 1, 152)])
+def test_lattices_per_cta_follow_the_rounds_a_launch_takes(L, n, sweeps, grid):
+    """Somewhat more lattices than SMs: two to a CTA for a sweep of which the GPU
+    would otherwise take two rounds, one where the rounds of many sweeps fill it."""
+    import torch
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("the sizes are those of 152 SMs")
+    w = workloads._grid("rounds", [L], n, 0.60, 0.66, [8.0], 1, 3)
+    with llr.Batch.from_workload(w, max_approach=0) as b:
+        b.sweep(np.full(n, -1.0), sweeps)
+        assert b.last_launch()["grid"] == grid
