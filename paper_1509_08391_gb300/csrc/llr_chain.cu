@@ -2328,7 +2328,12 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     // thread for each of the L^3 / 2 links of a slab's class
     const int links = a.max_L <= kResidentMaxL ? a.max_L * a.max_L * a.max_L / 2 : kThreads;
     const int or_most = links <= kWarps / a.teams * 32 ? a.teams : std::min(a.teams, 3);
-    a.resident = a.max_L <= kResidentMaxL && lattices + stage1 <= kDynMax &&
+    // A launch that only sums energies reads every angle a few times and writes none:
+    // lattices stay where they are (2000 of L = 4 / 8: 66 / 217 us copied in, 58 / 169).
+    const bool sums = a.program == kProgResync || a.program == kProgFinish ||
+                      a.program == kProgBegin || a.program == kProgUpdate ||
+                      (a.program == kProgPass && a.pass_kind == 3);
+    a.resident = !sums && a.max_L <= kResidentMaxL && lattices + stage1 <= kDynMax &&
                  links <= kWarps / or_most * 32;
     while (a.resident && lattices + stage1 * a.ring > kDynMax) a.ring >>= 1;
     size_t rings = stage1 * a.ring;
@@ -2338,6 +2343,10 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
         a.slab = (int)(lattice_bytes(a.max_L) / sizeof(float));
         a.ring_off = (int)(lattices / sizeof(float));
         dyn = lattices + rings;
+    } else if (sums) {
+        a.or_teams = 1;
+        a.slab = a.ring_off = 0;
+        dyn = 0;
     } else {
         const size_t slab = a.slab_L > 0 ? slab_bytes(a.slab_L) : 0;
         const size_t stage = (size_t)kStaged * kThreads * sizeof(float2);
