@@ -322,10 +322,10 @@ int llr_set_kernel_config(llr_handle h, int threads, int fast_math);
  * it; none of these changes the chains (every shape runs the same per-link
  * arithmetic in the same order), only the speed.
  *   threads, fast_math: as llr_set_kernel_config.
- *   ring: the most stages of the heat-bath producer/consumer ring in use, 1, 2
- *     or 4 (how many chunks the proposing warps may run ahead of the warp that
- *     takes the window decisions; fewer where shared memory or the lattices per
- *     CTA leave no room).
+ *   ring: the most stages of the heat-bath producer/consumer ring, 1, 2 or 4
+ *     (how many chunks the proposing warps may run ahead of the warp that
+ *     takes the window decisions); never more than two are used, and one where
+ *     shared memory or the lattices per CTA leave no room.
  *   carveout: preferred share of the SM's unified L1/shared storage given to
  *     shared memory, in percent: 50, 75 or 100, or -1 for the driver's default
  *     (a hint; it is a property of the kernel variant in this process, so the

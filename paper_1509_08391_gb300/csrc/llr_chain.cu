@@ -39,7 +39,7 @@
 //     dist(E + dE_block) <= dist(E), using a ballot to find the first rejected
 //     block among those of 32 speculatively accepted links, and publishes the
 //     accepted links; the producers write their angles.  Chunks pass through a ring of
-//     1 to 4 stages in shared memory guarded by named barriers, so proposals
+//     1 or 2 stages in shared memory guarded by named barriers, so proposals
 //     for later chunks overlap with the scan of earlier ones.
 //   * The multicanonical pass (Sec. 2.6) has the same producers at a fixed
 //     proposal slope; its consumer replaces the window rule by a
@@ -390,6 +390,14 @@ __device__ __forceinline__ void staple_sums2(Get v, float2 &Sr, float2 &Si)
 // Threads of the sweep kernel's CTA (one CTA per SM, 80 registers a thread) and
 // the lattices one CTA works on at a time, each with a team of warps.
 constexpr int kThreads = 768, kWarps = kThreads / 32, kMaxTeams = 6;
+
+// Most producer warps of a lattice's heat-bath team, which are the 64-link groups of
+// a ring stage: one warp decides, and for a lone lattice, where that warp is the
+// bound, it has a quarter of the SM (a scheduler) to itself.
+__host__ __device__ constexpr int producers(int teams)
+{
+    return teams == 1 ? kWarps / 4 * 3 : kWarps / teams - 1;
+}
 
 // Dynamic shared memory: the whole lattices where they fit (RES; then the
 // heat-bath rings), otherwise used by one phase of a sweep at a time: the
@@ -1601,16 +1609,15 @@ __device__ __noinline__ void heatbath_phase(Smem &sm, const Phase &ph, const Ker
         const int k = threadIdx.x;
         sm.acc_cnt[k] = 0ull;
         HbTeam &hb = sm.hb[k];
-        // No more producers than groups.  With one lattice the deciding warp is the
-        // bound, so it has a quarter of the SM (a scheduler) to itself.
-        const int most = ph.teams == 1 ? kWarps / 4 * 3 + 1 : ph.tw;
-        hb.nw = min(most, 1 + (sm.st[k].half + 63) / 64);
+        // no more producers than groups
+        const int most = producers(ph.teams);
+        hb.nw = 1 + min(most, (sm.st[k].half + 63) / 64);
         // the consumers of different teams on different quarters of the SM
         hb.cw = hb.nw - 1;
         for (int c = hb.nw - 1; c >= max(0, hb.nw - 4); --c)
             if (((k * ph.tw + c) & 3) == 3 - (k & 3)) hb.cw = c;
         hb.D = ph.D;
-        hb.ring = ph.ring + k * ph.D * (ph.tw - 1) * (kStageGroupBytes / 4);
+        hb.ring = ph.ring + k * ph.D * most * (kStageGroupBytes / 4);
         hb.full = 1 + 2 * ph.D * k;
     }
     __syncthreads();
@@ -2312,16 +2319,12 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     if ((long long)a.n_lat * per_lat <= 0) return cudaSuccess;
     const int sms = prepare_kernel<FAST>(cfg.carveout);
     a.teams = choose_teams(cfg, a.n_lat, std::min(a.n_lat, a.work), per_lat, sms, a.max_L);
-    // 15 named barriers, two per ring stage of each team
-    const int most = a.teams == 1 ? 4 : a.teams <= 3 ? 2 : 1;
+    // Two stages, where there are barriers for them (15 named ones, two per ring stage
+    // of each team).  Four take L1 from the other passes: ten sweeps of 128 of L = 20
+    // 63.2 ms, 60.9 with two, 59.7 with one; of L = 12 9.77, 9.66 and 9.85.
+    const int most = a.teams <= 3 ? 2 : 1;
     a.ring = cfg.ring < most ? cfg.ring : most;
-    const int groups = kWarps / a.teams - 1;
-    // two stages serve a class of two chunks (128 of L = 8: a sweep 0.272 ms with
-    // two, 0.285 ms with four); longer classes use all (152 of L = 20 6.50, 6.60 ms
-    // with one)
-    if (a.ring > 2 && a.max_L <= kResidentMaxL &&
-        a.max_L * a.max_L * a.max_L * a.max_L / 2 <= 2 * 64 * groups)
-        a.ring = 2;
+    const int groups = producers(a.teams);
     const size_t stage1 = (size_t)a.teams * groups * kStageGroupBytes;
     const size_t lattices = (size_t)a.teams * lattice_bytes(a.max_L);
     // a lattice may be resident if a team of the overrelaxation pass has a

@@ -76,7 +76,7 @@ cudaError_t launch_step_increment(int *step, cudaStream_t s);
 struct LaunchCfg {
     int threads = 256;    // threads per lattice: 128, 160, 192 or 512, or 256: by the batch
     bool fast_math = true;
-    int ring = 4;         // stages of the heat-bath producer/consumer ring in use: 1, 2 or 4
+    int ring = 4;         // most stages of the heat-bath ring: 1, 2 or 4 (two at most are used)
     int carveout = -1;    // shared-memory carve-out preference in percent, -1 = default
 };
 
