@@ -857,7 +857,7 @@ struct MucaSamples {
     static constexpr int kBetaBatch = 512;
     DevBuf buf;
     long long ns = 0;
-    int gx = 1;
+    int gx = 1, parts = 1, wave = 1;   // blocks, parts of the table form, its blocks in all
     double shift = 0.0;
     double reach = 0.0, lr_reach = 0.0;   // bounds of |E - shift| and |ln rho~| over the samples
     double *tab = nullptr;
@@ -908,9 +908,14 @@ int muca_samples_init(MucaSamples &w, long long ns, const double *E, int n, doub
     int dev = 0, sms = 1;
     LLR_CUDA(cudaGetDevice(&dev));
     LLR_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    // sample blocks per coupling: two per SM, none without samples
+    // sample blocks per coupling: two per SM, none without samples.  In the table form a
+    // part for every SM, of 2048 samples at least, since a part's end costs as much as
+    // some hundred samples (300 couplings of 2000000 samples: 16.8 ms, with two parts per
+    // SM 17.5), on three blocks per SM (by registers).
     const long long tiles = (ns + 255) / 256;
     w.gx = (int)std::max(1LL, std::min(tiles, 2LL * sms));
+    w.parts = (int)std::max(1LL, std::min(tiles / 8, 1LL * sms));
+    w.wave = 3 * sms;
     w.ns = ns;
     w.shift = e0;
     const int nb = MucaSamples::kBetaBatch;
@@ -937,18 +942,19 @@ int muca_samples_init(MucaSamples &w, long long ns, const double *E, int n, doub
 }
 
 // <E>, <E^2> and <E^2> - <E>^2 at nb couplings (host arrays; any output may
-// be null), kBetaBatch couplings per launch.
+// be null), up to kBetaBatch couplings per launch.  Each coupling takes the form that
+// its own exponents allow, so its result does not depend on the others.
 int muca_moments(MucaSamples &w, int nb, const double *beta, double *E1, double *E2, double *var)
 {
-    for (int b0 = 0; b0 < nb; b0 += MucaSamples::kBetaBatch) {
-        const int m = std::min(MucaSamples::kBetaBatch, nb - b0);
+    auto fits = [&](double b) { return std::fabs(b) * w.reach + w.lr_reach < 549755813888.0; };   // 2^39
+    for (int b0 = 0, m = 1; b0 < nb; b0 += m) {
+        const bool small = fits(beta[b0]);
+        for (m = 1; b0 + m < nb && m < MucaSamples::kBetaBatch && fits(beta[b0 + m]) == small;) ++m;
         LLR_CUDA(cudaMemcpy(w.beta, beta + b0, sizeof(double) * (size_t)m,
                             cudaMemcpyHostToDevice));
-        double most = 0.0;
-        for (int i = 0; i < m; ++i) most = std::max(most, std::fabs(beta[b0 + i]));
-        const bool small = most * w.reach + w.lr_reach < 549755813888.0;   // 2^39
         LLR_CUDA(llr::launch_reweight(w.ns, w.E, w.lr, w.shift, m, w.beta, small ? w.tab : nullptr,
-                                      w.gx, w.part, w.E1, w.E2, w.var, nullptr));
+                                      small ? w.parts : w.gx, w.wave, w.part, w.E1, w.E2, w.var,
+                                      nullptr));
         const size_t bytes = sizeof(double) * (size_t)m;
         if (E1) LLR_CUDA(cudaMemcpy(E1 + b0, w.E1, bytes, cudaMemcpyDeviceToHost));
         if (E2) LLR_CUDA(cudaMemcpy(E2 + b0, w.E2, bytes, cudaMemcpyDeviceToHost));

@@ -137,12 +137,13 @@ cudaError_t launch_muca_lnrho(long long ns, const double *E, const double *lnr, 
                               int n, double e0, double de, double *out, int grid,
                               cudaStream_t s);
 // tab: launch_reweight_table's reweight_table_doubles() doubles, or null where an
-// exponent beta (E - shift) + lr may exceed 2^39 in size.
+// exponent beta (E - shift) + lr may exceed 2^39 in size.  wave: blocks of the table
+// form to launch at most, about (one wave on the GPU).
 size_t reweight_table_doubles();
 cudaError_t launch_reweight_table(double *tab, cudaStream_t s);
 cudaError_t launch_reweight(long long ns, const double *E, const double *lr, double shift,
                             int n_beta, const double *beta, const double *tab, int gx,
-                            double *part, double *E1, double *E2, double *var, cudaStream_t s);
+                            int wave, double *part, double *E1, double *E2, double *var, cudaStream_t s);
 cudaError_t launch_tunnellings(int n_steps, int n_chains, const double *E, double lo, double hi,
                                int *out, cudaStream_t s);
 

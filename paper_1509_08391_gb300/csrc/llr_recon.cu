@@ -378,10 +378,11 @@ __global__ void __launch_bounds__(kT) reweight_partial_kernel(long long ns, cons
 // exponent field, and the sums' scale is an exact power of two, found and kept as
 // an integer.  12 FP64 operations per sample and coupling (87 % of the pipe's time)
 // where the library's exp and the running maximum took about twice as many, and
-// fewer, longer blocks: a coupling of 512000 samples 47 us -> 18 us.  The exponent
+// fewer, longer blocks: a coupling of 512000 samples among 300 50 us -> 15 us.  The exponent
 // is formed over d = E - shift, whose rounding is smaller than E's.  Writes
 // (N, s0, s1, s2), s_j = sum d^j exp(b d + lr) / 2^N.
 constexpr int kExpBits = 11, kExpTable = 1 << kExpBits;
+constexpr long long kNoTerm = -(1ll << 62);   // the scale before the first term
 
 __global__ void __launch_bounds__(kT) exp_table_kernel(double *tab)
 {
@@ -389,71 +390,140 @@ __global__ void __launch_bounds__(kT) exp_table_kernel(double *tab)
     if (j < kExpTable) tab[j] = exp2((double)j / kExpTable);
 }
 
+// 2^-d, d >= 0, from the exponent field (0 below the normal numbers).
+__device__ __forceinline__ double pow2_down(long long d)
+{
+    return d < 1022 ? __hiloint2double((1023 - (int)d) << 20, 0) : 0.0;
+}
+
+// Sums of n values over a warp, every value in the order of a xor butterfly; a
+// step hands half of the values to each half of the lanes, so 12 values take 13
+// additions and not 60 (the FP64 pipe is the kernel's bound).  Returns which value
+// the lane's v[0] is the sum of (n or more: none; one lane for every value).
+template <int n, int o = 16>
+__device__ __forceinline__ int warp_sums(double *v, int lane)
+{
+    if constexpr (o == 0) {
+        return 0;
+    } else if constexpr (n == 1) {
+        v[0] += __shfl_xor_sync(kFull, v[0], o);
+        const int at = warp_sums<1, o / 2>(v, lane);
+        return (lane & o) ? 1 : at;   // one lane answers
+    } else {
+        constexpr int h = (n + 1) / 2;
+        const bool up = lane & o;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+            const double other = i + h < n ? v[i + h] : 0.0;
+            const double give = up ? v[i] : other, keep = up ? other : v[i];
+            v[i] = keep + __shfl_xor_sync(kFull, give, o);
+        }
+        const int at = warp_sums<h, o / 2>(v, lane);
+        return at < h && at + (up ? h : 0) < n ? at + (up ? h : 0) : n;
+    }
+}
+
+// Part x of the samples: tiles x, x + parts, ...  A block takes parts blockIdx.x,
+// blockIdx.x + gridDim.x, ... for its couplings.  The parts are set by the number of
+// samples alone and each is summed in an order of its own, so a coupling's result
+// does not depend on how many are asked for with it.
 template <int NB>
-__global__ void __launch_bounds__(kT) reweight_table_kernel(long long ns, const double *E,
-                                                            const double *lr, double shift,
-                                                            int n_beta, const double *beta,
+__global__ void __launch_bounds__(kT) reweight_table_kernel(long long ns, int parts,
+                                                            const double *E, const double *lr,
+                                                            double shift, int n_beta,
+                                                            const double *beta,
                                                             const double *tab, double *part)
 {
     __shared__ double T[kExpTable];
-    __shared__ double red[kT / 32];
+    static_assert(kT / 32 == 8 && (NB == 1 || NB == 4), "the first warp has a lane for each sum");
+    __shared__ long long redN[2][8][NB];
+    __shared__ double redS[2][8][3 * NB];
     constexpr double kMagic = 6755399441055744.0;   // 1.5 2^52: rounds to an integer in the low bits
     constexpr double kInv = 2954.639443740597;     // 2048 / ln 2
     constexpr double kHi = 3.384507717577858e-4;   // ln 2 / 2048, and what its rounding leaves
     constexpr double kLo = 1.1323470770733885e-20;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     for (int j = threadIdx.x; j < kExpTable; j += kT) T[j] = tab[j];
     const int b0 = blockIdx.y * NB;
-    double b[NB], s0[NB], s1[NB], s2[NB];
-    long long N[NB];
+    double b[NB];
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-        b[q] = beta[min(b0 + q, n_beta - 1)];
-        s0[q] = s1[q] = s2[q] = 0.0;
-        N[q] = LLONG_MIN;
-    }
+    for (int q = 0; q < NB; ++q) b[q] = beta[min(b0 + q, n_beta - 1)];
     __syncthreads();
-    const long long stride = (long long)gridDim.x * kT;
-    for (long long i = (long long)blockIdx.x * kT + threadIdx.x; i < ns; i += stride) {
-        const double d = E[i] - shift, l = lr[i], d2 = d * d;
+    const long long stride = (long long)parts * kT;
+    for (int x = blockIdx.x, buf = 0; x < parts; x += gridDim.x, buf ^= 1) {
+        double s0[NB], s1[NB], s2[NB];
+        long long N[NB];
 #pragma unroll
         for (int q = 0; q < NB; ++q) {
-            const double y = fma(b[q], d, l);
-            const double kd = fma(y, kInv, kMagic);
-            const double kf = kd - kMagic;
-            const double r = fma(kf, -kLo, fma(kf, -kHi, y));
-            const long long k = __double_as_longlong(kd) - 0x4338000000000000ll;
-            const long long n = k >> kExpBits;   // power of two
-            if (n > N[q]) {   // a larger term than any before: rescale, rarely
-                const double f = N[q] == LLONG_MIN ? 0.0 : exp2((double)(N[q] - n));
-                s0[q] *= f;
-                s1[q] *= f;
-                s2[q] *= f;
-                N[q] = n;
-            }
-            const double t = T[(int)k & (kExpTable - 1)];
-            double w = fma(t, r * fma(r, fma(r, 1.0 / 6.0, 0.5), 1.0), t);   // in [1, 2)
-            const long long down = N[q] - n;
-            w = down < 1000 ? __hiloint2double(__double2hiint(w) - ((int)down << 20),
-                                               __double2loint(w))
-                            : 0.0;
-            s0[q] += w;
-            s1[q] = fma(d, w, s1[q]);
-            s2[q] = fma(d2, w, s2[q]);
+            s0[q] = s1[q] = s2[q] = 0.0;
+            N[q] = kNoTerm;
         }
-    }
+        for (long long i = (long long)x * kT + threadIdx.x; i < ns; i += stride) {
+            const double d = E[i] - shift, l = lr[i], d2 = d * d;
 #pragma unroll
-    for (int q = 0; q < NB; ++q) {
-        const double nq = N[q] == LLONG_MIN ? -INFINITY : (double)N[q];
-        const double M = block_max(nq, red);
-        const double f = N[q] == LLONG_MIN ? 0.0 : exp2(nq - M);
-        const double t0 = block_sum(s0[q] * f, red), t1 = block_sum(s1[q] * f, red),
-                     t2 = block_sum(s2[q] * f, red);
-        if (threadIdx.x == 0 && b0 + q < n_beta) {
-            double *p = part + 4 * ((size_t)(b0 + q) * gridDim.x + blockIdx.x);
-            p[0] = M;
-            p[1] = t0;
-            p[2] = t1;
-            p[3] = t2;
+            for (int q = 0; q < NB; ++q) {
+                const double y = fma(b[q], d, l);
+                const double kd = fma(y, kInv, kMagic);
+                const double kf = kd - kMagic;
+                const double r = fma(kf, -kLo, fma(kf, -kHi, y));
+                const long long k = __double_as_longlong(kd) - 0x4338000000000000ll;
+                const long long n = k >> kExpBits;   // power of two
+                if (n > N[q]) {   // a larger term than any before: rescale, rarely
+                    const double f = pow2_down(n - N[q]);
+                    s0[q] *= f;
+                    s1[q] *= f;
+                    s2[q] *= f;
+                    N[q] = n;
+                }
+                const double t = T[(int)k & (kExpTable - 1)];
+                double w = fma(t, r * fma(r, fma(r, 1.0 / 6.0, 0.5), 1.0), t);   // in [1, 2)
+                const long long down = N[q] - n;
+                w = down < 1000 ? __hiloint2double(__double2hiint(w) - ((int)down << 20),
+                                                   __double2loint(w))
+                                : 0.0;
+                s0[q] += w;
+                s1[q] = fma(d, w, s1[q]);
+                s2[q] = fma(d2, w, s2[q]);
+            }
+        }
+        // the block's sums: within the warps, then over them
+        double v[3 * NB];
+#pragma unroll
+        for (int q = 0; q < NB; ++q) {
+            long long M = N[q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) M = max(M, __shfl_xor_sync(kFull, M, o));
+            const double f = pow2_down(M - N[q]);
+            v[3 * q] = s0[q] * f;
+            v[3 * q + 1] = s1[q] * f;
+            v[3 * q + 2] = s2[q] * f;
+            if (lane == 0) redN[buf][warp][q] = M;
+        }
+        const int at = warp_sums<3 * NB>(v, lane);
+        if (at < 3 * NB) redS[buf][warp][at] = v[0];
+        __syncthreads();
+        // lane 8 q + w of the first warp: warp w's sums of coupling q.  The other warps
+        // go on to the next part, which has the other buffer.
+        const int q = lane >> 3, w = lane & 7;
+        if (warp == 0 && q < NB) {
+            const unsigned lanes = NB == 4 ? kFull : (1u << (8 * NB)) - 1u;
+            const long long n = redN[buf][w][q];
+            long long M = n;
+            for (int o = 4; o > 0; o >>= 1) M = max(M, __shfl_xor_sync(lanes, M, o));
+            const double f = pow2_down(M - n);
+            double t[3];
+#pragma unroll
+            for (int m = 0; m < 3; ++m) {
+                t[m] = redS[buf][w][3 * q + m] * f;
+                for (int o = 4; o > 0; o >>= 1) t[m] += __shfl_xor_sync(lanes, t[m], o);
+            }
+            if (w == 0 && b0 + q < n_beta) {
+                double *p = part + 4 * ((size_t)(b0 + q) * parts + x);
+                p[0] = (double)M;
+                p[1] = t[0];
+                p[2] = t[1];
+                p[3] = t[2];
+            }
         }
     }
 }
@@ -536,21 +606,21 @@ cudaError_t launch_reweight_table(double *tab, cudaStream_t s)
 
 cudaError_t launch_reweight(long long ns, const double *E, const double *lr, double shift,
                             int n_beta, const double *beta, const double *tab, int gx,
-                            double *part, double *E1, double *E2, double *var, cudaStream_t s)
+                            int wave, double *part, double *E1, double *E2, double *var, cudaStream_t s)
 {
     if (n_beta <= 0) return cudaSuccess;
     constexpr int NB = 4;   // couplings a block: samples and table are read once for all
     if (tab && n_beta >= NB) {
-        // one wave over all couplings (three blocks an SM by registers; gx is two): a
-        // block's table and reductions cost as much as some thousand samples
+        // one wave over all couplings: a block's table costs as much as some hundred
+        // samples
         const int groups = (n_beta + NB - 1) / NB;
-        gx = std::max(1, std::min(gx, 3 * gx / 2 / groups));
-        reweight_table_kernel<NB><<<dim3(gx, groups), kT, 0, s>>>(ns, E, lr, shift, n_beta, beta,
-                                                                 tab, part);
+        const int bx = std::max(1, std::min(gx, wave / groups));
+        reweight_table_kernel<NB><<<dim3(bx, groups), kT, 0, s>>>(ns, gx, E, lr, shift, n_beta,
+                                                                 beta, tab, part);
     }
     else if (tab)
-        reweight_table_kernel<1><<<dim3(gx, n_beta), kT, 0, s>>>(ns, E, lr, shift, n_beta, beta,
-                                                                 tab, part);
+        reweight_table_kernel<1><<<dim3(gx, n_beta), kT, 0, s>>>(ns, gx, E, lr, shift, n_beta,
+                                                                 beta, tab, part);
     else
         reweight_partial_kernel<<<dim3(gx, n_beta), kT, 0, s>>>(ns, E, lr, shift, beta, part);
     reweight_combine_kernel<<<n_beta, kT, 0, s>>>(gx, part, tab != nullptr, shift, E1, E2, var);

@@ -137,3 +137,19 @@ def test_lattices_per_cta_follow_the_rounds_a_launch_takes(L, n, sweeps, grid):
     with llr.Batch.from_workload(w, max_approach=0) as b:
         b.sweep(np.full(n, -1.0), sweeps)
         assert b.last_launch()["grid"] == grid
+
+
+def test_a_coupling_does_not_depend_on_those_asked_for_with_it():
+    """Bit for bit, for few and many couplings a launch, whole and ragged groups."""
+    rng = np.random.default_rng(3)
+    E = rng.normal(37000.0, 150.0, 200000)
+    a = -1.0 + 1e-3 * rng.normal(size=64)
+    betas = np.linspace(0.99, 1.01, 301)
+
+    def f(b):
+        return np.array(llr.muca_reweight(E, 36000.0, 2000 / 64, a, b))
+
+    ref = f(betas)
+    for k in (1, 3, 4, 5, 43):
+        got = np.concatenate([f(betas[i:i + k]) for i in range(0, betas.size, k)], axis=1)
+        assert np.array_equal(got, ref), k
