@@ -42,7 +42,7 @@ def parse():
     p.add_argument("--n-therm", type=int, default=2)
     p.add_argument("--n-meas", type=int, default=8)
     p.add_argument("--threads", type=int, default=0,
-                   help="threads per lattice (128/256/512); 0 = autotuned")
+                   help="threads per lattice (128/160/512, 256 = the library's choice); 0 = autotuned")
     p.add_argument("--no-e2e", action="store_true")
     p.add_argument("--no-cpu", action="store_true")
     p.add_argument("--intervals", type=int, default=256)
@@ -197,7 +197,7 @@ def config_dict(args, w, world):
             "sweeps_per_step": args.n_therm + args.n_meas, "n_therm": args.n_therm,
             "n_meas": args.n_meas, "accept_block": w.block,
             "parallelism": "dp%d (independent lattices, no collective)" % world,
-            "threads_per_cta": getattr(args, "threads_used", args.threads),
+            "threads_per_lattice": getattr(args, "threads_used", args.threads),
             "launch_shape": getattr(args, "shape_used", None),
             "l2": "inputs larger than L2 (5.2 GB of links per GPU)"}
 

@@ -21,11 +21,12 @@
 //     that sweep.  Items run sweep-major, so uneven lattice sizes balance
 //     across SMs.  The lattices of an item advance together, phase by phase
 //     (heat-bath pass, overrelaxation passes, energy).
-//   * Lattices per item (choose_teams): with fewer lattices than SMs, one with
-//     all 24 warps; with many, three with 8 warps each or four with 6 in the
-//     heat-bath pass, whose deciding warps are serial and need company, while
-//     the overrelaxation pass takes up to three together, or one after another
-//     where a slab fills the shared memory; up to six of L <= 6.
+//   * Lattices per item (choose_teams, by the time the launch takes): with fewer
+//     lattices than SMs, one with all 24 warps; with many, three with 8 warps
+//     each or four with 6 in the heat-bath pass, whose deciding warps are serial
+//     and need company, while the overrelaxation pass takes up to three together,
+//     or one after another where a slab fills the shared memory; six of L <= 6.
+//     Lattices of an uneven batch are taken by falling side, so like ones meet.
 //   * A heat-bath pass runs class by class over the whole lattice (one
 //     pipeline drain per class); an overrelaxation pass is slab-major: for
 //     each x3 slab, all 8 checkerboard classes of that slab in order.
@@ -163,9 +164,6 @@ __device__ __forceinline__ void von_mises2(float kappa0, float kappa1, uint32_t 
                                            uint32_t k0, uint32_t k1, float2 &cX, float2 &sX,
                                            bool &ok0, bool &ok1)
 {
-    // keep the round keys from being hoisted out of the caller's loop: 18 more
-    // live registers would be spilled
-    //KEY
     const VonMises v0(kappa0), v1(kappa1);
     const bool flat0 = fabsf(kappa0) < kKappaFlat, flat1 = fabsf(kappa1) < kKappaFlat;
     const U4 w0 = philox4x32_10(link0, sweep, tag, 0u, k0, k1);
@@ -649,7 +647,7 @@ __device__ __noinline__ void produce_class(Smem &sm, int slot, int pw, float *th
 }
 
 // Neighbour angles of link theta_MU(x) (site s, parity p) loaded straight into
-// registers v[18], in the order of staple_fetch.
+// registers v[18], in the order of neighbour_pairs.
 template <int MU>
 __device__ __forceinline__ void staple_load(const float *th, int half, int L, const int x[4],
                                             int s, int p, float v[18])
@@ -681,7 +679,7 @@ __device__ __forceinline__ void staple_load(const float *th, int half, int L, co
 }
 
 // Staple sum of one link from its 18 neighbour angles, formed exactly as in
-// staple_from.
+// staple_sums2.
 template <bool FAST>
 __device__ __forceinline__ void staple_sum_regs(const float v[18], float &Sr, float &Si)
 {
@@ -1304,7 +1302,7 @@ __device__ __forceinline__ void reflect_pair(const SlabGeo &g, int x2, int h, in
             b3 = g2;
             b1 = g3;
         }
-        // the staple sums of both links, formed exactly as in staple_from
+        // the staple sums of both links, formed exactly as in staple_sums2
         const float2 pf = sub2(sub2(a1, a2), a3), pb = sub2(sub2(b3, b1), b2);
         float2 sf, cf, sb, cb;
         sin_cos<FAST>(pf.x, &sf.x, &cf.x);

@@ -290,7 +290,10 @@ __global__ void __launch_bounds__(kT) golden_result_kernel(int n, const double *
     }
 }
 
-// Rounds that are sure to reach the tolerance (two steps of slack for rounding).
+// Rounds that are sure to reach the tolerance (two steps of slack for rounding), or,
+// for one below a few units in the last place of the couplings, the width at which
+// the interval stops shrinking (the steps a longer search would add leave its
+// middle where it is).
 int golden_rounds(double blo, double bhi, int n_grid, double tol)
 {
     const double len = 2.0 * (bhi - blo) / (double)(n_grid - 1);
