@@ -32,6 +32,7 @@ struct llr_ctx {
     int max_half = 0;
     int max_L = 0;
     int work = 1;                    // links in lattices of side max_L, rounded up
+    double inv_width = 0.0;          // mean 1 / dE
     int slab_L = 0;                  // largest L <= 24 (the sweep kernel's shared-memory slabs)
     int n_or = 4, block = 1;
     double beta_up = 1.5, beta_dn = 0.5;
@@ -96,6 +97,7 @@ llr::KernelArgs base_args(llr_handle h)
     a.wait_limit_ns = h->wait_limit_ns;
     a.max_L = h->max_L;
     a.work = h->work;
+    a.inv_width = h->inv_width;
     a.slab_L = h->slab_L;
     return a;
 }
@@ -262,7 +264,10 @@ int llr_init_lattice(llr_handle *out, const llr_config *cfg, void *cuda_stream)
     h->max_half = max_half;
     h->max_L = max_L;
     long long halves = 0;
-    for (const LatState &s : st) halves += s.half;
+    for (const LatState &s : st) {
+        halves += s.half;
+        h->inv_width += 1.0 / s.dE / n;
+    }
     h->work = (int)((halves + max_half - 1) / max_half);
     h->slab_L = slab_L;
     h->n_floats = off;

@@ -62,7 +62,7 @@
 // 2.7 -> 1.9 (184 -> 120), energy 1.3 -> 0.97, against one CTA of 256 threads per
 // lattice and one link per thread.
 #include <algorithm>
-#include <climits>
+#include <cmath>
 #include <cstdio>
 
 #include "llr_internal.h"
@@ -2260,50 +2260,74 @@ int prepare_kernel(int carveout)
 // Lattices a CTA works on at a time: those that let the launch end soonest.
 //
 // A CTA takes longer over G lattices than over one, but less than G times as long.
-// kGroupTime is that ratio for a composite sweep, in percent (measured with 152 G
-// lattices, one group for every SM).  A launch of `groups` groups and per_lat sweeps
-// takes max(per_lat, groups per_lat / SMs) rounds of it.
+// kGroupTime has what the phases of a composite sweep take for G = 1, 2, 3, 4, 6, in
+// percent of the sweep of one (measured with 152 G lattices and windows of width L^2 / 8;
+// the rest: four overrelaxation passes and the energy).
 //   * L <= 6 leaves most of a CTA idle, so six go in little more than the time of one.
 //   * L = 8: up to three are held in shared memory.
 //   * L >= 18: the slabs go one or two at a time, and a fourth lattice keeps the
 //     heat-bath's schedulers fuller.
-//   * L > 24, read in place, was measured up to three.
+// A deciding warp takes 2.75 + 40 / width ns a link (6.0, 9.4 and 12.7 measured at widths
+// 12, 6 and 4; 22 in a multicanonical pass): in narrow windows it is the heat-bath's
+// bound and company costs less.  The two times are joined by the sum of their cubes.
+// A launch of `groups` groups takes ceil(groups / SMs) rounds; of several sweeps, which
+// run into one another, half a round more than fills the SMs, but no fewer than the sweeps.
+// A larger group has to gain 2 %.
 // One sweep of 200 lattices of L = 4 / 8 / 12: 0.247 / 0.613 / 1.97 ms one to a CTA,
-// 0.149 / 0.383 / 1.60 ms two to a CTA; six sweeps of 200 of L = 12 7.74 and 9.33 ms.
-constexpr int kGroupTime[6][7] = {
-    {0, 100, 108, 118, 130, 0, 155},   // L <= 6
-    {0, 100, 124, 145, 270, 0, 340},   // L = 8
-    {0, 100, 165, 214, 330, 0, 445},   // L = 10, 12
-    {0, 100, 156, 219, 322, 0, 440},   // L = 14, 16
-    {0, 100, 161, 252, 314, 0, 483},   // L = 18
-    {0, 100, 172, 254, 330, 0, 510},   // L >= 20
+// 0.149 / 0.383 / 1.60 ms two to a CTA; six sweeps of 200 of L = 12 7.74 and 9.33 ms; six
+// of 608 of L = 16 in windows of 6 54.0 ms three to a CTA, 60.7 ms two.
+struct GroupTime {
+    int max_L;
+    double link;        // ns a link of the sweep of one
+    int hb[5], rest[5];
+};
+constexpr int kGroups[5] = {1, 2, 3, 4, 6};
+constexpr GroupTime kGroupTime[] = {
+    {4, 98.0, {54, 59, 58, 60, 70}, {46, 43, 49, 48, 67}},
+    {6, 37.0, {58, 61, 66, 72, 86}, {42, 50, 52, 57, 69}},
+    {8, 18.3, {63, 72, 82, 97, 0}, {37, 47, 57, 163, 0}},
+    {10, 12.5, {62, 84, 109, 142, 0}, {38, 96, 122, 196, 0}},
+    {12, 12.2, {52, 74, 103, 131, 0}, {48, 88, 107, 178, 0}},
+    {16, 10.8, {52, 77, 110, 144, 0}, {48, 77, 109, 178, 0}},
+    {18, 11.0, {54, 80, 114, 151, 0}, {46, 81, 138, 163, 0}},
+    {kSlabMaxL, 9.7, {56, 82, 120, 154, 0}, {44, 89, 134, 175, 0}},
+    {64, 9.7, {56, 82, 120, 0, 0}, {44, 89, 134, 0, 0}},
 };
 
-// work: the batch's lattices, counted in lattices of its largest side.
-int choose_teams(const LaunchCfg &cfg, int n_lat, int work, int per_lat, int sms, int max_L)
+int choose_teams(const LaunchCfg &cfg, const KernelArgs &a, int per_lat, int sms)
 {
     if (cfg.threads != 256) {
         // asked for, but no more than the batch has for every SM (152 lattices of
         // L = 8 asked to run six to a CTA: 1.90 ms on 26 SMs, 0.65 ms on all)
         const int most = cfg.threads >= 512 ? 1 : cfg.threads >= 160 ? 4 : 6;
-        const int each = (n_lat + sms - 1) / sms;
+        const int each = (a.n_lat + sms - 1) / sms;
         return each >= most ? most : each == 5 ? 4 : each;
     }
-    const int *t = kGroupTime[max_L <= 6    ? 0
-                              : max_L <= 8  ? 1
-                              : max_L <= 12 ? 2
-                              : max_L <= 16 ? 3
-                              : max_L <= 18 ? 4
-                                            : 5];
+    const GroupTime *t = kGroupTime;
+    while (a.max_L > t->max_L) ++t;
+    const bool pass = a.program == kProgPass, approach = a.program == kProgApproach;
+    const bool muca = a.program == kProgMuca || (pass && a.pass_kind == 2);
+    const double heatbath = pass && (a.pass_kind == 1 || a.pass_kind == 3) ? 0.0 : 1.0;
+    const double rest = pass ? 1.0 - heatbath : (a.n_or + 0.5) / 4.5;
+    // the deciding warp's time, and that in the measured hb
+    const double usual = (2.75 + 320.0 / (a.max_L * a.max_L)) / t->link * 100.0;
+    const double decide =
+        (muca ? 22.0 : 2.75 + (approach ? 0.0 : 40.0 * a.inv_width / a.block)) / t->link * 100.0;
+    const double more = std::max(0.0, std::pow(decide, 3) - std::pow(usual, 3));
+    const int work = std::min(a.n_lat, a.work);
     int best = 1;
-    long long least = LLONG_MAX;
-    for (int g = 1; g <= (max_L > kSlabMaxL ? 3 : kMaxTeams); ++g) {
-        if (t[g] == 0) continue;
-        const long long items = (long long)((work + g - 1) / g) * per_lat;
-        const long long time = std::max<long long>(per_lat, (items + sms - 1) / sms) * t[g];
-        if (time < least) {
+    double least = INFINITY;
+    for (int k = 0; k < 5 && t->hb[k] > 0; ++k) {
+        const int groups = (work + kGroups[k] - 1) / kGroups[k];
+        const double rounds = groups <= sms  ? per_lat
+                              : per_lat == 1 ? (groups + sms - 1) / sms
+                                             : (double)groups * per_lat / sms + 0.5;
+        const double hb = k == 0 ? std::max((double)t->hb[0], decide)
+                                 : std::cbrt(std::pow((double)t->hb[k], 3) + more);
+        const double time = rounds * (heatbath * hb + rest * t->rest[k]);
+        if (time * 1.02 < least) {
             least = time;
-            best = g;
+            best = kGroups[k];
         }
     }
     return best;
@@ -2316,7 +2340,7 @@ cudaError_t launch_t(KernelArgs a, const LaunchCfg &cfg, cudaStream_t s, int *gr
     const int per_lat = multi ? (a.n_therm + a.n_meas) : 1;
     if ((long long)a.n_lat * per_lat <= 0) return cudaSuccess;
     const int sms = prepare_kernel<FAST>(cfg.carveout);
-    a.teams = choose_teams(cfg, a.n_lat, std::min(a.n_lat, a.work), per_lat, sms, a.max_L);
+    a.teams = choose_teams(cfg, a, per_lat, sms);
     // Two stages, where there are barriers for them (15 named ones, two per ring stage
     // of each team).  Four take L1 from the other passes: ten sweeps of 128 of L = 20
     // 63.2 ms, 60.9 with two, 59.7 with one; of L = 12 9.77, 9.66 and 9.85.

@@ -63,6 +63,7 @@ struct KernelArgs {
     double *e_hist;       // kProgMuca, nullable: e_hist[sweep * n_lat + lattice] = E
     int max_L;            // largest L of the handle's lattices
     int work;             // the handle's links in lattices of that side, rounded up
+    double inv_width;     // mean 1 / dE of the handle's windows
     int slab_L;           // largest L <= 24 of them (0: none): shared-memory slabs
     // set at launch: lattices a CTA works on at a time; whether it holds them in
     // shared memory as a whole; otherwise slabs in shared memory at a time; the
